@@ -234,22 +234,13 @@ DTYPE = {"fp64": "f64", "tf32": "tf32+f64", "bf16": "bf16+f64"}
 # for the sources of that stage's kernels as they were measured (a SHA-256 of
 # the code without comments, stage_sources_sha): after any change to them the
 # roofline's traffic is null until it is measured again.
-#   reduction: dram__bytes_read.sum + dram__bytes_write.sum of k_trd_panel,
-#   k_trd_s2k_pack and k_trd_s2k over four generations of the first 32
-#   searches of the 256-search batch, scaled to the full batch by the sum of
-#   n^3 over the decompositions a step does (367.2e9 / 17.35e9 = 21.2). The
-#   full batch keeps more matrices in flight than L2 holds, so this is a lower
-#   bound on its traffic.
-KERNEL_TRAFFIC = {
-    "reduction": {"bytes_per_step": 6.0181e9 * 21.16, "sources_sha256_16": "601f2a358980cfb8",
-                  "capture": "batch256-first32, 4 generations (24.07 GB), scaled by sum n^3"},
-}
+KERNEL_TRAFFIC = {}
 
-# The code each stage's kernels are built from: the part of the tridiagonal
-# route's source up to the end of the reduction (its kernels and every helper
-# they call) and the headers they include.
+# The code each stage's kernels are built from: the reduction's source up to
+# its host part (its kernel and every helper it calls) and the headers it
+# includes.
 STAGE_SOURCES = {
-    "reduction": {"prefix": ("kernels_eig_trd.cu", "// Scans of one CTA over n entries"),
+    "reduction": {"prefix": ("kernels_eig_trd_reduce.cu", "using RedFn ="),
                   "headers": ("device_common.cuh", "ozaki.cuh", "trd_common.cuh", "engine.h")},
 }
 

@@ -58,7 +58,8 @@ struct cmaes_s {
   int trd_bis_lanes = 8;  // lanes per eigenvalue of the multisection (1 for large batches)
   int4* d_trd_grp = nullptr;
   int trd_grp_blocks = 0;
-  std::vector<TrdChunk> trd_chunks;  // the cooperative launches of the reduction, panel by panel
+  std::vector<TrdChunk> trd_chunks;  // the cooperative launches of the reduction
+  TrdReducePlan trd_plan;
   // per-stage times of the tridiagonal route in profiling mode: one set of
   // kTrdStages + 1 events per profiled generation, drained with the phases
   std::vector<cudaEvent_t> trd_pool;
@@ -306,16 +307,15 @@ static int enqueue_jacobi32_big(cmaes_t h, int s0, int s1, cudaStream_t st) {
 static void enqueue_eig(cmaes_t h, int s0, int s1, cudaStream_t st) {
   TileMap sq = h->tiles(TK_SQUARE, s0, s1);
   if (h->max_n_trd > 0) {
-    // the cooperative reduction always covers every search of the handle (its
-    // group table is fixed at create); the searches outside [s0, s1) that
-    // are due are reduced too, which only repeats their decomposition
+    // the group table of the cooperative reduction is fixed at create and holds
+    // every search; the CTAs of searches outside [s0, s1) leave at once
     const TrdMaps tmaps{h->tiles(TK_TRD, s0, s1),   h->tiles(TK_TRDBIS, s0, s1), h->tiles(TK_TRDSQ, s0, s1),
                         h->tiles(TK_TRDBT, s0, s1), h->tiles(TK_TRDOZP, s0, s1), h->tiles(TK_TRDOZG, s0, s1),
                         h->tiles(TK_BTPACK, s0, s1), h->tiles(TK_BTGRAM, s0, s1), h->tiles(TK_BTTFAC, s0, s1),
                         h->tiles(TK_BTROWS, s0, s1), h->tiles(TK_BTCOLS, s0, s1), h->tiles(TK_BTUPD, s0, s1),
-                        h->tiles(TK_BTFIN, s0, s1),  h->tiles(TK_TRDS2KP, s0, s1), h->tiles(TK_TRDS2K, s0, s1)};
+                        h->tiles(TK_BTFIN, s0, s1)};
     const int nl = launch_eig_trd(h->dS, h->d_trd_grp, h->trd_chunks.data(), static_cast<int>(h->trd_chunks.size()),
-                                  h->d_trd_bar, h->count, s0, s1, tmaps, h->max_n_trd, h->trd_bis_lanes, st,
+                                  h->d_trd_bar, s0, s1, h->trd_plan, tmaps, h->max_n_trd, h->trd_bis_lanes, st,
                                   h->trd_marks);
     h->launches += nl;
     h->phase_launch[kPhaseEig] += nl;
@@ -782,77 +782,86 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
   CREATE_TRY(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
   for (int s = 0; s < count; ++s) h->hs[s].err = h->d_err;
   if (h->max_n_trd > 0) {
-    CREATE_TRY(cudaMalloc(&h->d_trd_bar, sizeof(unsigned) * count * kTrdBarStride));
-    CREATE_TRY(cudaMemsetAsync(h->d_trd_bar, 0, sizeof(unsigned) * count * kTrdBarStride, h->stream));
+    CREATE_TRY(cudaMalloc(&h->d_trd_bar, sizeof(unsigned) * count));
+    CREATE_TRY(cudaMemsetAsync(h->d_trd_bar, 0, sizeof(unsigned) * count, h->stream));
     for (int s = 0; s < count; ++s)
-      if (h->hs[s].trd) h->hs[s].trd_bar = h->d_trd_bar + static_cast<size_t>(s) * kTrdBarStride;
+      if (h->hs[s].trd) h->hs[s].trd_bar = h->d_trd_bar + s;
     // groups of the cooperative reduction, within what can be resident at once
     int dev = 0, sms = 0;
     CREATE_TRY(cudaGetDevice(&dev));
     CREATE_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    trd_set_attributes(h->max_n_trd);
-    // the largest group of a search: at least 16 columns per CTA, and enough
-    // work per step to outweigh the group barriers ((n - 64 q)^2 / 16384)
-    auto gcap = [](long long m) { return std::max(1, static_cast<int>(std::min(m / 16, m * m / 16384))); };
-    // the unblocked form (one barrier per step) when every search can have its
-    // largest group at once: the GPU is then partly idle and a step's latency
-    // sets the time; the panel form otherwise
-    long long caps = 0;
-    for (int s = 0; s < count; ++s)
-      if (h->hs[s].trd) caps += gcap(h->hs[s].n);
-    const long long budget_u = static_cast<long long>(trd_reduce_blocks_per_sm(h->max_n_trd, 0)) * sms;
-    const bool blocked = caps > budget_u;
-    const int per_sm = trd_reduce_blocks_per_sm(h->max_n_trd, blocked ? 1 : 0);
-    long long budget = static_cast<long long>(per_sm) * sms;
+    trd_set_attributes();
+    // CTAs per search: at least kTrdCols columns each. When every search can
+    // have that many with one CTA per SM the columns stay in shared memory if
+    // they fit; otherwise the resident CTAs are shared in proportion to the
+    // work n^3 (so that the searches end together), one CTA at least, first
+    // with one CTA per SM and the columns in shared memory, then with as many
+    // as fit and the columns in HBM.
+    constexpr int kTrdCols = 4;
+    std::vector<int> G(count, 0);
+    auto share = [&](long long budget) {
+      double wsum = 0.0;
+      long long nact = 0, caps = 0;
+      for (int s = 0; s < count; ++s) {
+        if (!h->hs[s].trd) continue;
+        const double n = h->hs[s].n;
+        wsum += n * n * n;
+        ++nact;
+        caps += std::min<long long>(h->hs[s].n / kTrdCols, sms);
+      }
+      for (int s = 0; s < count; ++s) {
+        if (!h->hs[s].trd) continue;
+        const double n = h->hs[s].n;
+        const long long cap = std::min<long long>(h->hs[s].n / kTrdCols, sms);
+        const long long spare = budget > nact ? budget - nact : 0;
+        G[s] = caps <= budget ? static_cast<int>(cap)
+                              : static_cast<int>(std::min(cap, 1 + static_cast<long long>(spare * (n * n * n / wsum))));
+      }
+    };
+    auto smem_of = [&](int in_smem) {
+      size_t b = 0;
+      for (int s = 0; s < count; ++s)
+        if (h->hs[s].trd) b = std::max(b, trd_reduce_smem(h->hs[s].n, G[s], in_smem));
+      return b;
+    };
+    long long budget = sms;
+    share(budget);
+    long long ctas = 0;
+    for (int s = 0; s < count; ++s) ctas += G[s];
+    h->trd_plan.smem = smem_of(1);
+    h->trd_plan.in_smem = ctas <= sms && trd_reduce_blocks_per_sm(h->trd_plan.smem, 1, 512) >= 1;
+    if (!h->trd_plan.in_smem) {
+      h->trd_plan.smem = smem_of(0);
+      if (ctas > sms || trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 512) < 1) h->trd_plan.threads = 256;
+    }
+    if (h->trd_plan.threads == 256) {
+      // (the accumulators' size depends on the shares)
+      int per_sm = trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 256);
+      for (int pass = 0; pass < 2; ++pass) {
+        budget = static_cast<long long>(per_sm) * sms;
+        share(budget);
+        h->trd_plan.smem = smem_of(0);
+        per_sm = std::min(per_sm, trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 256));
+      }
+      budget = static_cast<long long>(per_sm) * sms;
+    }
     if (budget < 1) {
       set_error(h, CMAES_EUNSUPPORTED, "the tridiagonal reduction cannot be resident on this device");
       return fail(CMAES_EUNSUPPORTED);
     }
-    // the panel form: one group table per panel of kTrdPanel columns: the searches with
-    // columns left in panel q share the resident CTAs in proportion to their
-    // trailing work (n - kTrdPanel q)^2, each with at least one CTA and at most
-    // (n - kTrdPanel q) / 16 and (n - kTrdPanel q)^2 / 16384 (enough work per
-    // step to outweigh the group barriers); launches of at most `budget` CTAs
-    // never split a group
-    std::vector<int4> grp;
+    std::vector<int4> grp;  // launches of at most `budget` CTAs never split a group
     h->trd_chunks.clear();
-    if (!blocked) {
-      for (int s = 0; s < count; ++s) {
-        if (!h->hs[s].trd) continue;
-        const int G = gcap(h->hs[s].n);
-        for (int r = 0; r < G; ++r) grp.push_back(make_int4(s, r, G, 0));
+    int chunk_start = 0;
+    for (int s = 0; s < count; ++s) {
+      if (!h->hs[s].trd) continue;
+      const int Gs = static_cast<int>(std::min<long long>(G[s], budget));
+      if (static_cast<long long>(grp.size()) + Gs - chunk_start > budget) {
+        h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start});
+        chunk_start = static_cast<int>(grp.size());
       }
-      h->trd_chunks.push_back(TrdChunk{0, static_cast<int>(grp.size()), -1});
+      for (int r = 0; r < Gs; ++r) grp.push_back(make_int4(s, r, Gs, 0));
     }
-    const int panels = blocked ? ceil_div(h->max_n_trd, kTrdPanel) : 0;
-    for (int q = 0; q < panels; ++q) {
-      double wsum = 0.0;
-      int nact = 0;
-      for (int s = 0; s < count; ++s) {
-        const Search& x = h->hs[s];
-        if (!x.trd || x.n <= kTrdPanel * q) continue;
-        const double m = static_cast<double>(x.n - kTrdPanel * q);
-        wsum += m * m;
-        ++nact;
-      }
-      if (nact == 0) continue;
-      const long long spare = budget > nact ? budget - nact : 0;
-      int chunk_start = static_cast<int>(grp.size());
-      for (int s = 0; s < count; ++s) {
-        const Search& x = h->hs[s];
-        if (!x.trd || x.n <= kTrdPanel * q) continue;
-        const long long m = x.n - kTrdPanel * q;
-        const double share = static_cast<double>(m * m) / wsum;
-        int G = static_cast<int>(std::floor(share * static_cast<double>(spare))) + 1;
-        G = std::min(G, gcap(m));
-        if (static_cast<long long>(grp.size()) + G - chunk_start > budget) {
-          h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start, q});
-          chunk_start = static_cast<int>(grp.size());
-        }
-        for (int r = 0; r < G; ++r) grp.push_back(make_int4(s, r, G, 0));
-      }
-      h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start, q});
-    }
+    h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start});
     h->trd_grp_blocks = static_cast<int>(grp.size());
     // eigenvalues to find per decomposition of the whole batch: with more than
     // the GPU holds as 8-lane groups, plain bisection does the least work
@@ -907,8 +916,6 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
         case TK_BTCOLS: t = x.trd ? tiles_bt_cols(x.n) : 0; break;
         case TK_BTUPD: t = x.trd ? tiles_bt_update(x.n) : 0; break;
         case TK_BTFIN: t = x.trd ? tiles_bt_final(x.n) : 0; break;
-        case TK_TRDS2KP: t = x.trd ? tiles_trd_s2k_pack(x.n) : 0; break;
-        case TK_TRDS2K: t = x.trd ? tiles_trd_s2k(x.n) : 0; break;
         case TK_JBBLK: t = x.trd ? 0 : tiles_jb_blocks(x.n); break;
         case TK_JBLOAD: t = x.trd ? 0 : tiles_jb_load(x.n); break;
         case TK_JBROWS: t = x.trd ? 0 : tiles_jb_rows(x.n); break;

@@ -94,7 +94,7 @@ struct Search {
   int trd, trd_pad_;  // 1: this search's eigendecomposition takes the tridiagonal route
   double* trd_v;      // 11 x ldn doubles: d, e, split e, e^2, tau, eigenvalues (two orders), p and p.v buffers, scalars
   int* trd_i;         // 5 x ldn ints: block start / end, rank, cluster start, V^T V tile flags
-  unsigned* trd_bar;  // the reduction's counters: group barrier, work per panel step (kTrdBarStride)
+  unsigned* trd_bar;  // the reduction's group barrier
   unsigned char* ozp; // packed digit planes of the FP64-accurate tensor-core products (trd_oz_bytes)
   int* oze;           // their row exponents (trd_oz_exps ints)
 };
@@ -125,7 +125,7 @@ int tiles_square(int n);                    // all 64 x 64 tiles of n x n
 
 enum TileKind {
   TK_SAMPLE_Z = 0, TK_PANEL, TK_COLRED, TK_RANK, TK_ROWS, TK_RECOMB, TK_GEMV, TK_SYM, TK_SQUARE,
-  TK_COVP, TK_RANK2D, TK_TCSAMPLE, TK_TCOBJ, TK_TCCOVP, TK_TCSYM, TK_FLAT, TK_FLATSYM, TK_REEVAL, TK_JBBLK, TK_JBLOAD, TK_JBROWS, TK_TRD, TK_TRDBIS, TK_TRDSQ, TK_TRDBT, TK_TRDOZP, TK_TRDOZG, TK_BTPACK, TK_BTGRAM, TK_BTTFAC, TK_BTROWS, TK_BTCOLS, TK_BTUPD, TK_BTFIN, TK_TRDS2KP, TK_TRDS2K, TK_COUNT
+  TK_COVP, TK_RANK2D, TK_TCSAMPLE, TK_TCOBJ, TK_TCCOVP, TK_TCSYM, TK_FLAT, TK_FLATSYM, TK_REEVAL, TK_JBBLK, TK_JBLOAD, TK_JBROWS, TK_TRD, TK_TRDBIS, TK_TRDSQ, TK_TRDBT, TK_TRDOZP, TK_TRDOZG, TK_BTPACK, TK_BTGRAM, TK_BTTFAC, TK_BTROWS, TK_BTCOLS, TK_BTUPD, TK_BTFIN, TK_COUNT
 };
 
 // launchers (kernels_gen.cu)
@@ -242,30 +242,29 @@ int tiles_bt_cols(int n);    // 64-column tiles of a 128 x n product
 int tiles_bt_update(int n);  // 128 x 64 tiles of the largest panel's update
 int tiles_bt_final(int n);   // 8 columns per tile
 void bt_set_attributes();
-size_t trd_reduce_smem(int max_n, int blocked);
-int trd_reduce_blocks_per_sm(int max_n, int blocked);
-int tiles_trd_s2k_pack(int n);  // 64-row blocks of the reduction's trailing-update operands
-int tiles_trd_s2k(int n);       // 128 x 64 tiles of its trailing update
-void trd_set_attributes(int max_n);
+void trd_set_attributes();
 constexpr int kTrdStages = 6;  // reduction, eigenvalues, inverse iteration, clusters, orthogonalisation, back-transformation
-constexpr int kTrdPanel = 64;  // columns per panel of the tridiagonal reduction
-// counters per search of the reduction (Search::trd_bar): the group barrier,
-// then one work counter per step of a panel
-constexpr int kTrdBarStride = 1 + kTrdPanel;
-// One cooperative launch of the reduction: CTAs [first, first + count) of the
-// group table, all working on panel `panel` (-1: the unblocked form, the
-// whole reduction in one launch).
+// The reduction (kernels_eig_trd_reduce.cu): one cooperative launch per chunk,
+// CTAs [first, first + count) of the group table; the columns in shared memory
+// or in EA, and the dynamic shared memory of a CTA.
 struct TrdChunk {
-  int first, count, panel;
+  int first, count;
 };
+struct TrdReducePlan {
+  int in_smem = 0, threads = 512;
+  size_t smem = 0;
+};
+size_t trd_reduce_smem(int n, int G, int in_smem);
+int trd_reduce_blocks_per_sm(size_t smem, int in_smem, int threads);
+int launch_trd_reduce(Search* S, const int4* grp, const TrdChunk* chunks, int nchunks, unsigned* bars, int s0, int s1,
+                      const TrdReducePlan& plan, cudaStream_t st);
 struct TrdMaps {
   TileMap tt, tbis, tsq, tbt, ozp, ozg;  // TK_TRD, TK_TRDBIS, TK_TRDSQ, TK_TRDBT, TK_TRDOZP, TK_TRDOZG
   TileMap btpack, btgram, bttfac, btrows, btcols, btupd, btfin;  // TK_BTPACK .. TK_BTFIN
-  TileMap s2kp, s2k;  // TK_TRDS2KP, TK_TRDS2K
 };
 int launch_bt(Search* S, const TrdMaps& m, int max_n, cudaStream_t st);
-int launch_eig_trd(Search* S, const int4* grp, const TrdChunk* chunks, int nchunks, unsigned* bars,
-                   int bar_count, int s0, int s1, const TrdMaps& tm, int max_n, int bis_lanes, cudaStream_t st,
+int launch_eig_trd(Search* S, const int4* grp, const TrdChunk* chunks, int nchunks, unsigned* bars, int s0, int s1,
+                   const TrdReducePlan& plan, const TrdMaps& tm, int max_n, int bis_lanes, cudaStream_t st,
                    cudaEvent_t* marks);
 
 }  // namespace cmaes_gb300

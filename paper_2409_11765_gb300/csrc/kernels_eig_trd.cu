@@ -4,15 +4,8 @@
 // The paper computes B and D with LAPACK's dsyev (§3.1), i.e. Householder
 // reduction to tridiagonal form followed by a tridiagonal eigensolver. On
 // GB300 FP64 issues at 1/64 of the FP32 rate, so the route is built for few
-// FP64 flops and few sequential steps, all in FP64 (no refinement needed):
-//   1. Householder tridiagonalisation T = Q^T C Q (unblocked, lower part;
-//      Golub & Van Loan §8.3.1), by a group of CTAs per search in one
-//      cooperative launch: per step every CTA of the group forms the reflector
-//      of column k itself (the same fixed-order arithmetic everywhere), then
-//      each CTA applies the pending rank-2 update A <- A - v w^T - w v^T of the
-//      previous step to the columns it owns while it accumulates the symmetric
-//      product p = tau A v for the new v: one pass over the trailing matrix and
-//      one group barrier per step.
+// FP64 flops and few sequential steps, all to FP64 accuracy (no refinement needed):
+//   1. Householder tridiagonalisation T = Q^T C Q (kernels_eig_trd_reduce.cu).
 //   2. Splitting: off-diagonal entries below 4 sqrt(n) eps64 ||T|| are set to
 //      zero, which cuts T into independent blocks (this is where the repeated
 //      eigenvalues of a low-rank update of a multiple of I separate).
@@ -49,597 +42,6 @@
 #include "trd_common.cuh"
 
 namespace cmaes_gb300 {
-
-__device__ __forceinline__ double warp_sum_xor(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// Barrier of the G CTAs of one search. The launch is cooperative, so every
-// CTA of the group is resident; the wait is still bounded: after ~1 s the
-// device status word records a time-out and the CTA leaves the reduction.
-__device__ bool trd_group_sync(unsigned* ctr, unsigned target, int* err, int* sh_ok) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(ctr, 1u);
-    const long long t0 = clock64();
-    int ok = 1;
-    while (ld_acquire_u32(ctr) < target) {
-      if (clock64() - t0 > kTrdWaitCycles) {
-        atomicOr(err, kDevErrTimeout);
-        ok = 0;
-        break;
-      }
-    }
-    __threadfence();
-    *sh_ok = ok;
-  }
-  __syncthreads();
-  return *sh_ok != 0;
-}
-
-// --------------------------------------------------------------------------
-// 1. Householder tridiagonalisation in panels of kPnb columns (the blocked
-// form of LAPACK's dsytrd / dlatrd). Within panel [k0, k1) the matrix A (EA)
-// is only read: the current matrix is A - V W^T - W V^T with V the panel's
-// reflectors so far (columns k0.. of EX) and W (columns 0.. of EG) built step
-// by step; after the panel the trailing part of A takes that rank-2 kPnb
-// update as FP64-accurate products on the tensor cores (k_trd_s2k_*).
-// CTA blockIdx.x works for search grp[b].x as member r = grp[b].y of a group
-// of G = grp[b].z CTAs: it owns the 32-row chunks c with c mod G = r (the
-// column products are dealt at run time). Step k (panel column j = k - k0) in
-// two phases:
-//   A. with u_W = W^T v, u_V = V^T v (the previous step's v, from the previous
-//      phase B) and q = A v on the own rows, the previous step's
-//      p = tau (q - V u_W - W u_V) and w = p - (tau / 2)(p . v) v, where
-//      p . v = tau (q . v - 2 u_W . u_V); then, in the same pass over the own
-//      rows, column k of the current matrix, c = A(:, k) - V W(k, :)^T -
-//      W V(k, :)^T (to cbuf), and the partial sum of |c(k+2:)|^2;
-//                                                               group barrier
-//   B. (every CTA) the reflector of c and its vector v; then the products
-//      q(j') = A(:, j')^T v (to qbuf, and q(j') v(j') to qv) and
-//      u = [W V]^T v over rows k+1.., column pairs dealt to the group's warps
-//      from a per-step counter; q . v is summed in phase A of the next step
-//      over all rows by all warps, in a fixed order;
-//                                                               group barrier
-// The group (its size may differ from panel to panel) counts its barriers
-// from the start of the panel: barrier m waits for G m arrivals; in panel 0
-// the one after the symmetrisation is m = 1 and step k's are 2k + 2 and
-// 2k + 3, in the others step k's are 2(k - k0) + 1 and 2(k - k0) + 2.
-// Dynamic shared memory: v (n doubles).
-// --------------------------------------------------------------------------
-constexpr int kUbuf = 2 * kPnb;  // u_W then u_V at the start of Search::EH, then the partial sums
-
-__global__ void __launch_bounds__(kTrdNT, 4) k_trd_panel(Search* S, const int4* grp, int q) {
-  extern __shared__ double vsm[];
-  __shared__ double sVk[kPnb], sWk[kPnb], su[2 * kPnb];
-  __shared__ double red[kTrdNT / 32 + 8];
-  __shared__ int sh_ok;
-  const int4 g = grp[blockIdx.x];
-  Search& s = S[g.x];
-  if (!trd_due(s)) return;
-  const int n = s.n, k0 = kPnb * q;
-  if (k0 >= n) return;
-  const int k1 = min(k0 + kPnb, n);
-  const long long L = s.ldn;
-  const int r = g.y, G = g.z;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = kTrdNT / 32;
-  double* A = s.EA;
-  double* Hv = s.EX;
-  double* Wp = s.EG;
-  double* d = tv(s, TV_D);
-  double* e = tv(s, TV_E);
-  double* tau = tv(s, TV_TAU);
-  double* cbuf = tv(s, TV_P0);
-  double* qbuf = tv(s, TV_P1);
-  double* qv = tv(s, TV_SD);          // q(j) v(j) per column
-  double* ubuf = s.EH;                // u_W (kPnb), u_V (kPnb)
-  double* part = s.EH + kUbuf;        // per-CTA partial |c|^2, kPartStride apart
-  unsigned* bar = s.trd_bar;
-  auto barrier = [&](unsigned m) -> bool {
-    if (G > 1) return trd_group_sync(bar, static_cast<unsigned>(G) * m, s.err, &sh_ok);
-    __syncthreads();
-    return true;
-  };
-  if (q == 0) {  // A = (C + C^T) / 2, owned columns
-    const double* C = s.C;
-    for (int jc = r; jc < n; jc += G)
-      for (int i = tid; i < n; i += kTrdNT) A[i + L * jc] = 0.5 * (C[i + L * jc] + C[jc + L * i]);
-    if (!barrier(1u)) return;
-  }
-  // the first own 32-row chunk at or after row `row`
-  auto first_chunk = [&](int row) {
-    const int c0 = row >> 5;
-    return c0 + ((r - c0 % G) % G + G) % G;
-  };
-  const unsigned mbase = q == 0 ? 1u : 0u;
-  double tprev = 0.0;
-  // Phase A of step k (j = k - k0); with last, only the previous step's w on
-  // the own rows i >= k (the end of the panel). Returns the partial |c|^2.
-  auto phase_a = [&](int k, int j, bool last) -> double {
-    const int jp = j - 1;  // columns of W and V before the previous step
-    if (j > 0) {
-      for (int l = tid; l < jp; l += kTrdNT) {
-        su[l] = __ldcg(&ubuf[l]);
-        su[kPnb + l] = __ldcg(&ubuf[kPnb + l]);
-        sVk[l] = __ldcg(&Hv[k + L * (k0 + l)]);
-        sWk[l] = __ldcg(&Wp[k + L * l]);
-      }
-      {  // q . v: warp w sums rows k + 32 w + lane + 256 m (two chains), in fixed order
-        double s0 = 0.0, s1 = 0.0;
-        int c = k + 32 * warp + lane;
-        for (; c + kTrdNT < n; c += 2 * kTrdNT) {
-          s0 += __ldcg(&qv[c]);
-          s1 += __ldcg(&qv[c + kTrdNT]);
-        }
-        if (c < n) s0 += __ldcg(&qv[c]);
-        const double sw = warp_sum_xor(s0 + s1);
-        if (lane == 0) red[warp] = sw;
-      }
-      __syncthreads();
-      if (warp == 0) {  // u_W . u_V and the row-k correction, lanes in fixed order
-        double uu = 0.0, ck = 0.0;
-        for (int l = lane; l < jp; l += 32) {
-          uu = fma(su[l], su[kPnb + l], uu);
-          ck = fma(sVk[l], su[l], fma(sWk[l], su[kPnb + l], ck));
-        }
-        uu = warp_sum_xor(uu);
-        ck = warp_sum_xor(ck);
-        if (lane == 0) {
-          double sq = 0.0;
-          for (int w = 0; w < NW; ++w) sq += red[w];
-          const double half = 0.5 * tprev * tprev * (sq - 2.0 * uu);  // (tau / 2) p . v
-          const double pk = tprev * (__ldcg(&qbuf[k]) - ck);
-          sVk[jp] = 1.0;                // v_{k-1}(k)
-          sWk[jp] = fma(-half, 1.0, pk);  // w_{k-1}(k)
-          red[NW] = half;
-        }
-      }
-      __syncthreads();
-    }
-    const double half = j > 0 ? red[NW] : 0.0;
-    double nrm = 0.0;
-    for (int c = first_chunk(k) + G * warp; 32 * c < n; c += G * NW) {
-      const int i = 32 * c + lane;
-      if (i < k || i >= n) continue;
-      // V u_W + W u_V (previous step), then the column correction: two
-      // chains each (even and odd columns of every group of eight), summed last
-      double pc0 = 0.0, pc1 = 0.0, cc0 = 0.0, cc1 = 0.0;
-      int l = 0;
-      for (; l + 8 <= jp; l += 8) {  // eight columns' loads in flight
-        double hv[8], wv[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          hv[u] = __ldcg(&Hv[i + L * (k0 + l + u)]);
-          wv[u] = __ldcg(&Wp[i + L * (l + u)]);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; u += 2) {
-          pc0 = fma(hv[u], su[l + u], fma(wv[u], su[kPnb + l + u], pc0));
-          cc0 = fma(hv[u], sWk[l + u], fma(wv[u], sVk[l + u], cc0));
-          pc1 = fma(hv[u + 1], su[l + u + 1], fma(wv[u + 1], su[kPnb + l + u + 1], pc1));
-          cc1 = fma(hv[u + 1], sWk[l + u + 1], fma(wv[u + 1], sVk[l + u + 1], cc1));
-        }
-      }
-      for (; l < jp; ++l) {
-        const double hv = __ldcg(&Hv[i + L * (k0 + l)]), wv = __ldcg(&Wp[i + L * l]);
-        pc0 = fma(hv, su[l], fma(wv, su[kPnb + l], pc0));
-        cc0 = fma(hv, sWk[l], fma(wv, sVk[l], cc0));
-      }
-      const double pc = pc0 + pc1;
-      double cc = cc0 + cc1;
-      if (j > 0) {
-        const double vi = vsm[i];  // v_{k-1}(i)
-        const double wi = fma(-half, vi, tprev * (__ldcg(&qbuf[i]) - pc));
-        Wp[i + L * jp] = wi;
-        cc = fma(vi, sWk[jp], fma(wi, sVk[jp], cc));
-      }
-      if (!last && i > k) {
-        const double ci = __ldcg(&A[i + L * k]) - cc;
-        vsm[i] = ci;
-        cbuf[i] = ci;
-        if (i >= k + 2) nrm = fma(ci, ci, nrm);
-      }
-    }
-    return nrm;
-  };
-  for (int k = k0; k < k1; ++k) {
-    const int j = k - k0;
-    // ---------------- A ----------------
-    double nrm = phase_a(k, j, false);
-    if (k == n - 1) {  // the last diagonal entry
-      if (r == 0 && tid == 0) {
-        double acc = __ldcg(&A[k + L * k]);
-        for (int l = 0; l < j; ++l) acc = fma(-2.0 * sVk[l], sWk[l], acc);
-        d[k] = acc;
-      }
-      return;
-    }
-    nrm = warp_sum_xor(nrm);
-    if (lane == 0) red[warp] = nrm;
-    __syncthreads();
-    if (tid == 0) {
-      double a = 0.0;
-      for (int w = 0; w < NW; ++w) a += red[w];
-      part[static_cast<long long>(r) * kPartStride] = a;
-    }
-    if (!barrier(mbase + 2u * j + 1u)) return;
-    // ---------------- B ----------------
-    if (warp == 0) {
-      double a = 0.0;
-      for (int c = lane; c < G; c += 32) a += __ldcg(&part[static_cast<long long>(c) * kPartStride]);
-      a = warp_sum_xor(a);
-      if (lane == 0) red[NW + 1] = a;
-    }
-    if (warp == 1) {  // the diagonal entry of column k: A(k, k) - 2 V(k, :) W(k, :)^T
-      double acc = 0.0;
-      for (int l = lane; l < j; l += 32) acc = fma(sVk[l], sWk[l], acc);
-      acc = warp_sum_xor(acc);
-      if (lane == 0) red[NW + 2] = fma(-2.0, acc, __ldcg(&A[k + L * k]));
-    }
-    if (tid == 64) red[NW + 5] = __ldcg(&cbuf[k + 1]);  // alpha
-    __syncthreads();
-    if (tid == 0) {
-      const double xn2 = red[NW + 1];
-      const double alpha = red[NW + 5];
-      double t = 0.0, beta = alpha, scale = 0.0;
-      if (xn2 > 0.0) {
-        beta = -copysign(sqrt(fma(alpha, alpha, xn2)), alpha);
-        t = (beta - alpha) / beta;
-        scale = 1.0 / (alpha - beta);
-      }
-      red[NW] = t;
-      red[NW + 3] = scale;
-      if (r == 0) {
-        d[k] = red[NW + 2];
-        e[k] = beta;
-        tau[k] = t;
-      }
-    }
-    __syncthreads();
-    const double t = red[NW], scale = red[NW + 3];
-    for (int i = k + 1 + tid; i < n; i += kTrdNT) vsm[i] = (i == k + 1) ? 1.0 : __ldcg(&cbuf[i]) * scale;
-    __syncthreads();
-    for (int c = first_chunk(k + 1) + G * warp; 32 * c < n; c += G * NW) {
-      const int i = 32 * c + lane;
-      if (i > k && i < n) Hv[i + L * k] = vsm[i];
-    }
-    // columns j' >= k + 1 of A two at a time, then the 2j columns of [W V]
-    // two at a time (u = [W V]^T v over rows k+1..), dealt at run time to the
-    // group's warps from the step's work counter (the next pair is claimed
-    // before the current one is worked)
-    {
-      unsigned* wctr = bar + 1 + j;
-      const int units_a = (n - k) >> 1;  // pairs (k+1, k+2), (k+3, k+4), ...; the last may be single
-      const int units = units_a + j;
-      int u = 0;
-      if (lane == 0) u = static_cast<int>(atomicAdd(wctr, 1u));
-      u = __shfl_sync(0xffffffffu, u, 0);
-      while (u < units) {
-        int un = 0;
-        if (lane == 0) un = static_cast<int>(atomicAdd(wctr, 1u));
-        const bool is_a = u < units_a;
-        int j1, j2;            // A: columns j1, j2; [W V]: entries j1, j2 of the 2j
-        const double *A1, *A2;
-        bool two = true;
-        if (is_a) {
-          j1 = k + 1 + 2 * u;
-          j2 = j1 + 1;
-          two = j2 < n;
-          A1 = A + L * j1;
-          A2 = A + L * (two ? j2 : j1);
-        } else {
-          j1 = 2 * (u - units_a);
-          j2 = j1 + 1;
-          A1 = j1 < j ? Wp + L * j1 : Hv + L * (k0 + j1 - j);
-          A2 = j2 < j ? Wp + L * j2 : Hv + L * (k0 + j2 - j);
-        }
-        double q1 = 0.0, q2 = 0.0;
-        int i = k + 1 + lane;
-        constexpr int U = 8;  // rows per lane in flight, two columns
-        for (; i + 32 * (U - 1) < n; i += 32 * U) {
-          double a1[U], a2[U];
-#pragma unroll
-          for (int uu = 0; uu < U; ++uu) {
-            a1[uu] = __ldcg(&A1[i + 32 * uu]);
-            a2[uu] = two ? __ldcg(&A2[i + 32 * uu]) : 0.0;
-          }
-#pragma unroll
-          for (int uu = 0; uu < U; ++uu) {
-            const double vi = vsm[i + 32 * uu];
-            q1 = fma(a1[uu], vi, q1);
-            q2 = fma(a2[uu], vi, q2);
-          }
-        }
-        for (; i < n; i += 32) {
-          const double vi = vsm[i];
-          q1 = fma(__ldcg(&A1[i]), vi, q1);
-          if (two) q2 = fma(__ldcg(&A2[i]), vi, q2);
-        }
-        // both sums in one tree: the first level leaves column 1's pairs on
-        // lanes 0-15 and column 2's on lanes 16-31 (five FP64 adds, not ten)
-        const bool hi = (lane & 16) != 0;
-        double qs = (hi ? q2 : q1) + __shfl_xor_sync(0xffffffffu, hi ? q1 : q2, 16);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) qs += __shfl_xor_sync(0xffffffffu, qs, o);
-        const int jw = lane == 0 ? j1 : j2;
-        if ((lane == 0 || (lane == 16 && two)) && is_a) {
-          qbuf[jw] = qs;
-          qv[jw] = qs * vsm[jw];
-        } else if ((lane == 0 || lane == 16) && !is_a) {
-          ubuf[jw < j ? jw : kPnb + jw - j] = qs;
-        }
-        u = __shfl_sync(0xffffffffu, un, 0);
-      }
-    }
-    if (!barrier(mbase + 2u * j + 2u)) return;
-    tprev = t;
-  }
-  // the panel's last w (its last step was a full one: k1 < n)
-  phase_a(k1, k1 - k0, true);
-}
-
-// --------------------------------------------------------------------------
-// 1'. The unblocked reduction, for handles whose searches leave the GPU
-// partly idle (each group at its largest size): then a step's latency, not
-// the FP64 work, sets the time, and this form has one group barrier per step
-// (against two in the panel form). Golub & Van Loan §8.3.1: per step every
-// CTA forms the reflector of column k itself (the same fixed-order
-// arithmetic everywhere), then applies the pending rank-2 update
-// A <- A - v w^T - w v^T of the previous step to the columns it owns while it
-// accumulates p = tau A v for the new v: one pass over the trailing matrix.
-// CTA blockIdx.x works for search grp[b].x as member grp[b].y of a group of
-// grp[b].z CTAs; column j belongs to member j mod G, and within it to warp
-// (j div G) mod 8. Dynamic shared memory: v and w of the previous step and v
-// of the current one (3 n doubles).
-// --------------------------------------------------------------------------
-__global__ void __launch_bounds__(kTrdNT) k_trd_sytrd(Search* S, const int4* grp) {
-  extern __shared__ double tsm[];
-  __shared__ double red[kTrdNT / 32 + 8];
-  __shared__ int sh_ok;
-  const int4 g = grp[blockIdx.x];
-  Search& s = S[g.x];
-  if (!trd_due(s)) return;
-  const int n = s.n;
-  const long long L = s.ldn;
-  const int r = g.y, G = g.z;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = kTrdNT / 32;
-  double* W = s.EA;
-  double* Hv = s.EX;
-  const double* C = s.C;
-  double* d = tv(s, TV_D);
-  double* e = tv(s, TV_E);
-  double* tau = tv(s, TV_TAU);
-  double* pbuf = tv(s, TV_P0);  // two buffers: step k uses pbuf + (k & 1) L
-  double* sdot = tv(s, TV_SD);  // per-CTA partial p.v, two buffers of L / 2
-  unsigned* bar = s.trd_bar;
-  double* vprev = tsm;
-  double* wprev = tsm + n;
-  double* vcur = tsm + 2 * n;
-  // W = (C + C^T) / 2, owned columns only
-  for (int j = r; j < n; j += G)
-    for (int i = tid; i < n; i += kTrdNT) W[i + L * j] = 0.5 * (C[i + L * j] + C[j + L * i]);
-  for (int i = tid; i < n; i += kTrdNT) {
-    vprev[i] = 0.0;
-    wprev[i] = 0.0;
-  }
-  unsigned nb = 0;
-  if (G > 1) {
-    if (!trd_group_sync(bar, G * ++nb, s.err, &sh_ok)) return;
-  } else {
-    __syncthreads();
-  }
-  for (int k = 0; k + 1 < n; ++k) {
-    // column k with the pending update of step k - 1
-    for (int i = k + tid; i < n; i += kTrdNT)
-      vcur[i] = fma(-wprev[i], vprev[k], fma(-vprev[i], wprev[k], __ldcg(&W[i + L * k])));
-    __syncthreads();
-    // its reflector (warp 0, fixed-order sum)
-    if (warp == 0) {
-      double part = 0.0;
-      for (int i = k + 2 + lane; i < n; i += 32) part = fma(vcur[i], vcur[i], part);
-      const double xn2 = warp_sum_xor(part);
-      if (lane == 0) {
-        const double alpha = vcur[k + 1];
-        double t = 0.0, beta = alpha, scale = 0.0;
-        if (xn2 > 0.0) {
-          beta = -copysign(sqrt(fma(alpha, alpha, xn2)), alpha);
-          t = (beta - alpha) / beta;
-          scale = 1.0 / (alpha - beta);
-        }
-        red[NW] = t;
-        red[NW + 1] = beta;
-        red[NW + 2] = scale;
-        red[NW + 3] = vcur[k];
-      }
-    }
-    __syncthreads();
-    const double t = red[NW], scale = red[NW + 2];
-    for (int i = k + 2 + tid; i < n; i += kTrdNT) vcur[i] *= scale;
-    if (tid == 0) vcur[k + 1] = 1.0;
-    __syncthreads();
-    if (r == 0) {
-      for (int i = k + 1 + tid; i < n; i += kTrdNT) Hv[i + L * k] = vcur[i];
-      if (tid == 0) {
-        d[k] = red[NW + 3];
-        e[k] = red[NW + 1];
-        tau[k] = t;
-      }
-    }
-    // owned columns j >= k + 1, two per warp at a time: pending update, then
-    // p_j = tau (A v)_j, and this CTA's share of p . v
-    double* pk = pbuf + (k & 1) * L;
-    const int m0 = (k + 1 > r) ? (k + 1 - r + G - 1) / G : 0;
-    double pv = 0.0;
-    for (int m = m0 + warp;; m += 2 * NW) {
-      const int j1 = r + G * m, j2 = r + G * (m + NW);
-      if (j1 >= n) break;
-      const bool two = j2 < n;
-      const int j2c = two ? j2 : j1;
-      const double vp1 = vprev[j1], wp1 = wprev[j1], vp2 = vprev[j2c], wp2 = wprev[j2c];
-      double q1 = 0.0, q2 = 0.0;
-      double* W1 = W + L * j1;
-      double* W2 = W + L * j2c;
-      int i = k + 1 + lane;
-      // four rows per lane in flight: the column loads are issued before use
-      for (; i + 96 < n; i += 128) {
-        double a1[4], a2[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          a1[u] = W1[i + 32 * u];
-          a2[u] = two ? W2[i + 32 * u] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int ii = i + 32 * u;
-          const double vi = vprev[ii], wi = wprev[ii], ci = vcur[ii];
-          a1[u] = fma(-wi, vp1, fma(-vi, wp1, a1[u]));
-          q1 = fma(a1[u], ci, q1);
-          if (two) {
-            a2[u] = fma(-wi, vp2, fma(-vi, wp2, a2[u]));
-            q2 = fma(a2[u], ci, q2);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          W1[i + 32 * u] = a1[u];
-          if (two) W2[i + 32 * u] = a2[u];
-        }
-      }
-      for (; i < n; i += 32) {
-        const double vi = vprev[i], wi = wprev[i], ci = vcur[i];
-        const double a1 = fma(-wi, vp1, fma(-vi, wp1, W1[i]));
-        W1[i] = a1;
-        q1 = fma(a1, ci, q1);
-        if (two) {
-          const double a2 = fma(-wi, vp2, fma(-vi, wp2, W2[i]));
-          W2[i] = a2;
-          q2 = fma(a2, ci, q2);
-        }
-        if (k == n - 2) d[n - 1] = a1;  // the last diagonal entry (i = j = n - 1)
-      }
-      q1 = t * warp_sum_xor(q1);
-      q2 = t * warp_sum_xor(q2);
-      if (lane == 0) {
-        pk[j1] = q1;
-        pv = fma(q1, vcur[j1], pv);
-        if (two) {
-          pk[j2] = q2;
-          pv = fma(q2, vcur[j2], pv);
-        }
-      }
-    }
-    if (lane == 0) red[warp] = pv;
-    __syncthreads();
-    double* sdk = sdot + (k & 1) * (L / 2);
-    if (tid == 0) {
-      double sp = 0.0;
-      for (int w = 0; w < NW; ++w) sp += red[w];
-      sdk[r] = sp;
-    }
-    if (G > 1) {
-      if (!trd_group_sync(bar, G * ++nb, s.err, &sh_ok)) return;
-    } else {
-      __syncthreads();
-    }
-    // w = p - (tau / 2) (p . v) v, kept with v for the next step's update
-    if (warp == 0) {
-      double sp = 0.0;
-      for (int c = lane; c < G; c += 32) sp += __ldcg(&sdk[c]);
-      sp = warp_sum_xor(sp);
-      if (lane == 0) red[NW + 4] = 0.5 * t * sp;
-    }
-    for (int i = k + 1 + tid; i < n; i += kTrdNT) wprev[i] = __ldcg(&pk[i]);
-    __syncthreads();
-    const double half = red[NW + 4];
-    for (int i = k + 1 + tid; i < n; i += kTrdNT) {
-      wprev[i] = fma(-half, vcur[i], wprev[i]);
-      vprev[i] = vcur[i];
-    }
-    __syncthreads();
-  }
-}
-
-// The trailing update after panel q: A(k1:, k1:) -= V W^T + W V^T (rows and
-// columns k1.., K = kPnb) on the tensor cores, as two FP64-accurate products
-// whose operand rows are each all reflector entries or all W entries (one
-// exponent per row then fits both, whatever the scale of C). Pack tiles: the
-// 64-row blocks of V (first half of the tile range, sized for q = 0), then
-// those of W.
-int tiles_trd_s2k_pack(int n) { return n > kPnb ? 2 * (oz_rows_padded(n - kPnb) / 64) : 0; }
-int tiles_trd_s2k(int n) { return n > kPnb ? ceil_div(n - kPnb, kOzBM) * ceil_div(n - kPnb, kOzBN) : 0; }
-
-__global__ void __launch_bounds__(kOzNT) k_trd_s2k_pack(Search* S, TileMap tm, int q) {
-  __shared__ int sh_e[64];
-  int tile;
-  const int si = find_search(tm, tile);
-  const Search& s = S[si];
-  if (!trd_due(s)) return;
-  const int n = s.n, k0 = kPnb * q, k1 = k0 + kPnb;
-  if (k1 >= n) return;
-  const int R = n - k1, half = oz_rows_padded(n - kPnb) / 64;
-  const int which = tile >= half ? 1 : 0, rb = tile - which * half;
-  if (rb >= oz_rows_padded(R) / 64) return;
-  const TrdOz lay = trd_oz_layout(n);
-  const long long L = s.ldn;
-  const double* X = which == 0 ? s.EX + (k1 + L * k0) : s.EG + k1;  // V(k1 + i, l) or W(k1 + i, l)
-  oz_pack_block_get([=] __device__(int i, int l) { return X[i + L * l]; }, false, R, kPnb, rb, oz_nks(kPnb),
-                    s.ozp + (which == 0 ? lay.s2a : lay.s2b), s.oze + (which == 0 ? lay.ev : lay.ew), sh_e);
-}
-
-__global__ void __launch_bounds__(kOzNT, 1) k_trd_s2k(Search* S, TileMap tm, int q) {
-  extern __shared__ unsigned char dyn[];
-  __shared__ uint64_t bar[5];
-  __shared__ uint32_t tslot;
-  int tile;
-  const int si = find_search(tm, tile);
-  const Search& s = S[si];
-  if (!trd_due(s)) return;
-  const int n = s.n, k1 = kPnb * q + kPnb;
-  if (k1 >= n) return;
-  const int R = n - k1, TN = ceil_div(n - kPnb, kOzBN), mt = tile / TN, nt = tile % TN;
-  if (mt * kOzBM >= R || nt * kOzBN >= R) return;
-  const TrdOz lay = trd_oz_layout(n);
-  const unsigned char* Vp = s.ozp + lay.s2a;
-  const unsigned char* Wq8 = s.ozp + lay.s2b;
-  const int* ev = s.oze + lay.ev;
-  const int* ew = s.oze + lay.ew;
-  OzCtx cx;
-  oz_begin(cx, dyn, bar, &tslot);
-  long long Wq[32];
-  float Lq[32];
-  const long long pitch = oz_pitch(oz_nks(kPnb));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = kOzBM * mt + 32 * (warp & 3) + lane, jb = kOzBN * nt + 32 * (warp >> 2);
-  const long long L = s.ldn;
-  double* Ai = s.EA + (k1 + i);
-  bool ok = true;
-  for (int part = 0; part < 2 && ok; ++part) {
-    // part 0: V_i . W_j, part 1: W_i . V_j
-    ok = oz_tile(cx, part == 0 ? Vp : Wq8, pitch, 2 * mt, part == 0 ? Wq8 : Vp, pitch, nt, oz_nks(kPnb), Wq, Lq);
-    if (ok && i < R) {
-      const int ei = part == 0 ? ev[i] : ew[i];
-      const int* eb = part == 0 ? ew : ev;
-#pragma unroll
-      for (int qq = 0; qq < 32; ++qq) {
-        const int jj = jb + qq;
-        if (jj < R) Ai[L * (k1 + jj)] -= oz_value(Wq[qq], Lq[qq], ei, eb[jj]);
-      }
-    }
-  }
-  if (!ok && threadIdx.x == 0) atomicOr(s.err, kDevErrTimeout);
-  oz_end(cx);
-}
 
 // --------------------------------------------------------------------------
 // Scans of one CTA over n entries (n <= 4096): last index u <= t with
@@ -688,11 +90,23 @@ __global__ void __launch_bounds__(kTrdNT) k_trd_blocks(Search* S, int s0) {
   Search& s = S[s0 + blockIdx.x];
   if (!trd_due(s)) return;
   const int n = s.n;
-  const double* d = tv(s, TV_D);
-  const double* e = tv(s, TV_E);
+  double* d = tv(s, TV_D);
+  double* e = tv(s, TV_E);
   double* es = tv(s, TV_ES);
   double* e2 = tv(s, TV_E2);
   double* sc = tv(s, TV_SCAL);
+  {  // from the reduction's integers: d in q above mu, tau in 2^-61, e in 2^(x - 62) q with x in TV_ES
+    const double q = sc[8], mu = sc[9];
+    double* tau = tv(s, TV_TAU);
+    for (int i = threadIdx.x; i < n; i += kTrdNT) {
+      d[i] = fma(static_cast<double>(__double_as_longlong(d[i])), q, mu);
+      if (i + 1 < n) {
+        e[i] = scalbn(static_cast<double>(__double_as_longlong(e[i])), static_cast<int>(__double_as_longlong(es[i])) - 62) * q;
+        tau[i] = static_cast<double>(__double_as_longlong(tau[i])) * 0x1p-61;
+      }
+    }
+    __syncthreads();
+  }
   double tn = 0.0, em = 0.0;
   for (int i = threadIdx.x; i < n; i += kTrdNT) {
     const double lo = i > 0 ? fabs(e[i - 1]) : 0.0, hi = i + 1 < n ? fabs(e[i]) : 0.0;
@@ -1634,26 +1048,7 @@ __global__ void __launch_bounds__(kTrdNT) k_trd_finish(Search* S, int s0) {
 // --------------------------------------------------------------------------
 // Host side
 // --------------------------------------------------------------------------
-size_t trd_reduce_smem(int max_n, int blocked) { return static_cast<size_t>(max_n) * (blocked ? 8 : 24); }
-
-int trd_reduce_blocks_per_sm(int max_n, int blocked) {
-  int b = 0;
-  const size_t smem = trd_reduce_smem(max_n, blocked);
-  const void* fn = blocked ? reinterpret_cast<const void*>(k_trd_panel) : reinterpret_cast<const void*>(k_trd_sytrd);
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kTrdNT, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return b;
-}
-
-void trd_set_attributes(int max_n) {
-  cudaFuncSetAttribute(k_trd_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       static_cast<int>(trd_reduce_smem(max_n, 1)));
-  cudaFuncSetAttribute(k_trd_sytrd, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       static_cast<int>(trd_reduce_smem(max_n, 0)));
-  cudaFuncSetAttribute(k_trd_s2k, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSmem);
+void trd_set_attributes() {
   cudaFuncSetAttribute(k_trd_oz_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSmem);
   bt_set_attributes();
 }
@@ -1662,8 +1057,8 @@ void trd_set_attributes(int max_n) {
 // after each stage (reduction, eigenvalues, inverse iteration, Gram-Schmidt in
 // clusters, orthogonalisation, back-transformation), for the per-stage times
 // of the profiling mode.
-int launch_eig_trd(Search* S, const int4* grp, const TrdChunk* chunks, int nchunks, unsigned* bars,
-                   int bar_count, int s0, int s1, const TrdMaps& tm, int max_n, int bis_lanes, cudaStream_t st,
+int launch_eig_trd(Search* S, const int4* grp, const TrdChunk* chunks, int nchunks, unsigned* bars, int s0, int s1,
+                   const TrdReducePlan& plan, const TrdMaps& tm, int max_n, int bis_lanes, cudaStream_t st,
                    cudaEvent_t* marks) {
   if (nchunks <= 0 || s1 <= s0) return 0;
   int nl = 0;
@@ -1671,35 +1066,7 @@ int launch_eig_trd(Search* S, const int4* grp, const TrdChunk* chunks, int nchun
     if (marks) cudaEventRecord(marks[k], st);
   };
   mark(0);
-  int q_prev = -2;  // chunks of the unblocked form carry panel -1
-  for (int c = 0; c < nchunks; ++c) {
-    const int q = chunks[c].panel;
-    if (q != q_prev) {
-      if (q_prev >= 0 && q >= 0 && tm.s2kp.total > 0 && tm.s2k.total > 0) {  // the previous panel's trailing update
-        k_trd_s2k_pack<<<tm.s2kp.total, kOzNT, 0, st>>>(S, tm.s2kp, q_prev);
-        k_trd_s2k<<<tm.s2k.total, kOzNT, kOzSmem, st>>>(S, tm.s2k, q_prev);
-        nl += 2;
-      }
-      // the group barriers and work counters restart per panel
-      cudaMemsetAsync(bars, 0, sizeof(unsigned) * bar_count * kTrdBarStride, st);
-      q_prev = q;
-    }
-    if (chunks[c].count <= 0) continue;
-    const bool blocked = q >= 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(chunks[c].count);
-    cfg.blockDim = dim3(kTrdNT);
-    cfg.dynamicSmemBytes = trd_reduce_smem(max_n, blocked ? 1 : 0);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (blocked) cudaLaunchKernelEx(&cfg, k_trd_panel, S, grp + chunks[c].first, q);
-    else cudaLaunchKernelEx(&cfg, k_trd_sytrd, S, grp + chunks[c].first);
-    ++nl;
-  }
+  nl += launch_trd_reduce(S, grp, chunks, nchunks, bars, s0, s1, plan, st);
   mark(1);
   k_trd_blocks<<<s1 - s0, kTrdNT, 0, st>>>(S, s0);
   if (bis_lanes > 1) k_trd_bisect<kTrdBisLanes><<<tm.tbis.total, kTrdTT, 0, st>>>(S, tm.tbis);

@@ -36,6 +36,18 @@ constexpr int kTrdNT = 256;
 
 __device__ __forceinline__ bool trd_due(const Search& s) { return s.trd && !s.done && s.eig_due; }
 
+__device__ __forceinline__ double warp_sum_xor(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ double* tv(const Search& s, int which) {
   return s.trd_v + static_cast<long long>(which) * s.ldn;
 }
@@ -54,14 +66,11 @@ __device__ __forceinline__ int* ti(const Search& s, int which) {
 //   w   the columns of W = Y_p^T V (or T_p W) as a packed operand (K = 128)
 //   g, tf  per panel, Y_p^T Y_p and T_p in FP64 (128 x 128, column-major)
 //   wf  W in FP64 (128 x n, column-major)
-//   s2a, s2b  the reduction's trailing update: [V W] and [W V] (K = 2 kPnb)
 // Search::oze, int offsets: v [0, np), w [np, 2 np), yt 2 np + 128 p,
 // y 2 np + 128 P + (padded rows of the earlier panels), t after y (128 per
 // panel), with np the padded n.
 // --------------------------------------------------------------------------
 constexpr int kBtNb = 128;  // reflectors per panel of the back-transformation
-constexpr int kPnb = kTrdPanel;  // columns per panel of the reduction
-constexpr int kPartStride = 2 * kPnb + 8;  // per-CTA partial sums of a reduction step
 // Back-transformation: blocked on the tensor cores from this size on, one
 // register-resident column per warp in FP64 below it. The launches of the
 // blocked form are shared by every search of a batch, so in a large batch it
@@ -80,7 +89,7 @@ __host__ __device__ inline int trd_panel_nb(int n, int p) {
 }
 
 struct TrdOz {
-  size_t v, yt, y, t, w, g, tf, wf, s2a, s2b, total;  // bytes
+  size_t v, yt, y, t, w, g, tf, wf, total;  // bytes
   int ev, ew, eyt, ey, et, etotal;         // ints
 };
 
@@ -104,10 +113,6 @@ __host__ __device__ inline TrdOz trd_oz_layout(int n) {
   o += static_cast<size_t>(P) * kBtNb * kBtNb * 8;
   L.wf = o;
   o += trd_align256(static_cast<size_t>(kBtNb) * n * 8);
-  L.s2a = o;
-  o += trd_align256(oz_bytes(n, 2 * kPnb));
-  L.s2b = o;
-  o += trd_align256(oz_bytes(n, 2 * kPnb));
   L.total = o;
   int e = 0;
   L.ev = e;
