@@ -55,7 +55,7 @@ struct cmaes_s {
   // tridiagonal route: largest n, the CTA -> (search, member, group size) table
   // of the cooperative reduction, and one barrier counter per search
   int max_n_trd = 0;
-  int trd_bis_lanes = 8;  // lanes per eigenvalue of the multisection (1 for large batches)
+  int trd_bis_lanes = 8;  // lanes per eigenvalue of the multisection
   int4* d_trd_grp = nullptr;
   int trd_grp_blocks = 0;
   std::vector<TrdChunk> trd_chunks;  // the cooperative launches of the reduction
@@ -863,12 +863,10 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     }
     h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start});
     h->trd_grp_blocks = static_cast<int>(grp.size());
-    // eigenvalues to find per decomposition of the whole batch: with more than
-    // the GPU holds as 8-lane groups, plain bisection does the least work
     long long eig_total = 0;
     for (int s = 0; s < count; ++s)
       if (h->hs[s].trd) eig_total += h->hs[s].n;
-    h->trd_bis_lanes = eig_total * 8 > static_cast<long long>(sms) * 2048 ? 1 : 8;
+    h->trd_bis_lanes = trd_bis_lanes(eig_total);
     CREATE_TRY(cudaMalloc(&h->d_trd_grp, sizeof(int4) * grp.size()));
     CREATE_TRY(cudaMemcpyAsync(h->d_trd_grp, grp.data(), sizeof(int4) * grp.size(), cudaMemcpyHostToDevice,
                                h->stream));
@@ -904,7 +902,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
         case TK_REEVAL: t = h->mixed ? tiles_reeval(x.n) : 0; break;
         case TK_FLATSYM: t = eig_refined_route(x) ? tiles_flat_sym(x.n) : 0; break;
         case TK_TRD: t = x.trd ? tiles_trd(x.n) : 0; break;
-        case TK_TRDBIS: t = x.trd ? tiles_trd_bis(x.n) : 0; break;
+        case TK_TRDBIS: t = x.trd ? tiles_trd_bis(x.n, h->trd_bis_lanes) : 0; break;
         case TK_TRDSQ: t = x.trd ? tiles_trd_sq(x.n) : 0; break;
         case TK_TRDBT: t = x.trd ? tiles_trd_bt(x.n) : 0; break;
         case TK_TRDOZP: t = x.trd ? tiles_trd_ozp(x.n) : 0; break;

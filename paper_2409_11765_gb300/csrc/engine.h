@@ -225,8 +225,9 @@ void set_global_error(const char* msg);
 constexpr int kEigAutoTrdN = kEigMixedMaxN;
 constexpr int kTrdVectors = 11;  // Search::trd_v, in ldn doubles
 constexpr int kTrdInts = 5;      // Search::trd_i, in ldn ints
-int tiles_trd(int n);      // 128 eigenvalues per tile
-int tiles_trd_bis(int n);  // 16 eigenvalues per tile (8 lanes each)
+int tiles_trd(int n);      // 32 eigenvalues per tile
+int tiles_trd_bis(int n, int lanes);  // 32 / lanes eigenvalues per tile
+int trd_bis_lanes(long long eigenvalues);
 int tiles_trd_sq(int n);   // all 64 x 64 tiles of n x n
 int tiles_trd_bt(int n);   // column groups of the back-transformation
 int tiles_trd_ozp(int n);  // 64-row blocks of a packed n x n operand

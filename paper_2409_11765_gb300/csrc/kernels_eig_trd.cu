@@ -37,6 +37,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 #include "device_common.cuh"
 #include "ozaki.cuh"
 #include "trd_common.cuh"
@@ -116,26 +117,25 @@ __global__ void __launch_bounds__(kTrdNT) k_trd_blocks(Search* S, int s0) {
   tn = block_max<kTrdNT>(tn, red);
   em = block_max<kTrdNT>(em, red);
   const double split = kTrdSplit * sqrt(static_cast<double>(n)) * kTrdEps * tn;
-  for (int i = threadIdx.x; i + 1 < n; i += kTrdNT) {
-    const double x = fabs(e[i]) <= split ? 0.0 : e[i];
-    es[i] = x;
-    e2[i] = x * x;
-  }
-  // d and e^2 scaled by a power of two (|d| <= 1) in FP32 for the first
-  // bisection steps (the reduction's buffers TV_P0 and TV_P1 are free now)
+  for (int i = threadIdx.x; i + 1 < n; i += kTrdNT) es[i] = fabs(e[i]) <= split ? 0.0 : e[i];
+  // d (TV_SD) and e^2 (TV_E2) scaled by a power of two (|d| <= 1) for the
+  // bisection, and as pairs hi + lo of floats (hi the rounded value, lo the
+  // rounded rest): d at TV_P0 (hi, then lo from ldn on), e^2 at TV_P1 likewise
+  // (the reduction's buffers are free now)
   const double scl = tn > 0.0 ? exp2(-static_cast<double>(ilogb(tn) + 1)) : 1.0;
-  // as pairs hi + lo of floats (hi the rounded value, lo the rounded rest):
-  // d at TV_P0 (hi, then lo from ldn on), e^2 at TV_P1 likewise
+  double* sd = tv(s, TV_SD);
   float* d32 = reinterpret_cast<float*>(tv(s, TV_P0));
   float* e32 = reinterpret_cast<float*>(tv(s, TV_P1));
   const long long L2 = s.ldn;
   for (int i = threadIdx.x; i < n; i += kTrdNT) {
     const double ds = d[i] * scl;
+    sd[i] = ds;
     d32[i] = static_cast<float>(ds);
     d32[L2 + i] = static_cast<float>(ds - static_cast<double>(d32[i]));
     if (i + 1 < n) {
       const double x = fabs(e[i]) <= split ? 0.0 : e[i] * scl;
       const double x2 = x * x;
+      e2[i] = x2;
       e32[i] = static_cast<float>(x2);
       e32[L2 + i] = static_cast<float>(x2 - static_cast<double>(e32[i]));
     }
@@ -160,129 +160,185 @@ __global__ void __launch_bounds__(kTrdNT) k_trd_blocks(Search* S, int s0) {
 // --------------------------------------------------------------------------
 // 3. Multisection: a group of LANES lanes finds eigenvalue t - b0 (ascending)
 // of its block; each round the lanes take the Sturm counts at LANES interior
-// points of the bracket, which shrinks it (LANES + 1)-fold. Eight lanes cut the
-// sequential rounds from ~52 to ~17 for the few eigenvalues of one search; a
-// large batch, which fills the GPU with eigenvalues anyway, takes one lane
-// (plain bisection: the fewest counts in total). The counts' reciprocals come
-// from an FP32 estimate and two Newton steps in FP64 (exact to rounding)
-// instead of an FP64 divide.
+// points of the bracket, which shrinks it (LANES + 1)-fold: fewer sequential
+// rounds for more counts in all.
+//
+// A Sturm count is the number of sign changes of the leading minors of T - x I,
+//   p_j = (d_j - x) p_{j-1} - e_{j-1}^2 p_{j-2},
+// rescaled by a power of two every few rows. Per row the dependent chain is one
+// FMA (the quotient form p_j / p_{j-1} has a reciprocal on it: FP64 ~600 clocks
+// a row against ~75) and the FP64 work three operations against ten. As with
+// the quotients, the computed signs are exact for a T whose d_j - x and e_j^2
+// are off by a few rounding errors each. A zero p_j takes the sign opposite to
+// p_{j-1} (a pivot -0), shrunk far below it.
 // --------------------------------------------------------------------------
-constexpr int kTrdTT = 128;   // threads per tile of the per-eigenvalue kernels
-constexpr int kTrdBisLanes = 8;
+// Threads per tile of the per-eigenvalue kernels: one warp, so that the warps
+// of a single search spread over the SMs and their FP64 pipes.
+constexpr int kTrdTT = 32;
 int tiles_trd(int n) { return ceil_div(n, kTrdTT); }
-int tiles_trd_bis(int n) { return ceil_div(n * kTrdBisLanes, kTrdTT); }
+int tiles_trd_bis(int n, int lanes) { return ceil_div(n * lanes, kTrdTT); }
 
-// 1 / q from the FP32 reciprocal and two Newton steps inside 2^-99 < |q| <
-// 2^99 (exponent tested on the integer pattern), the division elsewhere.
-__device__ __forceinline__ double fast_rcp(double q) {
-  const int ex = (__double2hiint(q) >> 20) & 0x7FF;
-  if (ex > 1023 - 99 && ex < 1023 + 99) {
-    double r = static_cast<double>(__frcp_rn(static_cast<float>(q)));
-    r = r * fma(-q, r, 2.0);
-    return r * fma(-q, r, 2.0);
-  }
-  return 1.0 / q;
+// Lanes per eigenvalue by the number of eigenvalues of the handle's searches:
+// the rounds' latency against the counts' FP64 work (three operations of ~19
+// clocks per warp and row on each SM).
+int trd_bis_lanes(long long eigenvalues) {
+  return eigenvalues <= 700 ? 16 : eigenvalues <= 2500 ? 8 : eigenvalues <= 7000 ? 4 : 1;
 }
 
-// Sturm count: eigenvalues of block [b0, b1) below x (pivots of magnitude at
-// most pivmin replaced by -pivmin; |q| and pivmin compared as ordered bit
-// patterns, the sign read from the sign bit).
-__device__ __forceinline__ int sturm64(const double* d, const double* e2, int b0, int b1, double x, double pivmin) {
-  const long long pb = __double_as_longlong(pivmin);
+// Eigenvalues of block [b0, b1) below x; d and e2 the scaled copies (|d| <= 1).
+__device__ __forceinline__ int sturm64(const double* __restrict__ d, const double* __restrict__ e2, int b0, int b1,
+                                       double x) {
+  double p0 = 1.0, p1 = d[b0] - x;
   int cnt = 0;
-  double qq = d[b0] - x;
-  if ((__double_as_longlong(qq) & 0x7FFFFFFFFFFFFFFFLL) <= pb) qq = -pivmin;
-  cnt += static_cast<int>(static_cast<unsigned long long>(__double_as_longlong(qq)) >> 63);
-  for (int j = b0 + 1; j < b1; ++j) {
-    qq = (d[j] - x) - e2[j - 1] * fast_rcp(qq);
-    if ((__double_as_longlong(qq) & 0x7FFFFFFFFFFFFFFFLL) <= pb) qq = -pivmin;
-    cnt += static_cast<int>(static_cast<unsigned long long>(__double_as_longlong(qq)) >> 63);
+  auto row = [&](double p, double before) -> double {  // counts the sign change from `before`
+    if (((__double2hiint(p) & 0x7fffffff) | __double2loint(p)) == 0)
+      p = __hiloint2double((__double2hiint(before) ^ static_cast<int>(0x80000000u)) - (100 << 20), 0);
+    cnt += static_cast<int>(static_cast<unsigned>(__double2hiint(p) ^ __double2hiint(before)) >> 31);
+    return p;
+  };
+  p1 = row(p1, p0);
+  int j = b0 + 1;
+  for (; j + 8 <= b1; j += 8) {
+    double dd[8], ee[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      dd[u] = d[j + u];
+      ee[u] = e2[j + u - 1];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double p = row(fma(dd[u] - x, p1, -(ee[u] * p0)), p1);
+      p0 = p1;
+      p1 = p;
+    }
+    const int ex = max(__double2hiint(p1) & 0x7ff00000, __double2hiint(p0) & 0x7ff00000);
+    if (ex < ((1023 - 200) << 20) || ex > ((1023 + 200) << 20)) {
+      const double sc = __hiloint2double((2046 << 20) - ex, 0);
+      p0 *= sc;
+      p1 *= sc;
+    }
+  }
+  for (; j < b1; ++j) {
+    const double p = row(fma(d[j] - x, p1, -(e2[j - 1] * p0)), p1);
+    p0 = p1;
+    p1 = p;
   }
   return cnt;
 }
 
-// The same in FP32 on the scaled copies (|d| <= 1).
-__device__ __forceinline__ int sturm32(const float* d, const float* e2, int b0, int b1, float x) {
-  constexpr float piv = 0x1p-90f;
+// The power of two that brings the larger of two floats near 1.
+__device__ __forceinline__ float rescale32(float a, float b) {
+  const int ex = max(__float_as_int(a) & 0x7f800000, __float_as_int(b) & 0x7f800000);
+  return __int_as_float((254 << 23) - min(max(ex, 1 << 23), 253 << 23));
+}
+
+// The same in FP32.
+__device__ __forceinline__ int sturm32(const float* __restrict__ d, const float* __restrict__ e2, int b0, int b1,
+                                       float x) {
+  float p0 = 1.0f, p1 = d[b0] - x;
   int cnt = 0;
-  float qq = d[b0] - x;
-  if (fabsf(qq) <= piv) qq = -piv;
-  cnt += qq < 0.0f;
-  for (int j = b0 + 1; j < b1; ++j) {
-    qq = (d[j] - x) - e2[j - 1] * __frcp_rn(qq);
-    if (fabsf(qq) <= piv) qq = -piv;
-    cnt += qq < 0.0f;
+  auto row = [&](float p, float before) -> float {
+    if (p == 0.0f) p = before * -0x1p-30f;
+    cnt += static_cast<int>(static_cast<unsigned>(__float_as_int(p) ^ __float_as_int(before)) >> 31);
+    return p;
+  };
+  p1 = row(p1, p0);
+  int j = b0 + 1;
+  for (; j + 4 <= b1; j += 4) {
+    float dd[4], ee[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      dd[u] = d[j + u];
+      ee[u] = e2[j + u - 1];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float p = row(fmaf(dd[u] - x, p1, -(ee[u] * p0)), p1);
+      p0 = p1;
+      p1 = p;
+    }
+    const float sc = rescale32(p0, p1);
+    p0 *= sc;
+    p1 *= sc;
+  }
+  for (; j < b1; ++j) {
+    const float p = row(fmaf(d[j] - x, p1, -(e2[j - 1] * p0)), p1);
+    p0 = p1;
+    p1 = p;
   }
   return cnt;
 }
 
 // The same in double-float arithmetic (each value a pair hi + lo of floats,
-// ~48 significant bits; error-free sums and products from FMA) on the scaled
-// pairs: d at d32 / d32 + ldn, e^2 at e32 / e32 + ldn, x = xh + xl.
+// ~46 significant bits; error-free sums and products from FMA) on the scaled
+// pairs: d at dh / dl, e^2 at eh / el, x = xh + xl.
+struct Df {
+  float h, l;
+};
 __device__ __forceinline__ void df_two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   const float bb = __fsub_rn(s, a);
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
-__device__ __forceinline__ int sturm_df(const float* dh, const float* dl, const float* eh, const float* el,
-                                        int b0, int b1, float xh, float xl) {
-  constexpr float piv = 0x1p-90f;
+__device__ __forceinline__ Df df_sub(Df a, Df b) {
+  float s, e;
+  df_two_sum(a.h, -b.h, s, e);
+  e = __fadd_rn(e, __fsub_rn(a.l, b.l));
+  const float h = __fadd_rn(s, e);
+  return Df{h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ Df df_mul(Df a, Df b) {
+  const float h = __fmul_rn(a.h, b.h);
+  return Df{h, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -h)))};
+}
+__device__ __forceinline__ int sturm_df(const float* __restrict__ dh, const float* __restrict__ dl,
+                                        const float* __restrict__ eh, const float* __restrict__ el, int b0, int b1,
+                                        float xh, float xl) {
+  const Df x{xh, xl};
+  Df p0{1.0f, 0.0f}, p1 = df_sub(Df{dh[b0], dl[b0]}, x);
   int cnt = 0;
-  float qh, ql;
-  {
-    float s, e;
-    df_two_sum(dh[b0], -xh, s, e);
-    e = __fadd_rn(e, __fsub_rn(dl[b0], xl));
-    qh = __fadd_rn(s, e);
-    ql = __fsub_rn(e, __fsub_rn(qh, s));
-  }
-  if (fabsf(qh) <= piv) {
-    qh = -piv;
-    ql = 0.0f;
-  }
-  cnt += qh < 0.0f;
-  for (int j = b0 + 1; j < b1; ++j) {
-    // t = d_j - x
-    float th, tl;
-    {
-      float s, e;
-      df_two_sum(dh[j], -xh, s, e);
-      e = __fadd_rn(e, __fsub_rn(dl[j], xl));
-      th = __fadd_rn(s, e);
-      tl = __fsub_rn(e, __fsub_rn(th, s));
+  auto row = [&](Df p, float before) -> Df {
+    if (p.h == 0.0f) p = Df{before * -0x1p-30f, 0.0f};
+    cnt += static_cast<int>(static_cast<unsigned>(__float_as_int(p.h) ^ __float_as_int(before)) >> 31);
+    return p;
+  };
+  p1 = row(p1, p0.h);
+  int j = b0 + 1;
+  for (; j + 4 <= b1; j += 4) {
+    Df dd[4], ee[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      dd[u] = Df{dh[j + u], dl[j + u]};
+      ee[u] = Df{eh[j + u - 1], el[j + u - 1]};
     }
-    // u = e2 / q: leading quotient, then the rest from the exact residual
-    const float e2h = eh[j - 1], e2l = el[j - 1];
-    const float uh = __fdiv_rn(e2h, qh);
-    const float p = __fmul_rn(uh, qh);
-    const float pe = __fmaf_rn(uh, qh, -p);
-    const float r = __fadd_rn(__fsub_rn(__fsub_rn(e2h, p), pe), __fmaf_rn(-uh, ql, e2l));
-    const float ul = __fdiv_rn(r, qh);
-    // q = t - u
-    float s, e;
-    df_two_sum(th, -uh, s, e);
-    e = __fadd_rn(e, __fsub_rn(tl, ul));
-    qh = __fadd_rn(s, e);
-    ql = __fsub_rn(e, __fsub_rn(qh, s));
-    if (fabsf(qh) <= piv) {
-      qh = -piv;
-      ql = 0.0f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const Df p = row(df_sub(df_mul(df_sub(dd[u], x), p1), df_mul(ee[u], p0)), p1.h);
+      p0 = p1;
+      p1 = p;
     }
-    cnt += qh < 0.0f;
+    const float sc = rescale32(p0.h, p1.h);
+    p0 = Df{p0.h * sc, p0.l * sc};
+    p1 = Df{p1.h * sc, p1.l * sc};
+  }
+  for (; j < b1; ++j) {
+    const Df p = row(df_sub(df_mul(df_sub(Df{dh[j], dl[j]}, x), p1), df_mul(Df{eh[j - 1], el[j - 1]}, p0)), p1.h);
+    p0 = p1;
+    p1 = p;
   }
   return cnt;
 }
 
 // Eigenvalue t of its block by bisection (LANES = 1) or multisection with
-// LANES points per step, in three precisions: FP32 on the scaled block down to
+// LANES points per step, in three precisions, on the scaled copies: FP32 down to
 // a width of 2^-19 ||T||, widened by 2^-18 ||T|| (eight times the backward
 // error of an FP32 Sturm count, ~10 eps32 ||T||); double-float down to
-// 2^-43 ||T||, widened by 2^-42 ||T|| (six times that of a double-float
-// count, ~10 2^-48 ||T||); each widened bracket checked with two counts of
+// 2^-42 ||T||, widened by 2^-41 ||T|| (several times that of a double-float
+// count, ~10 2^-46 ||T||); each widened bracket checked with two counts of
 // the next precision (the previous bracket kept if the check fails), the
-// last step in FP64 to 4 eps64 ||T||. The FP64 counts are the bulk of the
-// work (the FP64 pipe is ~80 % busy), so every precision goes as far as its
-// counts stay reliable.
+// last step in FP64 to 4 eps64 ||T||. FP32 and double-float rows cost a warp
+// ~4 and ~10 clocks of an SM, an FP64 row 57, so every precision goes as far as
+// its counts stay reliable.
 template <int LANES>
 __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
   int tile;
@@ -295,8 +351,7 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
   if (t >= n) return;  // uniform across the lanes of a group
   const int base = (threadIdx.x & 31) & ~(LANES - 1);
   const unsigned gmask = static_cast<unsigned>((1ull << LANES) - 1) << base;
-  const double* d = tv(s, TV_D);
-  const double* es = tv(s, TV_ES);
+  const double* d = tv(s, TV_SD);
   const double* e2 = tv(s, TV_E2);
   const float* d32 = reinterpret_cast<const float*>(tv(s, TV_P0));
   const float* e32 = reinterpret_cast<const float*>(tv(s, TV_P1));
@@ -304,14 +359,14 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
   double* lamb = tv(s, TV_LAMB);
   const int b0 = ti(s, TI_B0)[t], b1 = ti(s, TI_B1)[t];
   if (b1 - b0 == 1) {
-    if (q == 0) lamb[t] = d[t];
+    if (q == 0) lamb[t] = tv(s, TV_D)[t];
     return;
   }
   // the start bracket: [-||T||, ||T||] with ||T|| the largest Gershgorin row
   // sum of the unsplit T (it holds every block's spectrum), widened for rounding
-  const double tn = sc[0], pivmin = sc[1], scl = sc[7];
+  const double scl = sc[7], tn = sc[0] * scl;  // in [1/2, 1), or 0
   const double atol = 4.0 * kTrdEps * tn;
-  const double fudge = 2.0 * kTrdEps * tn * (b1 - b0) + 2.0 * pivmin;
+  const double fudge = 2.0 * kTrdEps * tn * (b1 - b0) + 0x1p-1000;
   double lo = -tn - fudge, hi = tn + fudge;
   const int idx = t - b0;
   // one multisection step on [lo, hi] from the counts of the LANES points
@@ -329,24 +384,23 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
   // the left end, lane 1 the right one; one lane does both)
   auto check = [&](auto cnt, double a, double b) -> bool {
     if (LANES == 1) return cnt(a) <= idx && cnt(b) > idx;
-    bool mine = true;
-    if (q == 0) mine = cnt(a) <= idx;
-    if (q == 1) mine = cnt(b) > idx;
+    const int c = cnt(q == 0 ? a : b);
+    const bool mine = q == 0 ? c <= idx : q == 1 ? c > idx : true;
     return (__ballot_sync(gmask, !mine) & gmask) == 0;
   };
   if (tn > 0.0) {
     const long long L2 = s.ldn;
     // FP32
-    float lo32 = static_cast<float>(lo * scl), hi32 = static_cast<float>(hi * scl);
+    float lo32 = static_cast<float>(lo), hi32 = static_cast<float>(hi);
     for (int it = 0; it < 40 && hi32 - lo32 > 0x1p-19f; ++it) {
       const float w = (hi32 - lo32) / (LANES + 1);
       if (!narrow(lo32, hi32, sturm32(d32, e32, b0, b1, lo32 + w * (q + 1)), w)) break;
     }
-    auto cnt_df = [&](double xs) {  // x given scaled, in FP64
+    auto cnt_df = [&](double xs) {
       const float xh = static_cast<float>(xs);
       return sturm_df(d32, d32 + L2, e32, e32 + L2, b0, b1, xh, static_cast<float>(xs - static_cast<double>(xh)));
     };
-    double los = lo * scl, his = hi * scl;  // scaled bracket, FP64
+    double los = lo, his = hi;
     {
       const double a = fmax(los, static_cast<double>(lo32) - 0x1p-18), b = fmin(his, static_cast<double>(hi32) + 0x1p-18);
       if (a < b && check(cnt_df, a, b)) {
@@ -355,26 +409,27 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
       }
     }
     // double-float
-    for (int it = 0; it < 60 && his - los > 0x1p-43; ++it) {
-      const double w = (his - los) / (LANES + 1);
+    for (int it = 0; it < 60 && his - los > 0x1p-42; ++it) {
+      const double w = (his - los) * (1.0 / (LANES + 1));
       if (!narrow(los, his, cnt_df(los + w * (q + 1)), w)) break;
     }
-    const double lo2 = fmax(lo, (los - 0x1p-42) / scl), hi2 = fmin(hi, (his + 0x1p-42) / scl);
-    if (lo2 < hi2 && check([&](double x) { return sturm64(d, e2, b0, b1, x, pivmin); }, lo2, hi2)) {
+    const double lo2 = fmax(lo, los - 0x1p-41), hi2 = fmin(hi, his + 0x1p-41);
+    if (lo2 < hi2 && check([&](double x) { return sturm64(d, e2, b0, b1, x); }, lo2, hi2)) {
       lo = lo2;
       hi = hi2;
     }
   }
   for (int it = 0; it < 160 && hi - lo > atol; ++it) {
-    const double w = (hi - lo) / (LANES + 1);
-    if (!narrow(lo, hi, sturm64(d, e2, b0, b1, lo + w * (q + 1), pivmin), w)) break;
+    const double w = (hi - lo) * (1.0 / (LANES + 1));
+    if (!narrow(lo, hi, sturm64(d, e2, b0, b1, lo + w * (q + 1)), w)) break;
   }
-  if (q == 0) lamb[t] = 0.5 * (lo + hi);
+  if (q == 0) lamb[t] = 0.5 * (lo + hi) / scl;
 }
 
 // --------------------------------------------------------------------------
-// 4a. Ranks of the eigenvalues (ascending, ties by block-major index) and the
-// clusters of close eigenvalues within a block (one CTA per search).
+// 4a. Ranks of the eigenvalues (ascending, ties by block-major index; one thread
+// each) and the clusters of close eigenvalues within a block (one CTA per
+// search).
 // --------------------------------------------------------------------------
 constexpr int kTrdSortNT = 1024;
 
@@ -383,28 +438,35 @@ __device__ __forceinline__ long long order_key(double x) {
   return b >= 0 ? b : (b ^ 0x7fffffffffffffffLL);
 }
 
-__global__ void __launch_bounds__(kTrdSortNT) k_trd_rank(Search* S, int s0) {
+__global__ void __launch_bounds__(kTrdTT) k_trd_rank(Search* S, TileMap tm) {
+  int tile;
+  const int si = find_search(tm, tile);
+  const Search& s = S[si];
+  if (!trd_due(s)) return;
+  const int n = s.n, t = tile * kTrdTT + threadIdx.x;
+  if (t >= n) return;
+  const double* __restrict__ lamb = tv(s, TV_LAMB);
+  const double lt = lamb[t];
+  const long long kt = order_key(lt);
+  int r = 0;
+#pragma unroll 8
+  for (int u = 0; u < n; ++u) {
+    const long long ku = order_key(lamb[u]);
+    r += (ku < kt) || (ku == kt && u < t);
+  }
+  ti(s, TI_RANK)[t] = r;
+  tv(s, TV_LAMS)[r] = lt;
+}
+
+__global__ void __launch_bounds__(kTrdSortNT) k_trd_clusters(Search* S, int s0) {
   __shared__ int shi[kTrdSortNT];
   Search& s = S[s0 + blockIdx.x];
   if (!trd_due(s)) return;
-  const int n = s.n;
   const double* lamb = tv(s, TV_LAMB);
-  double* lams = tv(s, TV_LAMS);
-  int* rank = ti(s, TI_RANK);
   const int* b0 = ti(s, TI_B0);
   const double ctol = tv(s, TV_SCAL)[3];
-  for (int t = threadIdx.x; t < n; t += kTrdSortNT) {
-    const long long kt = order_key(lamb[t]);
-    int r = 0;
-    for (int u = 0; u < n; ++u) {
-      const long long ku = order_key(lamb[u]);
-      r += (ku < kt) || (ku == kt && u < t);
-    }
-    rank[t] = r;
-    lams[r] = lamb[t];
-  }
   scan_last_start<kTrdSortNT>(
-      n, [&](int u) { return u == b0[u] || !(lamb[u] - lamb[u - 1] <= ctol); }, ti(s, TI_CL0), shi);
+      s.n, [&](int u) { return u == b0[u] || !(lamb[u] - lamb[u - 1] <= ctol); }, ti(s, TI_CL0), shi);
 }
 
 // --------------------------------------------------------------------------
@@ -424,7 +486,27 @@ __device__ __forceinline__ double start_value(int t, int j) {
 }
 
 constexpr long long kInvitSwap = 0x7ff8000000000000LL;  // a quiet NaN: the row-interchange flag
+constexpr int kInvitU = 16;                              // rows whose loads are in flight together
 
+// 1 / m: an FP32 seed of the mantissa, built and read back on the integer pipe,
+// and one third-order Newton step (FP64 divides take ~560 clocks, this ~280);
+// the division itself near the ends of the exponent range.
+__device__ __forceinline__ double reciprocal(double m) {
+  const int h = __double2hiint(m), ex = (h >> 20) & 0x7ff;
+  if (ex < 8 || ex > 2038) return 1.0 / m;
+  const float f = __int_as_float(0x3f800000 | ((h & 0xfffff) << 3) |
+                                 static_cast<int>(static_cast<unsigned>(__double2loint(m)) >> 29));
+  const int b = __float_as_int(__fdividef(1.0f, f));  // in (1/2, 1]
+  double r = __hiloint2double(((b >> 3) + ((1023 - 127 + 1023 - ex) << 20)) | (h & static_cast<int>(0x80000000u)), b << 29);
+  const double g = fma(-m, r, 1.0);
+  r = fma(r, fma(g, g, g), r);
+  return r;
+}
+
+// The rows are a chain (factorisation ~6 dependent FP64 operations, forward 1,
+// back 2), so what is not on it is kept off it: the loads of kInvitU rows are
+// issued together before their chain (one load a row behind each step of it was
+// most of the time), and an iterate is scaled while the next solve reads it.
 __global__ void __launch_bounds__(kTrdTT) k_trd_invit(Search* S, TileMap tm) {
   int tile;
   const int si = find_search(tm, tile);
@@ -433,86 +515,130 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_invit(Search* S, TileMap tm) {
   const int n = s.n, t = tile * kTrdTT + threadIdx.x;
   if (t >= n) return;
   const long long L = s.ldn, nn = n;
-  const double* d = tv(s, TV_D);
-  const double* es = tv(s, TV_ES);
+  const double* __restrict__ d = tv(s, TV_D);
+  const double* __restrict__ es = tv(s, TV_ES);
   const double lam = tv(s, TV_LAMB)[t];
   const double tiny = kTrdEps * tv(s, TV_SCAL)[0];
   const int b0 = ti(s, TI_B0)[t], b1 = ti(s, TI_B1)[t];
-  double* x = s.ET + L * t;
-  for (int i = 0; i < n; ++i) x[i] = 0.0;
+  double* v_out = s.ET + L * t;
+  for (int i = 0; i < b0; ++i) v_out[i] = 0.0;
+  for (int i = b1; i < n; ++i) v_out[i] = 0.0;
   if (b1 - b0 == 1) {
-    x[t] = 1.0;
+    v_out[t] = 1.0;
     return;
   }
-  double* u0 = s.EA;
-  double* u1 = s.EG;
-  double* u2 = s.EH;
-  auto piv_of = [&](double a) { return fabs(a) > tiny ? a : (a < 0.0 ? -tiny : tiny); };
-  // factorisation of T - lambda I, once for the three solves: row j without
-  // an interchange keeps 1 / pivot (u0), its superdiagonal (u1) and the
-  // multiplier (u2); a row with one keeps the multiplier (u0) and the flag
-  // kInvitSwap in u1 (its U row, e_j, d_{j+1} - lambda, e_{j+1}, is read from
-  // T again when it is needed)
-  double a = d[b0] - lam, b = es[b0], c = 0.0;
-  for (int j = b0; j + 1 < b1; ++j) {
-    const double sub = es[j], nd = d[j + 1] - lam, nsup = (j + 2 < b1) ? es[j + 1] : 0.0;
-    const long long o = j * nn + t;
-    if (fabs(a) >= fabs(sub)) {
-      const double r = 1.0 / piv_of(a);
-      const double l = sub * r;
+  // the iterate and the factors interleaved by thread, so that a warp's access
+  // to a row is one line (B is free until the back-transformation writes it)
+  double* x = s.B + t;
+  double* u0 = s.EA + t;
+  double* u1 = s.EG + t;
+  double* u2 = s.EH + t;
+  // |a| as an ordered integer: comparing those keeps FP64 compares (~104 clocks) off the chain
+  auto magnitude = [](double a) { return __double_as_longlong(a) & 0x7fffffffffffffffLL; };
+  auto piv_of = [&](double a) { return magnitude(a) > magnitude(tiny) ? a : copysign(tiny, a); };
+  // factorisation of T - lambda I, once for the three solves: row j keeps its
+  // multiplier (u2), the reciprocal of its pivot (u0), and its superdiagonal or,
+  // for an interchanged row, the flag kInvitSwap (u1; the rest of its U row,
+  // d_{j+1} - lambda and e_{j+1}, is read from T again)
+  double a = d[b0] - lam, b = es[b0];
+  auto factor = [&](auto rows_c, int j0) {
+    constexpr int R = decltype(rows_c)::value;
+    double sub[R + 1], nd[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      sub[u] = es[j0 + u];
+      nd[u] = d[j0 + u + 1] - lam;
+    }
+    sub[R] = j0 + R + 1 < b1 ? es[j0 + R] : 0.0;
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const bool swap = magnitude(a) < magnitude(sub[u]);
+      const double r = reciprocal(swap ? sub[u] : piv_of(a));
+      const double l = (swap ? a : sub[u]) * r;
+      const long long o = (j0 + u) * nn;
       u0[o] = r;
-      u1[o] = b;
+      u1[o] = swap ? __longlong_as_double(kInvitSwap) : b;
       u2[o] = l;
-      a = nd - l * b;
-      b = nsup - l * c;
-    } else {
-      const double l = a / sub;
-      u0[o] = l;
-      u1[o] = __longlong_as_double(kInvitSwap);
-      const double a2 = b - l * nd;
-      b = c - l * nsup;
-      a = a2;
+      a = swap ? fma(-l, nd[u], b) : fma(-l, b, nd[u]);
+      b = swap ? -l * sub[u + 1] : sub[u + 1];
     }
-    c = 0.0;
-  }
-  const double rlast = 1.0 / piv_of(a);
-  for (int j = b0; j < b1; ++j) x[j] = start_value(t, j);
-  for (int it = 0; it < 3; ++it) {
-    // forward: the same row interchanges and multipliers on the iterate
-    double y = x[b0];
-    for (int j = b0; j + 1 < b1; ++j) {
-      const long long o = j * nn + t;
-      const double yn = x[j + 1];
-      if (__double_as_longlong(u1[o]) != kInvitSwap) {
-        x[j] = y;
-        y = yn - u2[o] * y;
-      } else {
-        x[j] = yn;
-        y = y - u0[o] * yn;
-      }
+  };
+  double inv = 1.0, y = 0.0, xn1 = 0.0, xn2 = 0.0, ss = 0.0;
+  int it = 0;
+  // forward: the same row interchanges and multipliers on the iterate
+  auto forward = [&](auto rows_c, int j0) {
+    constexpr int R = decltype(rows_c)::value;
+    double l[R], f[R], xr[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      l[u] = u2[(j0 + u) * nn];
+      f[u] = u1[(j0 + u) * nn];
+      xr[u] = it == 0 ? start_value(t, j0 + u + 1) : x[(j0 + u + 1) * nn];
     }
-    // back substitution, then normalise
-    double xn1 = y * rlast, xn2 = 0.0;
-    x[b1 - 1] = xn1;
-    double ss = xn1 * xn1;
-    for (int j = b1 - 2; j >= b0; --j) {
-      const long long o = j * nn + t;
-      const double ub = u1[o];
-      double v;
-      if (__double_as_longlong(ub) != kInvitSwap) {
-        v = (x[j] - ub * xn1) * u0[o];
-      } else {
-        const double nd = d[j + 1] - lam, nsup = (j + 2 < b1) ? es[j + 1] : 0.0;
-        v = (x[j] - nd * xn1 - nsup * xn2) / es[j];
-      }
-      x[j] = v;
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const bool swap = __double_as_longlong(f[u]) == kInvitSwap;
+      const double xs = xr[u] * inv;
+      x[(j0 + u) * nn] = swap ? xs : y;
+      y = fma(-l[u], swap ? xs : y, swap ? y : xs);
+    }
+  };
+  auto back = [&](auto rows_c, int j1) {  // rows j1, j1 - 1, ...
+    constexpr int R = decltype(rows_c)::value;
+    double r[R], c1[R], c2[R], xr[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const int j = j1 - u;
+      r[u] = u0[j * nn];
+      c1[u] = u1[j * nn];
+      xr[u] = x[j * nn];
+      c2[u] = j + 2 < b1 ? es[j + 1] : 0.0;
+      const double nd = d[j + 1] - lam;
+      const bool swap = __double_as_longlong(c1[u]) == kInvitSwap;
+      c1[u] = swap ? nd : c1[u];
+      c2[u] = swap ? c2[u] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const double v = fma(-c1[u], xn1, fma(-c2[u], xn2, xr[u])) * r[u];
+      x[(j1 - u) * nn] = v;
       xn2 = xn1;
       xn1 = v;
       ss = fma(v, v, ss);
     }
-    const double inv = 1.0 / sqrt(ss);
-    for (int j = b0; j < b1; ++j) x[j] *= inv;
+  };
+  using Many = std::integral_constant<int, kInvitU>;
+  using One = std::integral_constant<int, 1>;
+  {
+    int j = b0;
+    for (; j + kInvitU < b1; j += kInvitU) factor(Many{}, j);
+    for (; j + 1 < b1; ++j) factor(One{}, j);
   }
+  const double rlast = reciprocal(piv_of(a));
+  for (; it < 3; ++it) {
+    y = it == 0 ? start_value(t, b0) : x[b0 * nn] * inv;
+    int j = b0;
+    for (; j + kInvitU < b1; j += kInvitU) forward(Many{}, j);
+    for (; j + 1 < b1; ++j) forward(One{}, j);
+    xn1 = y * rlast;
+    xn2 = 0.0;
+    x[(b1 - 1) * nn] = xn1;
+    ss = xn1 * xn1;
+    for (j = b1 - 2; j - kInvitU + 1 >= b0; j -= kInvitU) back(Many{}, j);
+    for (; j >= b0; --j) back(One{}, j);
+    inv = 1.0 / sqrt(ss);
+  }
+  auto scale = [&](auto rows_c, int j0) {
+    constexpr int R = decltype(rows_c)::value;
+    double xr[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) xr[u] = x[(j0 + u) * nn];
+#pragma unroll
+    for (int u = 0; u < R; ++u) v_out[j0 + u] = xr[u] * inv;
+  };
+  int j = b0;
+  for (; j + kInvitU <= b1; j += kInvitU) scale(Many{}, j);
+  for (; j < b1; ++j) scale(One{}, j);
 }
 
 // --------------------------------------------------------------------------
@@ -1069,9 +1195,11 @@ int launch_eig_trd(Search* S, const int4* grp, const TrdChunk* chunks, int nchun
   nl += launch_trd_reduce(S, grp, chunks, nchunks, bars, s0, s1, plan, st);
   mark(1);
   k_trd_blocks<<<s1 - s0, kTrdNT, 0, st>>>(S, s0);
-  if (bis_lanes > 1) k_trd_bisect<kTrdBisLanes><<<tm.tbis.total, kTrdTT, 0, st>>>(S, tm.tbis);
-  else k_trd_bisect<1><<<tm.tt.total, kTrdTT, 0, st>>>(S, tm.tt);
-  k_trd_rank<<<s1 - s0, kTrdSortNT, 0, st>>>(S, s0);
+  const auto bisect = bis_lanes == 16 ? k_trd_bisect<16> : bis_lanes == 8 ? k_trd_bisect<8>
+                      : bis_lanes == 4 ? k_trd_bisect<4> : k_trd_bisect<1>;
+  bisect<<<tm.tbis.total, kTrdTT, 0, st>>>(S, tm.tbis);
+  k_trd_rank<<<tm.tt.total, kTrdTT, 0, st>>>(S, tm.tt);
+  k_trd_clusters<<<s1 - s0, kTrdSortNT, 0, st>>>(S, s0);
   mark(2);
   k_trd_invit<<<tm.tt.total, kTrdTT, 0, st>>>(S, tm.tt);
   mark(3);
@@ -1090,7 +1218,7 @@ int launch_eig_trd(Search* S, const int4* grp, const TrdChunk* chunks, int nchun
   nl += launch_bt(S, tm, max_n, st);  // the larger ones
   k_trd_finish<<<s1 - s0, kTrdNT, 0, st>>>(S, s0);
   mark(6);
-  return nl + 6 + 3 * kTrdNsSteps;
+  return nl + 7 + 3 * kTrdNsSteps;
 }
 
 }  // namespace cmaes_gb300
