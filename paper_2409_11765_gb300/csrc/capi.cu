@@ -50,7 +50,9 @@ struct cmaes_s {
   std::vector<int> ask_pending;
   int max_n = 0, max_n_small_jacobi = 0, max_n_cluster_jacobi = 0, max_n_global_jacobi = 0;
   bool any_rotated = false, any_sphere = false;
-  bool any_plain_eig = false;  // a search outside the refined eigensolver route (warm start B^T C B by k_eig_gemm_*)
+  bool any_plain_eig = false;  // a search above every other route (warm start B^T C B by k_eig_gemm_*)
+  bool all_small = true;       // whole generations run in one CTA per search (FP64 handles of small searches)
+  size_t small_smem = 0;
   int max_n_big = 0;           // largest n of the searches whose FP32 Jacobi runs over many CTAs
   // tridiagonal route: largest n, the CTA -> (search, member, group size) table
   // of the cooperative reduction, and one barrier counter per search
@@ -336,7 +338,7 @@ static void enqueue_eig(cmaes_t h, int s0, int s1, cudaStream_t st) {
     count_launch(h, kPhaseEig, sq.total);
   }
   if (h->max_n_small_jacobi > 0) {
-    launch_jacobi_variant(h->dS, s0, s1, true, 0, kJacobiSmallN, h->max_n_small_jacobi, st);
+    launch_small_eig(h->dS, s0, s1, h->max_n_small_jacobi, st);
     count_launch(h, kPhaseEig, s1 - s0);
   }
   if (h->max_n_cluster_jacobi > 0) {
@@ -344,7 +346,7 @@ static void enqueue_eig(cmaes_t h, int s0, int s1, cudaStream_t st) {
     count_launch(h, kPhaseEig, s1 - s0);
   }
   if (h->max_n_global_jacobi > 0) {
-    launch_jacobi_variant(h->dS, s0, s1, false, kJacobiClusterN, 1 << 30, h->max_n_global_jacobi, st);
+    launch_jacobi_global(h->dS, s0, s1, kJacobiClusterN, h->max_n_global_jacobi, st);
     count_launch(h, kPhaseEig, s1 - s0);
   }
   if (h->mixed) {
@@ -590,6 +592,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
   h->count = count;
   h->opt = opt;
   h->mixed = opt.precision != CMAES_FP64;
+  h->all_small = !h->mixed;
   const int esz = tc_elem_bytes(opt.precision);
   DevOptions& d = h->dopt;
   d.max_restarts = opt.max_restarts;
@@ -675,7 +678,9 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     base[s] = total;
     total += b;
     if (n > h->max_n) h->max_n = n;
-    if (!eig_refined_route(n)) h->any_plain_eig = true;
+    if (n > kEigBigMaxN) h->any_plain_eig = true;
+    if (small_generation(n, x.lam_cap)) h->small_smem = std::max(h->small_smem, small_generation_smem(n, x.lam_cap));
+    else h->all_small = false;
     if (x.trd) {
       if (n > h->max_n_trd) h->max_n_trd = n;
     } else {
@@ -705,6 +710,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
       return fail(CMAES_ECUDA);                                                                  \
     }                                                                                            \
   } while (0)
+  small_set_attributes();
   CREATE_TRY(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
   CREATE_TRY(cudaMemsetAsync(h->arena, 0, total, h->stream));
   for (int s = 0; s < count; ++s) {
@@ -1002,9 +1008,20 @@ cmaes_status cmaes_step_batch(cmaes_t h, int generations, void* stream) {
     CUDA_TRY(h, cudaStreamWaitEvent(st, ev, 0));
     CUDA_TRY(h, cudaEventDestroy(ev));
   }
-  for (int g = 0; g < generations; ++g) {
-    cmaes_status r = enqueue_generation(h, 0, h->count, st, true);
+  if (h->all_small && !h->profiling && generations > 0) {
+    // (with profiling on, the phases are timed: the phase kernels)
+    constexpr int kPerLaunch = 1 << 10;  // bounds a launch's time
+    for (int g = 0; g < generations; g += kPerLaunch) {
+      launch_small_generations(h->dS, h->count, h->dopt, std::min(kPerLaunch, generations - g), h->small_smem, st);
+      h->launches += 1;
+    }
+    cmaes_status r = launch_check(h, "small generations");
     if (r != CMAES_OK) return r;
+  } else {
+    for (int g = 0; g < generations; ++g) {
+      cmaes_status r = enqueue_generation(h, 0, h->count, st, true);
+      if (r != CMAES_OK) return r;
+    }
   }
   if (st != h->stream) {
     cudaEvent_t ev;

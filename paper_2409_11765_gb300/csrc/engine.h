@@ -173,13 +173,20 @@ __host__ __device__ inline int jlog_pairs(int n) { return (n + (n & 1)) / 2; }
 __host__ __device__ inline int jlog_steps_cap(int n) {
   return (eig_big_route(n) ? kJ32BigSweeps : kJ32MaxSweeps) * (n + (n & 1) - 1);
 }
-void launch_jacobi_variant(Search* S, int s0, int s1, bool smem, int lo_n, int hi_n, int max_n,
-                           cudaStream_t st);
+void launch_jacobi_global(Search* S, int s0, int s1, int lo_n, int max_n, cudaStream_t st);
+// small searches (kernels_small.cu): the eigendecomposition up to kJacobiSmallN,
+// and whole generations of FP64 searches with n lambda_cap <= kSmallPanel
+// (above it one CTA's FP64 pipe takes longer than the phase kernels' launches)
+constexpr int kSmallPanel = 2048;
+void launch_small_eig(Search* S, int s0, int s1, int max_n, cudaStream_t st);
+bool small_generation(int n, int lam_cap);
+size_t small_generation_smem(int n, int lam_cap);
+void small_set_attributes();
+void launch_small_generations(Search* S, int count, DevOptions o, int gens, size_t smem, cudaStream_t st);
 void launch_jacobi_cluster(Search* S, int s0, int s1, int lo_n, int hi_n, int layout_n, cudaStream_t st);
 void launch_set_bd(Search* S, TileMap tm, cudaStream_t st);
 void launch_set_bd_force(Search* S, TileMap tm, cudaStream_t st);
-int jacobi_smem_max_n();
-int jacobi_smem_bytes(int n, bool smem_mats);
+int jacobi_smem_bytes(int n);
 
 // mixed-precision path (kernels_mixed.cu)
 int tiles_tc_sample(int n, int lam_cap);

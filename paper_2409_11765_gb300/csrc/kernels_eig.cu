@@ -21,8 +21,8 @@
 //      the representative is fixed here so that any two solvers agree: columns
 //      in ascending eigenvalue order (ties by index) and each column's entry of
 //      largest magnitude (first on ties) positive.
-// Small n keeps A and B in shared memory (one CTA per search); larger n runs
-// the same steps on the global-memory copies. For 32 < n <= kEigBigMaxN the
+// Up to n = kJacobiSmallN the same method runs in shared memory
+// (kernels_small.cu); here it runs on the global-memory copies. For 32 < n <= kEigBigMaxN the
 // warm start and most of the work belong to the refined route
 // (kernels_eig_mixed.cu, kernels_eig_big.cu), and the global-memory variant
 // (n > kJacobiClusterN) is its cleanup: it starts from A = X^T C X, nearly
@@ -37,24 +37,14 @@ constexpr double kJacobiTol = 1e-14;
 constexpr int kJacobiMaxSweeps = 40;
 constexpr double kPdFloor = 1e-16;
 
-int jacobi_smem_bytes(int n, bool smem_mats) {
+int jacobi_smem_bytes(int n) {
   const int N = n + (n & 1), P = N / 2;
-  const int mats = smem_mats ? 2 * (N + 1) * N * 8 : 0;
-  return mats + P * (3 * 8 + 4 * 4) + N * (2 * 8 + 4) + 16;
+  return P * (3 * 8 + 4 * 4) + N * (2 * 8 + 4) + 16;
 }
 
-int jacobi_smem_max_n() {
-  int best = 0;
-  for (int n = 2; n <= 256; n += 2)
-    if (jacobi_smem_bytes(n, true) <= 227 * 1024) best = n;
-  return best;
-}
-
-// Searches whose warm start is prepared by the refined route
-// (kernels_eig_mixed.cu) skip the FP64 B^T C B below.
-// searches whose decomposition another route computes (the refined
-// Jacobi route or the tridiagonal route) skip the plain warm start
-__device__ __forceinline__ bool mixed_route(const Search& s) { return eig_refined_route(s) || s.trd; }
+// Searches whose decomposition another route computes (kernels_small.cu, the
+// refined Jacobi route or the tridiagonal route) skip the plain warm start.
+__device__ __forceinline__ bool mixed_route(const Search& s) { return s.n <= kEigBigMaxN; }
 
 // ET = C B (square tiles; only searches whose decomposition is due).
 __global__ void __launch_bounds__(256) k_eig_gemm_CB(Search* S, TileMap tm) {
@@ -111,8 +101,7 @@ __device__ __forceinline__ void rr_pair(int r, int i, int N, int& p, int& q) {
   }
 }
 
-template <bool SMEM>
-__global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_n, int hi_n) {
+__global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_n) {
   extern __shared__ double dsm[];
   __shared__ double shr[32];
   __shared__ long long sh_rot;
@@ -120,23 +109,13 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
   Search& s = S[s0 + blockIdx.x];
   if (s.done || !s.eig_due || s.trd) return;
   const int n = s.n, ldn = s.ldn;
-  if (n <= lo_n || n > hi_n) return;
+  if (n <= lo_n) return;
   const int N = n + (n & 1), P = N / 2;
   const int tid = threadIdx.x;
-  double *A, *V;
-  long long lda;
-  double* rc;
-  if (SMEM) {
-    lda = N + 1;
-    A = dsm;
-    V = dsm + lda * N;
-    rc = V + lda * N;
-  } else {
-    lda = ldn;
-    A = s.EA;
-    V = s.ET;  // free once EA = B^T (C B) is formed; B is rewritten at the end
-    rc = dsm;
-  }
+  const long long lda = ldn;
+  double* A = s.EA;
+  double* V = s.ET;  // free once EA = B^T (C B) is formed; B is rewritten at the end
+  double* rc = dsm;
   double* rsn = rc + P;
   double* rtn = rsn + P;
   double* ev = rtn + P;
@@ -148,18 +127,6 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
   int* al = rk + N;  // the rotating pairs of a step, in no particular order
 
   // symmetrised A = (EA + EA^T) / 2; V = B
-  if (SMEM) {
-    for (int e = tid; e < N * N; e += kJacobiNT) {
-      const int i = e % N, j = e / N;
-      double a = 0.0, v = 0.0;
-      if (i < n && j < n) {
-        a = 0.5 * (s.EA[i + static_cast<long long>(ldn) * j] + s.EA[j + static_cast<long long>(ldn) * i]);
-        v = s.B[i + static_cast<long long>(ldn) * j];
-      }
-      A[i + lda * j] = a;
-      V[i + lda * j] = v;
-    }
-  } else {
     for (long long e = tid; e < static_cast<long long>(n) * n; e += kJacobiNT) {
       const int i = static_cast<int>(e % n), j = static_cast<int>(e / n);
       if (i < j) {
@@ -169,7 +136,6 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
       }
       V[i + lda * j] = s.B[i + static_cast<long long>(ldn) * j];
     }
-  }
   if (tid == 0) {
     sh_rot = 0;
     sh_m = 0;
@@ -219,10 +185,9 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
         // a quiet step: if no off-diagonal entry passes the test any more, the
         // rest of the quiet window would change nothing
         ++quiet;
-        // (on global memory a check reads all of A: at the 64th quiet step and
-        // every 256th after it, so that isolated rotating steps, as in a
+        // (a check reads all of A: at the 64th quiet step and every 256th after it, so that isolated rotating steps, as in a
         // cleanup, do not each cost a pass over the matrix)
-        if (SMEM ? (quiet == 1 || quiet % 16 == 0) : (quiet == 64 || quiet % 256 == 0)) {
+        if (quiet == 64 || quiet % 256 == 0) {
           int pend = 0;
           for (int j = tid >> 5; j < n && !pend; j += kJacobiNT / 32) {
             const double ajj = A[j + lda * j];
@@ -239,7 +204,7 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
       }
       quiet = 0;
       const int m = sh_m;
-      if (!SMEM && 6LL * m * n < static_cast<long long>(P) * P) {
+      if (6LL * m * n < static_cast<long long>(P) * P) {
         // Few rotations (as in a cleanup after the refinement): the m pairs'
         // columns of A, then their rows, then their exact 2 x 2 blocks, then
         // V's columns, O(m n) instead of a pass over every block. Pairs are
@@ -288,60 +253,8 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
         __syncthreads();
         continue;
       }
-      // A <- J^T A J per 2x2 block (P <= Q), mirrored
-      const int nblk = P * (P + 1) / 2;
-      // row-major enumeration of the upper triangle of the P x P block grid:
-      // b = Qi (Qi + 1) / 2 + Pi, Pi <= Qi
-      auto block_of = [](int b, int& Pi, int& Qi) {
-        int bp = static_cast<int>((sqrtf(static_cast<float>(8 * b + 1)) - 1.0f) * 0.5f);
-        while ((bp + 1) * (bp + 2) / 2 <= b) ++bp;
-        while (bp * (bp + 1) / 2 > b) --bp;
-        Pi = b - bp * (bp + 1) / 2;
-        Qi = bp;
-      };
-      if (SMEM) {
-        for (int b = tid; b < nblk; b += kJacobiNT) {
-          int Pi, Qi;
-          block_of(b, Pi, Qi);
-          const int aP = ra[Pi], aQ = ra[Qi];
-          if (!aP && !aQ) continue;
-          const int p1 = rp[Pi], q1 = rq[Pi], p2 = rp[Qi], q2 = rq[Qi];
-          if (Pi == Qi) {
-            const double app = A[p1 + lda * p1], aqq = A[q1 + lda * q1], apq = A[p1 + lda * q1];
-            const double t = rtn[Pi];
-            A[p1 + lda * p1] = app - t * apq;
-            A[q1 + lda * q1] = aqq + t * apq;
-            A[p1 + lda * q1] = 0.0;
-            A[q1 + lda * p1] = 0.0;
-            continue;
-          }
-          const double cP = rc[Pi], sP = rsn[Pi], cQ = rc[Qi], sQ = rsn[Qi];
-          const bool vp1 = p1 < n, vq1 = q1 < n, vp2 = p2 < n, vq2 = q2 < n;
-          const double a = (vp1 && vp2) ? A[p1 + lda * p2] : 0.0;
-          const double bb = (vp1 && vq2) ? A[p1 + lda * q2] : 0.0;
-          const double c = (vq1 && vp2) ? A[q1 + lda * p2] : 0.0;
-          const double d = (vq1 && vq2) ? A[q1 + lda * q2] : 0.0;
-          const double y00 = a * cQ - bb * sQ, y01 = a * sQ + bb * cQ;
-          const double y10 = c * cQ - d * sQ, y11 = c * sQ + d * cQ;
-          const double x00 = cP * y00 - sP * y10, x01 = cP * y01 - sP * y11;
-          const double x10 = sP * y00 + cP * y10, x11 = sP * y01 + cP * y11;
-          if (vp1 && vp2) { A[p1 + lda * p2] = x00; A[p2 + lda * p1] = x00; }
-          if (vp1 && vq2) { A[p1 + lda * q2] = x01; A[q2 + lda * p1] = x01; }
-          if (vq1 && vp2) { A[q1 + lda * p2] = x10; A[p2 + lda * q1] = x10; }
-          if (vq1 && vq2) { A[q1 + lda * q2] = x11; A[q2 + lda * q1] = x11; }
-        }
-        // V <- V J for the active pairs
-        for (long long e = tid; e < static_cast<long long>(P) * n; e += kJacobiNT) {
-          const int pi = static_cast<int>(e / n), row = static_cast<int>(e % n);
-          if (!ra[pi]) continue;
-          const int p = rp[pi], q = rq[pi];
-          const double c = rc[pi], sn = rsn[pi];
-          const double vp = V[row + lda * p], vq = V[row + lda * q];
-          V[row + lda * p] = c * vp - sn * vq;
-          V[row + lda * q] = sn * vp + c * vq;
-        }
-      } else {
-        // On global memory the step is driven by the list of its m rotating
+      {
+        // The step is driven by the list of its m rotating
         // pairs: warp w takes pairs al[w], al[w + NW], ... and its lanes the
         // partner pairs, so only the blocks with a rotating pair are visited
         // (each once: a block of two rotating pairs belongs to the lower
@@ -449,19 +362,12 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
   }
 }
 
-// Each launch covers the whole search range and processes the searches with
-// lo_n < n <= hi_n (A and B in shared memory needs hi_n <= jacobi_smem_max_n()).
-void launch_jacobi_variant(Search* S, int s0, int s1, bool smem, int lo_n, int hi_n, int max_n,
-                           cudaStream_t st) {
+// Covers the whole search range and processes the searches with n > lo_n.
+void launch_jacobi_global(Search* S, int s0, int s1, int lo_n, int max_n, cudaStream_t st) {
   if (s1 <= s0 || max_n <= lo_n) return;
-  const int bytes = jacobi_smem_bytes(max_n, smem);
-  if (smem) {
-    cudaFuncSetAttribute(k_jacobi<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    k_jacobi<true><<<s1 - s0, kJacobiNT, bytes, st>>>(S, s0, lo_n, hi_n);
-  } else {
-    cudaFuncSetAttribute(k_jacobi<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    k_jacobi<false><<<s1 - s0, kJacobiNT, bytes, st>>>(S, s0, lo_n, hi_n);
-  }
+  const int bytes = jacobi_smem_bytes(max_n);
+  cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  k_jacobi<<<s1 - s0, kJacobiNT, bytes, st>>>(S, s0, lo_n);
 }
 
 // BD = B diag(D); force = 1 applies to every search (after set_state).
