@@ -307,7 +307,6 @@ __device__ __forceinline__ bool oz_tile(OzCtx& cx, const unsigned char* __restri
   uint64_t* full = cx.bar;
   uint64_t* empty = cx.bar + 2;
   uint64_t* drain = cx.bar + 4;
-  const uint32_t idesc = tc_idesc<1>(kOzBN);
   __shared__ int sh_fail;
   if (tid == 0) sh_fail = 0;
   auto issue = [&](int c) {
@@ -344,16 +343,23 @@ __device__ __forceinline__ bool oz_tile(OzCtx& cx, const unsigned char* __restri
         const unsigned char* sa = cx.base + b * kOzStage;
         const unsigned char* sb = sa + kOzS * 2 * kOzBlk;
         const bool first = (c == dc * kOzDrain);
+        const uint64_t da0 = tc_sdesc(smem_u32(sa), 128, 512), db0 = tc_sdesc(smem_u32(sb), 128, 512);
 #pragma unroll 1
         for (int ks = 0; ks < 2; ++ks) {
-#pragma unroll 1
+          // the planes of B follow one another as rows (8-row groups 512 bytes
+          // apart), and pair (p, q) adds to bucket p + q: plane p of A times
+          // planes q .. q + 3 of B is one product with N = 256 into four
+          // neighbouring buckets (10 instructions for 28 pairs)
+#pragma unroll
           for (int p = 0; p < kOzS; ++p) {
-            const uint64_t da = tc_sdesc(smem_u32(sa + p * 2 * kOzBlk) + ks * 256, 128, 512);
-#pragma unroll 1
-            for (int q = 0; q + p < kOzS; ++q) {
-              const uint64_t db = tc_sdesc(smem_u32(sb + q * kOzBlk) + ks * 256, 128, 512);
-              const uint32_t acc = (first && ks == 0 && p == 0) ? 0u : 1u;
-              tc_mma<1>(cx.tmem + static_cast<uint32_t>((p + q) * kOzBN), da, db, idesc, acc);
+#pragma unroll
+            for (int q = 0; q + p < kOzS; q += 4) {
+              const int planes = kOzS - p - q < 4 ? kOzS - p - q : 4;
+              // (descriptors hold addresses in 16-byte units in their low bits)
+              const uint64_t da = da0 + static_cast<uint64_t>((p * 2 * kOzBlk + ks * 256) >> 4);
+              const uint64_t db = db0 + static_cast<uint64_t>((q * kOzBlk + ks * 256) >> 4);
+              tc_mma<1>(cx.tmem + static_cast<uint32_t>((p + q) * kOzBN), da, db, tc_idesc<1>(kOzBN * planes),
+                        (first && ks == 0 && p == 0) ? 0u : 1u);
             }
           }
         }
@@ -388,22 +394,30 @@ __device__ __forceinline__ bool oz_tile(OzCtx& cx, const unsigned char* __restri
     tc_fence_after();
     const uint32_t taddr = cx.tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 32 * (warp >> 2);
     // the five heaviest buckets as one 64-bit fixed-point integer (exact), the
-    // lighter ones in FP32 in units of the fifth
-#pragma unroll 1
-    for (int t = 0; t < 5; ++t) {
-      float v[32];
-      tmem_ld32(taddr + t * kOzBN, v);
-      const int sh = 32 - 8 * t;
+    // lighter ones in FP32 in units of the fifth. A bucket of k pairs is below
+    // k 2^21, so neighbours combine in 32 bits before the 64-bit multiply-adds.
+    {
+      float u[32], v[32];
+      tmem_ld32(taddr, u);
+      tmem_ld32(taddr + kOzBN, v);
 #pragma unroll
-      for (int q = 0; q < 32; ++q) W[q] += static_cast<long long>(__float2int_rn(v[q])) << sh;
-    }
-#pragma unroll 1
-    for (int t = 5; t < kOzS; ++t) {
-      float v[32];
-      tmem_ld32(taddr + t * kOzBN, v);
-      const float w = __int_as_float((127 - 8 * (t - 4)) << 23);  // 2^(-8(t-4))
+      for (int q = 0; q < 32; ++q)
+        W[q] += static_cast<long long>((__float2int_rn(u[q]) << 8) + __float2int_rn(v[q])) * (1 << 24);
+      tmem_ld32(taddr + 2 * kOzBN, u);
+      tmem_ld32(taddr + 3 * kOzBN, v);
 #pragma unroll
-      for (int q = 0; q < 32; ++q) L[q] = __fmaf_rn(v[q], w, L[q]);
+      for (int q = 0; q < 32; ++q)
+        W[q] += static_cast<long long>((__float2int_rn(u[q]) << 8) + __float2int_rn(v[q])) * (1 << 8);
+      tmem_ld32(taddr + 4 * kOzBN, u);
+      tmem_ld32(taddr + 5 * kOzBN, v);
+#pragma unroll
+      for (int q = 0; q < 32; ++q) {
+        W[q] += __float2int_rn(u[q]);
+        L[q] = __fmaf_rn(v[q], 0x1p-8f, L[q]);
+      }
+      tmem_ld32(taddr + 6 * kOzBN, u);
+#pragma unroll
+      for (int q = 0; q < 32; ++q) L[q] = __fmaf_rn(u[q], 0x1p-16f, L[q]);
     }
     tc_fence_before();
     __syncthreads();
