@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
           term = rr[i] * rr[i];
         } else {
           const double u = sm_dot(n, g.Q + i, ld, rr);
-          term = obj == 1 ? g.ld_[i] * u * u : u * u - 10.0 * cos((2.0 * 3.141592653589793) * u);
+          term = obj == 1 ? g.ld_[i] * u * u : u * u - 10.0 * cospi(2.0 * u);
         }
         g.U[n * k + i] = term;
       }

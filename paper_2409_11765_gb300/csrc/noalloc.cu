@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) k_noalloc_reduce(int kind, int n, int lam
     for (int i = lane; i < n; i += 32) acc += lamdiag[i] * u[i] * u[i];
   } else {
     const double* u = U + static_cast<long long>(ld) * k;
-    for (int i = lane; i < n; i += 32) acc += u[i] * u[i] - 10.0 * cos((2.0 * 3.141592653589793) * u[i]);
+    for (int i = lane; i < n; i += 32) acc += u[i] * u[i] - 10.0 * cospi(2.0 * u[i]);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
