@@ -53,6 +53,7 @@ struct cmaes_s {
   bool any_plain_eig = false;  // a search above every other route (warm start B^T C B by k_eig_gemm_*)
   bool all_small = true;       // whole generations run in one CTA per search (FP64 handles of small searches)
   size_t small_smem = 0;
+  int max_n_refine = 0;        // largest n <= kEigMixedMaxN on the refined Jacobi route
   int max_n_big = 0;           // largest n of the searches whose FP32 Jacobi runs over many CTAs
   // tridiagonal route: largest n, the CTA -> (search, member, group size) table
   // of the cooperative reduction, and one barrier counter per search
@@ -325,9 +326,9 @@ static void enqueue_eig(cmaes_t h, int s0, int s1, cudaStream_t st) {
   {
     TileMap tfl = h->tiles(TK_FLAT, s0, s1);
     TileMap tsy = h->tiles(TK_FLATSYM, s0, s1);
-    int nl = launch_eig_mixed_head(h->dS, tfl, tsy, s0, s1, h->max_n, st);
+    int nl = launch_eig_mixed_head(h->dS, tfl, tsy, s0, s1, h->max_n_refine, st);
     if (h->max_n_big > 0) nl += enqueue_jacobi32_big(h, s0, s1, st);
-    nl += launch_eig_mixed_tail(h->dS, tfl, tsy, s0, s1, h->max_n, st);
+    nl += launch_eig_mixed_tail(h->dS, tfl, tsy, s0, s1, h->max_n_refine, st);
     h->launches += nl;
     h->phase_launch[kPhaseEig] += nl;
   }
@@ -685,6 +686,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
       if (n > h->max_n_trd) h->max_n_trd = n;
     } else {
       if (eig_big_route(n) && n > h->max_n_big) h->max_n_big = n;
+      if (eig_refined_route(n) && n <= kEigMixedMaxN && n > h->max_n_refine) h->max_n_refine = n;
       int* jm = n <= kJacobiSmallN ? &h->max_n_small_jacobi
                 : n <= kJacobiClusterN ? &h->max_n_cluster_jacobi : &h->max_n_global_jacobi;
       if (n > *jm) *jm = n;
@@ -904,9 +906,9 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
         case TK_TCOBJ: t = h->mixed ? tiles_tc_objective(x.lam_cap) : 0; break;
         case TK_TCCOVP: t = h->mixed ? tiles_tc_sym(x.n) * x.covm_nch : 0; break;
         case TK_TCSYM: t = h->mixed ? 16 * tiles_tc_sym(x.n) : 0; break;  // reduce: 16 blocks per tile
-        case TK_FLAT: t = eig_refined_route(x) ? tiles_flat(x.n) : 0; break;
+        case TK_FLAT: t = eig_big_route(x.n) && !x.trd ? tiles_flat(x.n) : 0; break;
         case TK_REEVAL: t = h->mixed ? tiles_reeval(x.n) : 0; break;
-        case TK_FLATSYM: t = eig_refined_route(x) ? tiles_flat_sym(x.n) : 0; break;
+        case TK_FLATSYM: t = eig_big_route(x.n) && !x.trd ? tiles_flat_sym(x.n) : 0; break;
         case TK_TRD: t = x.trd ? tiles_trd(x.n) : 0; break;
         case TK_TRDBIS: t = x.trd ? tiles_trd_bis(x.n, h->trd_bis_lanes) : 0; break;
         case TK_TRDSQ: t = x.trd ? tiles_trd_sq(x.n) : 0; break;

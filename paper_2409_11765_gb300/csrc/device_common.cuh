@@ -164,26 +164,32 @@ struct GemmSmem {
   int ea[kGBM], eb[kGBN];
 };
 
-// The limbs of x for a scale with biased exponent E (|x| < 2^(E - 1022)).
+// The limbs of x for a scale with biased exponent E (|x| < 2^(E - 1022)): x rounded
+// to 2 H - 1 bits of it, x = (h 2^H + l) 2^(E - 1022 - (2 H - 1)), |h|, |l| <= 2^(H - 1).
+template <int H>
 __device__ __forceinline__ int2 gemm_limbs(double x, int E) {
   const int hi = __double2hiint(x), be = (hi >> 20) & 0x7ff;
   long long m = (static_cast<long long>((hi & 0xfffff) | 0x100000) << 32) | static_cast<unsigned>(__double2loint(x));
-  const int s = E - be - 4;  // >= -4
+  const int s = E - be - (2 * H - 54);
   if (s <= 0) m <<= -s;
   else m = s > 54 ? 0 : (m + (1LL << (s - 1))) >> s;
   if (be == 0) m = 0;
   if (hi < 0) m = -m;
-  const int h = static_cast<int>((m + (1LL << 28)) >> 29);
-  return make_int2(h, static_cast<int>(m - (static_cast<long long>(h) << 29)));
+  const int h = static_cast<int>((m + (1LL << (H - 1))) >> H);
+  return make_int2(h, static_cast<int>(m - (static_cast<long long>(h) << H)));
 }
 
-// s 2^(ea + eb - 2100) for the biased exponents of the two scales.
-__device__ __forceinline__ double gemm_scaled(long long s, int e2) {
+// The value of sum (h h) + sum (h l + l h) / 2^H over two operands of that form
+// whose scales have the biased exponents ea and eb, e2 = ea + eb.
+template <int H>
+__device__ __forceinline__ double gemm_scaled(long long hh, long long mid, int e2) {
+  const long long s = hh + ((mid + (1LL << (H - 1))) >> H);
+  const int e = e2 - 2042 - 2 * H;
   const double d = static_cast<double>(s);
-  const int hi = __double2hiint(d), be = ((hi >> 20) & 0x7ff) + e2 - 2100;
+  const int hi = __double2hiint(d), be = ((hi >> 20) & 0x7ff) + e;
   if (s == 0) return 0.0;
-  if (be <= 0 || be >= 2047) return scalbn(d, e2 - 2100);
-  return __hiloint2double(hi + ((e2 - 2100) << 20), __double2loint(d));
+  if (be <= 0 || be >= 2047) return scalbn(d, e);
+  return __hiloint2double(hi + (e << 20), __double2loint(d));
 }
 
 template <bool A_I_CONTIG, bool B_K_CONTIG, class LA, class LB, class EPI>
@@ -255,8 +261,8 @@ __device__ __forceinline__ void gemm_tile_f64(int M, int N, int K, int i0, int j
     }
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-      sm.As[ak(q)][ai(q)] = gemm_limbs(av[q], sm.ea[ai(q)]);
-      sm.Bs[bk(q)][bj(q)] = gemm_limbs(bv[q], sm.eb[bj(q)]);
+      sm.As[ak(q)][ai(q)] = gemm_limbs<29>(av[q], sm.ea[ai(q)]);
+      sm.Bs[bk(q)][bj(q)] = gemm_limbs<29>(bv[q], sm.eb[bj(q)]);
     }
     __syncthreads();
     long long hh[4][4], mid[4][4];
@@ -285,7 +291,7 @@ __device__ __forceinline__ void gemm_tile_f64(int M, int N, int K, int i0, int j
     for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        acc[r][c] += gemm_scaled(hh[r][c] + ((mid[r][c] + (1LL << 28)) >> 29), sm.ea[tr + 16 * r] + sm.eb[tc + 16 * c]);
+        acc[r][c] += gemm_scaled<29>(hh[r][c], mid[r][c], sm.ea[tr + 16 * r] + sm.eb[tc + 16 * c]);
     __syncthreads();
   }
 #pragma unroll

@@ -41,9 +41,11 @@
 //      alone.
 // Because X^T X is measured and corrected every decomposition, rounding does
 // not accumulate in B from one generation's warm start to the next.
-// Every FP64 product reads its left operand along its leading dimension
-// (each X is also stored transposed) and computes 256 consecutive outputs of
-// the n x n result per CTA, two per lane, over the full K.
+// Up to kEigMixedMaxN the products of steps 1 to 5 are fused into two launches of
+// kernels_eig_refine.cu. The products here serve larger n (handles that ask for the
+// Jacobi route): each reads its left operand along its leading dimension (each X is
+// also stored transposed) and computes 256 consecutive outputs of the n x n result
+// per CTA, two per lane, over the full K.
 #include <cmath>
 #include "device_common.cuh"
 
@@ -53,11 +55,14 @@ constexpr int kE32Max = kEigMixedMaxN;  // FP32 Jacobi keeps A32 in shared memor
 constexpr int kJ32NT = 1024;
 constexpr float kJ32Tol = 1e-6f;
 
-__device__ __forceinline__ bool mixed_route_due(const Search& s) {
-  return !s.done && s.eig_due && eig_refined_route(s);
+// the dense products here
+__device__ __forceinline__ bool big_route_due(const Search& s) {
+  return !s.done && s.eig_due && !s.trd && eig_big_route(s.n);
 }
 // the one-CTA FP32 Jacobi, its log replay and the shared-memory pair rounds
-__device__ __forceinline__ bool small_route_due(const Search& s) { return mixed_route_due(s) && s.n <= kE32Max; }
+__device__ __forceinline__ bool small_route_due(const Search& s) {
+  return !s.done && s.eig_due && eig_refined_route(s) && s.n <= kE32Max;
+}
 
 // ---------------------------------------------------------------------------
 // FP64 products of the refinement: CTA t of a search computes outputs
@@ -185,7 +190,7 @@ __global__ void __launch_bounds__(kFW * 32) k_oa_gemm(Search* S, TileMap tm, int
   int t;
   const int si = find_search(tm, t);
   const Search& s = S[si];
-  if (!mixed_route_due(s)) return;
+  if (!big_route_due(s)) return;
   const int n = s.n;
   const long long L = s.ldn;
   const double* C = s.C;
@@ -309,16 +314,15 @@ __global__ void __launch_bounds__(kFW * 32) k_oa_gemm(Search* S, TileMap tm, int
 // of its corrections stay below 2^-10; otherwise both entries only get the
 // orthogonality half -g_ij / 2. The bound keeps the second-order loss of
 // orthogonality of a step, sum_k |e_ki e_kj| <= n 2^-20, small enough that the
-// second step and the Newton-Schulz step bring X^T X to I within rounding
-// (1.5 (n 2^-20)^4 << eps64 for n <= 160; at larger n only near neighbours in
-// the spectrum reach the bound, and what the refinement leaves goes to the
-// cleanup Jacobi).
+// second step and the Newton-Schulz step bring X^T X to I within rounding (only
+// near neighbours in the spectrum reach the bound, and what the refinement leaves
+// goes to the cleanup Jacobi).
 constexpr double kOaSep = 0x1p-10;
 __global__ void __launch_bounds__(kFW * 32) k_oa_e(Search* S, TileMap tm, int step) {
   int t;
   const int si = find_search(tm, t);
   const Search& s = S[si];
-  if (!mixed_route_due(s)) return;
+  if (!big_route_due(s)) return;
   const int n = s.n;
   const long long L = s.ldn;
   const double* Sm = step == 0 ? s.EG : s.ET;
@@ -340,7 +344,7 @@ __global__ void __launch_bounds__(kFW * 32) k_oa_e(Search* S, TileMap tm, int st
       const double li = lam[i], lj = lam[j];
       const double num = Sm[i + L * j] - lj * gij, num_t = Sm[j + L * i] - li * gij;
       const double den = lj - li, lim = kOaSep * fabs(den);
-      e = (fabs(num) <= lim && fabs(num_t) <= lim) ? num / den : -0.5 * gij;
+      e = (den != 0.0 && fabs(num) <= lim && fabs(num_t) <= lim) ? num / den : -0.5 * gij;
     }
     E[i + L * j] = e;
   }
@@ -1047,58 +1051,60 @@ __global__ void __launch_bounds__(kRoundsNT) k_pair_rounds(Search* S, int s0) {
 int pair_rounds_smem_bytes(int n) { return (n + 1) * n * 8; }
 
 
-int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_n, cudaStream_t st) {
-  if (tflat.total <= 0 || s1 <= s0) return 0;
+// max_small: the largest n <= kE32Max of this route (0: none).
+int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, cudaStream_t st) {
   int nl = 0;
-  k_oa_gemm<<<tflat.total, kFW * 32, 0, st>>>(S, tflat, OA_W0);
-  k_oa_gemm<<<tsym.total, kFW * 32, 0, st>>>(S, tsym, OA_W1);  // symmetric result: upper triangle only
-  nl += 2;
-  if (max_n > kJacobiSmallN) {
-    const int mn = max_n < kE32Max ? max_n : kE32Max;
-    const int bytes = jacobi32_smem_bytes(mn);
+  if (s1 <= s0) return nl;
+  if (tflat.total > 0) {
+    k_oa_gemm<<<tflat.total, kFW * 32, 0, st>>>(S, tflat, OA_W0);
+    k_oa_gemm<<<tsym.total, kFW * 32, 0, st>>>(S, tsym, OA_W1);  // symmetric result: upper triangle only
+    nl += 2;
+  }
+  if (max_small > 0) {
+    launch_eig_refine(S, s0, s1, max_small, 1, st);
+    const int bytes = jacobi32_smem_bytes(max_small);
     cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     k_jacobi32<<<s1 - s0, kJ32NT, bytes, st>>>(S, s0);
-    k_jlog_apply<<<dim3(ceil_div(mn, kLogRows), s1 - s0), kLogRows * 32, 0, st>>>(S, s0);
+    k_jlog_apply<<<dim3(ceil_div(max_small, kLogRows), s1 - s0), kLogRows * 32, 0, st>>>(S, s0);
+    nl += 3;
+  }
+  return nl;
+}
+
+int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, cudaStream_t st) {
+  int nl = 0;
+  if (s1 <= s0) return nl;
+  if (tflat.total > 0) {
+    const int gf = tflat.total, gs = tsym.total;
+    auto flat = [&](int op) {  // products with a general result
+      k_oa_gemm<<<gf, kFW * 32, 0, st>>>(S, tflat, op);
+      ++nl;
+    };
+    auto sym = [&](int op) {   // products with a symmetric result: upper triangle only
+      k_oa_gemm<<<gs, kFW * 32, 0, st>>>(S, tsym, op);
+      ++nl;
+    };
+    flat(OA_X0);
+    for (int step = 0; step < 2; ++step) {
+      flat(step == 0 ? OA_T0 : OA_T1);
+      sym(step == 0 ? OA_SG0 : OA_SG1);
+      k_oa_e<<<gf, kFW * 32, 0, st>>>(S, tflat, step);
+      ++nl;
+      flat(step == 0 ? OA_U0 : OA_U1);
+    }
+    sym(OA_G2);
+    flat(OA_N2);
+    flat(OA_T3);
+    sym(OA_A);
+  }
+  if (max_small > 0) {
+    launch_eig_refine(S, s0, s1, max_small, 0, st);
+    const int rbytes = pair_rounds_smem_bytes(max_small);
+    cudaFuncSetAttribute(k_pair_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, rbytes);
+    k_pair_rounds<<<s1 - s0, kRoundsNT, rbytes, st>>>(S, s0);
     nl += 2;
   }
   return nl;
-}
-
-int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_n, cudaStream_t st) {
-  if (tflat.total <= 0 || s1 <= s0) return 0;
-  int nl = 0;
-  const int gf = tflat.total, gs = tsym.total;
-  auto flat = [&](int op) {  // products with a general result
-    k_oa_gemm<<<gf, kFW * 32, 0, st>>>(S, tflat, op);
-    ++nl;
-  };
-  auto sym = [&](int op) {   // products with a symmetric result: upper triangle only
-    k_oa_gemm<<<gs, kFW * 32, 0, st>>>(S, tsym, op);
-    ++nl;
-  };
-  flat(OA_X0);
-  for (int step = 0; step < 2; ++step) {
-    flat(step == 0 ? OA_T0 : OA_T1);
-    sym(step == 0 ? OA_SG0 : OA_SG1);
-    k_oa_e<<<gf, kFW * 32, 0, st>>>(S, tflat, step);
-    ++nl;
-    flat(step == 0 ? OA_U0 : OA_U1);
-  }
-  sym(OA_G2);
-  flat(OA_N2);
-  flat(OA_T3);
-  sym(OA_A);
-  const int mn = max_n < kE32Max ? max_n : kE32Max;
-  const int rbytes = pair_rounds_smem_bytes(mn);
-  cudaFuncSetAttribute(k_pair_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, rbytes);
-  k_pair_rounds<<<s1 - s0, kRoundsNT, rbytes, st>>>(S, s0);
-  ++nl;
-  return nl;
-}
-
-int launch_eig_mixed(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_n, cudaStream_t st) {
-  return launch_eig_mixed_head(S, tflat, tsym, s0, s1, max_n, st) +
-         launch_eig_mixed_tail(S, tflat, tsym, s0, s1, max_n, st);
 }
 
 }  // namespace cmaes_gb300
