@@ -47,12 +47,12 @@
 // also stored transposed) and computes 256 consecutive outputs of the n x n result
 // per CTA, two per lane, over the full K.
 #include <cmath>
+#include <type_traits>
 #include "device_common.cuh"
 
 namespace cmaes_gb300 {
 
 constexpr int kE32Max = kEigMixedMaxN;  // FP32 Jacobi keeps A32 in shared memory
-constexpr int kJ32NT = 1024;
 constexpr float kJ32Tol = 1e-6f;
 
 // the dense products here
@@ -395,20 +395,32 @@ __global__ void __launch_bounds__(kFW * 32) k_oa_e(Search* S, TileMap tm, int st
 // log on the rows of V32 = I across the GPU.
 constexpr float kJ32Tol2 = kJ32Tol * kJ32Tol;
 __device__ __forceinline__ bool j32_rotates(float app, float aqq, float apq, float floor_abs) {
-  return fabsf(apq) > floor_abs && apq * apq > kJ32Tol2 * fabsf(app * aqq);
+  return (fabsf(apq) > floor_abs) & (apq * apq > fmaxf(kJ32Tol2 * fabsf(app * aqq), 0x1p-126f));
 }
 
-// (c, s, t) of the rotation that annihilates a_pq (a_pq passed j32_rotates,
-// so a_pq^2 > 0 and the root's argument is positive)
+// Approximations of 1 / sqrt(x) and 1 / x for normal x.
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// (c, s, t) of the rotation that annihilates a_pq (a_pq passed j32_rotates, so
+// a_pq^2 and with it the root's argument are normal; otherwise of no meaning)
 __device__ __forceinline__ void j32_rotation(float app, float aqq, float apq, float& c, float& s, float& t) {
   const float d = aqq - app;
   const float x = fmaf(d, d, 4.f * apq * apq);
-  const float h = x * rsqrtf(x);  // sqrt(d^2 + 4 a_pq^2)
-  const float mag = __fdividef(2.f * fabsf(apq), fabsf(d) + h);
+  const float h = x * rsqrt_approx(x);  // sqrt(d^2 + 4 a_pq^2)
+  const float mag = 2.f * fabsf(apq) * rcp_approx(fabsf(d) + h);
   // sign(theta), with theta = +-0 counted as positive
-  t = (d == 0.f || ((d > 0.f) == (apq > 0.f))) ? mag : -mag;
+  t = (d == 0.f) | ((d > 0.f) == (apq > 0.f)) ? mag : -mag;
   const float u = fmaf(t, t, 1.f);
-  float y = rsqrtf(u);
+  float y = rsqrt_approx(u);
   y = y * fmaf(-0.5f * u * y, y, 1.5f);  // Newton step for 1 / sqrt(u)
   c = y;
   s = t * y;
@@ -425,33 +437,75 @@ __device__ __forceinline__ void ring_next(int K, int x, int P, int& Kn, int& xn)
   }
 }
 
-// offset (plane * P^2 + slot) of the entry between positions (K, x), (L, y)
-__device__ __forceinline__ int ring_offset(int K, int x, int L, int y, int P) {
-  const int PP = P * P;
-  if (K < L) return (2 * x + y) * PP + K * P + L;
-  if (K > L) return (2 * y + x) * PP + L * P + K;
-  return (x == y ? 3 * x : 1) * PP + K * P + K;
+// offset (plane * PS + slot) of the entry between positions (K, x), (L, y); RS is
+// the row stride (even, so that diagonals K + const fall on different banks)
+__device__ __forceinline__ int ring_offset(int K, int x, int L, int y, int RS, int PS) {
+  if (K < L) return (2 * x + y) * PS + K * RS + L;
+  if (K > L) return (2 * y + x) * PS + L * RS + K;
+  return (x == y ? 3 * x : 1) * PS + K * RS + K;
 }
 
-// off-diagonal 2 x 2 blocks per thread at the largest size: one for every
-// thread, then the rest of P (P - 1) / 2 over the kJ32NT - P threads that
-// form no rotation
-constexpr int kJ32Blocks =
-    1 + ((kE32Max / 2) * (kE32Max / 2 - 1) / 2 - kJ32NT + (kJ32NT - kE32Max / 2) - 1) / (kJ32NT - kE32Max / 2);
+// v 2^-ex in FP32, rounded to nearest even, by the bits (a conversion takes the FP64
+// pipe); below 2^-126 it is zero, which is far under the rotation floor.
+__device__ __forceinline__ float j32_entry(double v, int ex) {
+  const int hi = __double2hiint(v), be = (hi >> 20) & 0x7ff, e = be - 896 - ex;
+  const unsigned lo = static_cast<unsigned>(__double2loint(v)), rest = lo & 0x1fffffffu;
+  unsigned m = (static_cast<unsigned>(hi & 0xfffff) << 3) | (lo >> 29);
+  m += rest > 0x10000000u || (rest == 0x10000000u && (m & 1u));
+  unsigned f = (static_cast<unsigned>(e) << 23) + m;
+  if (e <= 0 || be == 0) f = 0u;
+  if (be == 0x7ff) f = 0x7fc00000u;
+  return __uint_as_float(f | (static_cast<unsigned>(hi) & 0x80000000u));
+}
 
-__global__ void __launch_bounds__(kJ32NT, 1) k_jacobi32(Search* S, int s0) {
+// The block (K, L) of entry j of the list of blocks that hold no next-step pivot:
+// the rows L = K + 3 .. P - 1 of K = 0 .. P - 4, then (K, K + 1) for K = 1 .. P - 3.
+__device__ __forceinline__ void j32_block(int j, int P, int& K, int& L) {
+  const int T = (P - 3) * (P - 2) / 2;
+  if (j >= T) {
+    K = 1 + j - T;
+    L = K + 1;
+    return;
+  }
+  const int m = T - 1 - j;  // from the end: the last row has one block
+  int q = static_cast<int>((sqrtf(static_cast<float>(8 * m + 1)) - 1.0f) * 0.5f);
+  while ((q + 1) * (q + 2) / 2 <= m) ++q;
+  while (q * (q + 1) / 2 > m) --q;
+  K = P - 4 - q;
+  L = P - 1 - (m - q * (q + 1) / 2);
+}
+
+// NT threads serve P <= PM pairs: the first P threads form the rotations and own the
+// block of their next pivot, each other thread owns up to NB of the other blocks.
+// What bounds a step is the chain of those rotations (records and block from shared
+// memory, the update, three approximations of a root or a quotient, the record back,
+// the barrier: ~500 clocks) and, from n ~ 64, the shared-memory passes of the other
+// blocks, which the chain's own accesses queue behind (10 of 4 bytes per block: ~500
+// clocks at n = 100). So the rotation has no branches, every address of a step is
+// fixed (the step is written out for both buffers), a size takes no more warps than
+// it has blocks for and two blocks per thread at most where that fits, one after the
+// other (three loaded together hold the chain up by 40 clocks), and the starting
+// matrix is converted by integer operations. Measured with 1024 threads for every n,
+// a loop over up to four blocks, branches and conversions on the FP64 pipe -> here:
+// a step 1540 -> 584 clocks at n = 40, 2020 -> ~1250 at n = 100; the setup 35k -> 12k and
+// 58k -> 19k clocks.
+template <int NT, int NB, int PM>
+__global__ void __launch_bounds__(NT, 1) k_jacobi32(Search* S, int s0) {
+  constexpr int RM = (PM + 1) & ~1, PS = RM * RM;  // plane stride
+  static_assert((NT - PM) * NB >= PM * (PM - 3) / 2, "block list");
   extern __shared__ __align__(16) float fsm[];
   __shared__ float sh_amax;
+  __shared__ double sh_c;
+  __shared__ int sh_ex;
   Search& s = S[s0 + blockIdx.x];
   if (!small_route_due(s)) return;
-  constexpr int NW = kJ32NT / 32;
-  const int n = s.n, N = n + (n & 1), P = N / 2, tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int PP = P * P;
-  const int nblk = P * (P - 1) / 2;
+  constexpr int NW = NT / 32;
+  const int n = __shfl_sync(0xffffffffu, s.n, 0);
+  const int N = n + (n & 1), P = N / 2, M = N - 1, RS = (P + 1) & ~1, tid = threadIdx.x;
+  const int lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const bool pad = n & 1;  // pair 0 holds the padding element and never rotates
-  float2* rec = reinterpret_cast<float2*>(fsm);  // 2 x P step records (c, s)
-  float* buf = fsm + 4 * P;                       // 2 buffers x 4 planes x P^2
+  float* buf = fsm;                                      // 2 buffers x 4 planes x PS
+  float2* rec = reinterpret_cast<float2*>(fsm + 8 * PS);  // 2 x PM step records (c, s)
   // A32 = 2^-k (B^T C B - c I) rounded to FP32, with c the mean eigenvalue
   // (the trace over n, in FP64) and 2^k the power of two at or above
   // max a_ii. B^T C B is positive semi-definite, so |a_ij| <= max a_ii and
@@ -465,231 +519,244 @@ __global__ void __launch_bounds__(kJ32NT, 1) k_jacobi32(Search* S, int s0) {
   // 1 <= e <= P - 1 at (e, a), P <= e <= N - 2 at (N - 1 - e, b).
   const long long L = s.ldn;
   const double* A64 = s.EH;
-  double tr = 0.0, dmax = 0.0;
-  for (int i = tid; i < n; i += kJ32NT) {
-    const double d = A64[i + L * i];
-    tr += d;
-    dmax = fmax(dmax, fabs(d));
+  constexpr int kRow = (2 * PM + 31) / 32;
+  if (warp == 0) {
+    double tr = 0.0, dmax = 0.0;
+#pragma unroll
+    for (int u = 0; u < kRow; ++u) {
+      const int i = lane + 32 * u;
+      const double d = i < n ? A64[i + L * i] : 0.0;
+      tr += d;
+      dmax = fmax(dmax, fabs(d));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      tr += __shfl_xor_sync(0xffffffffu, tr, o);
+      dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    }
+    if (lane == 0) {
+      int ex = 0;
+      if (dmax > 0.0) frexp(dmax, &ex);  // dmax = m 2^ex, m in [0.5, 1)
+      sh_ex = ex;
+      sh_c = tr / n;
+    }
   }
-  __shared__ double shs[kJ32NT / 32];
-  const double c = block_sum<kJ32NT>(tr, shs) / n;
-  dmax = block_max<kJ32NT>(dmax, shs);
-  int ex = 0;
-  if (dmax > 0.0) frexp(dmax, &ex);  // dmax = m 2^ex, m in [0.5, 1)
-  const double scale = ldexp(1.0, -ex);
-  const int M = N - 1;
+  for (int e = tid; e < 8 * PS; e += NT) buf[e] = 0.f;  // (the padding's entries stay zero)
+  __syncthreads();
+  const int ex = sh_ex;
+  const double c = sh_c;
   auto pos0 = [=](int e, int& K, int& x) {
     if (e == 0) { K = 0; x = 0; }
     else if (e == M) { K = 0; x = 1; }
     else if (e <= P - 1) { K = e; x = 0; }
     else { K = M - e; x = 1; }
   };
-  constexpr int kRow = (kE32Max + 31) / 32;
-  for (int j = warp; j < N; j += NW) {
+  for (int j = warp; j < n; j += NW) {
     double v[kRow];
 #pragma unroll
     for (int u = 0; u < kRow; ++u) {
       const int i = lane + 32 * u;
-      v[u] = (i < n && j < n) ? A64[i + L * j] : 0.0;
+      v[u] = i < n ? A64[i + L * j] : 0.0;
+      if (i == j) v[u] -= c;
     }
     int Kj, xj;
     pos0(j, Kj, xj);
 #pragma unroll
     for (int u = 0; u < kRow; ++u) {
       const int i = lane + 32 * u;
-      if (i >= N) continue;
+      if (i >= n) continue;
       int Ki, xi;
       pos0(i, Ki, xi);
       // each unordered entry once: the upper block, or the diagonal block's a_aa, a_ab, a_bb
-      if (Ki < Kj || (Ki == Kj && xi <= xj))
-        buf[ring_offset(Ki, xi, Kj, xj, P)] =
-            (i < n && j < n) ? static_cast<float>((v[u] - (i == j ? c : 0.0)) * scale) : 0.f;
+      if (Ki < Kj || (Ki == Kj && xi <= xj)) buf[ring_offset(Ki, xi, Kj, xj, RS, PS)] = j32_entry(v[u], ex);
     }
   }
   __syncthreads();
   if (warp == 0) {
     float m = 0.f;
-    for (int K = lane; K < P; K += 32) m = fmaxf(m, fmaxf(fabsf(buf[K * P + K]), fabsf(buf[3 * PP + K * P + K])));
+    for (int K = lane; K < P; K += 32) m = fmaxf(m, fmaxf(fabsf(buf[K * RS + K]), fabsf(buf[3 * PS + K * RS + K])));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) sh_amax = m;
   }
-  __syncthreads();
-  // Each thread owns the same off-diagonal blocks (K, L), K < L, in every
-  // step: entry tid of a list, and entries kJ32NT + (kJ32NT - P)(u - 1) +
-  // tid - P for u >= 1 when tid >= P. The list starts with the P role blocks
-  // (block k holds the pivot of next-step pair k), then the others row by row
-  // (K ascending, L ascending). bKL: K | L << 8 (-1: none); bdst: the four
-  // entries' next offsets, (a, a) | (a, b) << 16 and (b, a) | (b, b) << 16.
-  int bKL[kJ32Blocks], bdst[kJ32Blocks][2];
+  // Each thread owns the same off-diagonal blocks (K, L), K < L, in every step:
+  // offset of the block, of the two records, and of its four entries' next places.
+  // Thread k < P owns the one block that holds the pivot of next-step pair k.
+  // With many blocks per thread the registers only hold packed offsets.
+  constexpr bool kPack = NT > 768;
+  int bo[NB], bK[kPack ? 1 : NB], bL[kPack ? 1 : NB], bd[NB][kPack ? 2 : 4];
 #pragma unroll
-  for (int u = 0; u < kJ32Blocks; ++u) {
-    const int k = u == 0 ? tid : (tid >= P ? kJ32NT + (kJ32NT - P) * (u - 1) + tid - P : nblk);
-    int K = 0, Lb = 0;
-    if (k < P) {
-      if (k == 0) { K = 0; Lb = 1; }
-      else if (k == 1) { K = 0; Lb = 2; }
-      else if (k == P - 1) { K = P - 2; Lb = P - 1; }
-      else { K = k - 1; Lb = k + 1; }
-    } else if (k < nblk) {
-      // the (k - P)-th block that holds no pivot, row by row: row K has
-      // P - 1 - K blocks, of which (K, K + 2), (0, 1) and (P - 2, P - 1) hold one
-      int j = k - P;
-      for (;;) {
-        const int cnt = (P - 1 - K) - (K + 2 <= P - 1) - (K == 0) - (K == P - 2);
-        if (j < cnt) break;
-        j -= cnt;
-        ++K;
+  for (int u = 0; u < NB; ++u) {
+    int K = -1, Lb = 0;
+    if (tid < P) {
+      if (u == 0) {
+        K = tid == 0 || tid == 1 ? 0 : (tid == P - 1 ? P - 2 : tid - 1);
+        Lb = tid == 0 ? 1 : (tid == 1 ? 2 : (tid == P - 1 ? P - 1 : tid + 1));
       }
-      for (Lb = K + 1;; ++Lb) {
-        const bool role = (K == 0 && Lb == 1) || (Lb == K + 2) || (K == P - 2 && Lb == P - 1);
-        if (role) continue;
-        if (j == 0) break;
-        --j;
-      }
+    } else {
+      const int j = (NT - P) * u + tid - P;
+      if (j < P * (P - 3) / 2) j32_block(j, P, K, Lb);
     }
-    bKL[u] = k < nblk ? K | (Lb << 8) : -1;
+    bo[u] = K < 0 ? -1 : kPack ? K | Lb << 8 : K * RS + Lb;
+    if (!kPack) {
+      bK[kPack ? 0 : u] = K;
+      bL[kPack ? 0 : u] = Lb;
+    }
     int d[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       int Kn, xn, Ln, yn;
       ring_next(K, e >> 1, P, Kn, xn);
       ring_next(Lb, e & 1, P, Ln, yn);
-      d[e] = ring_offset(Kn, xn, Ln, yn, P);
+      d[e] = ring_offset(Kn, xn, Ln, yn, RS, PS);
+      if (!kPack) bd[u][kPack ? 0 : e] = d[e];
     }
-    bdst[u][0] = d[0] | (d[1] << 16);
-    bdst[u][1] = d[2] | (d[3] << 16);
+    if (kPack) {
+      bd[u][0] = d[0] | d[1] << 16;
+      bd[u][1] = d[2] | d[3] << 16;
+    }
   }
-  // role of thread tid < P (its block is the list's entry tid): the entry
-  // holding the pivot of next pair k = tid (0: (a, a), 2: (b, a), 3: (b, b)),
-  // the current offsets of that pair's two diagonal entries, and the next
-  // offset of the current diagonal block k's off-diagonal entry
+  // role of thread tid < P: the entry holding the pivot of next pair k = tid
+  // (0: (a, a), 2: (b, a), 3: (b, b)), the current offsets of that pair's two
+  // diagonal entries, and the next offset of the current diagonal block k's
+  // off-diagonal entry
   int r_ent = 0, r_srcA = 0, r_srcB = 0, r_move = 0;
   if (tid < P) {
     const int k = tid;
     r_ent = k == 1 ? 0 : (k == P - 1 ? 3 : 2);
-    r_srcA = k <= P - 2 ? ring_offset(k + 1, 0, k + 1, 0, P) : ring_offset(P - 1, 1, P - 1, 1, P);
-    r_srcB = k >= 2 ? ring_offset(k - 1, 1, k - 1, 1, P) : ring_offset(0, k == 1 ? 0 : 1, 0, k == 1 ? 0 : 1, P);
+    r_srcA = k <= P - 2 ? ring_offset(k + 1, 0, k + 1, 0, RS, PS) : ring_offset(P - 1, 1, P - 1, 1, RS, PS);
+    r_srcB = k >= 2 ? ring_offset(k - 1, 1, k - 1, 1, RS, PS)
+                    : ring_offset(0, k == 1 ? 0 : 1, 0, k == 1 ? 0 : 1, RS, PS);
     int Ka, xa, Kb, xb;
     ring_next(k, 0, P, Ka, xa);
     ring_next(k, 1, P, Kb, xb);
-    r_move = ring_offset(Ka, xa, Kb, xb, P);
+    r_move = ring_offset(Ka, xa, Kb, xb, RS, PS);
   }
+  __syncthreads();
   // below 16 eps32 max|a_ii| an off-diagonal entry is FP32 rounding noise
   const float floor_abs = 16.f * 1.1920929e-7f * sh_amax;
   const int cap = jlog_steps_cap(n);
-  float2* jlog = reinterpret_cast<float2*>(s.jlog);
+  float2* jlog = reinterpret_cast<float2*>(s.jlog) + tid;  // the next logged step's record of pair tid
+  int* jlog_r = s.jlog_r;
   int logged = 0;
-  // The rotation of pair k of step rn from its 2 x 2 diagonal block: the
+  // The rotation of pair tid of step rn from its 2 x 2 diagonal block: the
   // new diagonal entries, the step record, and the log entry (at the index
   // the step gets if it rotates anything: later rotating steps overwrite the
   // entries of a quiet one). Returns whether it rotates; apq becomes zero then.
-  auto rotate_pair = [&](int rn, int k, float& app, float& aqq, float& apq, float2* recn) -> int {
-    float cr = 1.f, sr = 0.f;
-    int act = 0;
-    if (!(pad && k == 0) && j32_rotates(app, aqq, apq, floor_abs)) {
-      float tn;
-      j32_rotation(app, aqq, apq, cr, sr, tn);
-      app -= tn * apq;
-      aqq += tn * apq;
-      apq = 0.f;
-      act = 1;
-    }
-    recn[k] = make_float2(cr, sr);
+  const bool never = pad && tid == 0;
+  auto rotate_pair = [&](int rn, float& app, float& aqq, float& apq, float2* recn) -> int {
+    float cr, sr, tn;
+    const bool act = !never && j32_rotates(app, aqq, apq, floor_abs);
+    j32_rotation(app, aqq, apq, cr, sr, tn);
+    cr = act ? cr : 1.f;
+    sr = act ? sr : 0.f;
+    app = act ? app - tn * apq : app;
+    aqq = act ? aqq + tn * apq : aqq;
+    apq = act ? 0.f : apq;
+    recn[tid] = make_float2(cr, sr);
     if (logged < cap) {
-      jlog[static_cast<size_t>(logged) * P + k] = make_float2(cr, sr);
-      if (k == 0) s.jlog_r[logged] = rn;
+      *jlog = make_float2(cr, sr);
+      if (tid == 0) jlog_r[logged] = rn;
     }
     return act;
   };
   // step 0: the rotations from the diagonal blocks of buffer 0
   int act0 = 0;
   if (tid < P) {
-    float app = buf[tid * P + tid], aqq = buf[3 * PP + tid * P + tid], apq = buf[PP + tid * P + tid];
-    act0 = rotate_pair(0, tid, app, aqq, apq, rec);
-    buf[tid * P + tid] = app;
-    buf[3 * PP + tid * P + tid] = aqq;
-    buf[PP + tid * P + tid] = apq;
+    const int o = tid * RS + tid;
+    float app = buf[o], aqq = buf[3 * PS + o], apq = buf[PS + o];
+    act0 = rotate_pair(0, app, aqq, apq, rec);
+    buf[o] = app;
+    buf[3 * PS + o] = aqq;
+    buf[PS + o] = apq;
   }
-  int nact = __syncthreads_count(act0);
-  int cur = 0, r = 0, sweep = 0, quiet = 0;
+  int nact = __syncthreads_or(act0);
+  int r = 0, sweep = 0, quiet = 0;
   bool converged = false;
-  while (true) {
-    // step r: its rotations are in the records of buffer cur (diagonal blocks applied)
-    const float* bc = buf + cur * 4 * PP;
+  // Step r, its rotations in the records of buffer CUR (diagonal blocks applied).
+  // Returns false at the end.
+  auto step = [&](auto CUR) -> bool {
+    constexpr int cur = decltype(CUR)::value;
+    const float* bc = buf + cur * 4 * PS;
     if (nact == 0) {
       // a quiet step: if no off-diagonal entry passes the test any more, the
       // remaining quiet steps of the window would change nothing
       ++quiet;
       if (quiet == 1 || (quiet & 15) == 0) {
         int pend = 0;
-        for (int e = tid; e < PP && !pend; e += kJ32NT) {
-          const int K = e / P, Lb = e % P;
+        for (int e = tid; e < P * P && !pend; e += NT) {
+          const int K = e / P, Lb = e % P, o = K * RS + Lb;
           if (K > Lb) continue;
-          const float aK = bc[K * P + K], bK = bc[3 * PP + K * P + K];
+          const float aK = bc[K * RS + K], bK_ = bc[3 * PS + K * RS + K];
           if (K == Lb) {
-            pend |= j32_rotates(aK, bK, bc[PP + e], floor_abs);
+            pend |= j32_rotates(aK, bK_, bc[PS + o], floor_abs);
           } else {
-            const float aL = bc[Lb * P + Lb], bL = bc[3 * PP + Lb * P + Lb];
-            pend |= j32_rotates(aK, aL, bc[e], floor_abs) | j32_rotates(aK, bL, bc[PP + e], floor_abs) |
-                    j32_rotates(bK, aL, bc[2 * PP + e], floor_abs) | j32_rotates(bK, bL, bc[3 * PP + e], floor_abs);
+            const float aL = bc[Lb * RS + Lb], bL_ = bc[3 * PS + Lb * RS + Lb];
+            pend |= j32_rotates(aK, aL, bc[o], floor_abs) | j32_rotates(aK, bL_, bc[PS + o], floor_abs) |
+                    j32_rotates(bK_, aL, bc[2 * PS + o], floor_abs) | j32_rotates(bK_, bL_, bc[3 * PS + o], floor_abs);
           }
         }
         if (!__syncthreads_or(pend)) quiet = M;
       }
       if (quiet >= M) {
         converged = true;
-        break;  // uniform: the counts come from block barriers
+        return false;  // uniform: the counts come from block barriers
       }
     } else {
       quiet = 0;
       ++logged;  // its log entries were written with its rotations
+      jlog += P;
     }
     const int rn = (r + 1 == M) ? 0 : r + 1;
-    if (rn == 0 && ++sweep == kJ32MaxSweeps) break;
+    if (rn == 0 && ++sweep == kJ32MaxSweeps) return false;
     // A <- J^T A J on the thread's blocks, each entry written to its position
     // of step rn in the other buffer; the role threads form the rotations of
     // step rn and write the next diagonal blocks
-    float* bn = buf + (cur ^ 1) * 4 * PP;
-    const float2* rc = rec + cur * P;
-    float2* rnx = rec + (cur ^ 1) * P;
+    float* bn = buf + (cur ^ 1) * 4 * PS;
+    const float2* rc = rec + cur * PM;
     int act = 0;
+    float x[NB][4];
+    float2 gK[NB], gL[NB];
+    auto load = [&](int u) {
+      const int K = kPack ? bo[u] & 0xff : bK[kPack ? 0 : u], Lb = kPack ? bo[u] >> 8 : bL[kPack ? 0 : u];
+      const int o = kPack ? K * RS + Lb : bo[u];
 #pragma unroll
-    for (int u = 0; u < kJ32Blocks; ++u) {
-      if (bKL[u] < 0) continue;
-      const int K = bKL[u] & 0xff, Lb = bKL[u] >> 8;
-      const int o = K * P + Lb;
-      float x[4] = {bc[o], bc[PP + o], bc[2 * PP + o], bc[3 * PP + o]};
-      const float2 gK = rc[K], gL = rc[Lb];
-      if (gK.y != 0.f || gL.y != 0.f) {
-        const float cP = gK.x, sP = gK.y, cQ = gL.x, sQ = gL.y;
-        const float y00 = x[0] * cQ - x[1] * sQ, y01 = x[0] * sQ + x[1] * cQ;
-        const float y10 = x[2] * cQ - x[3] * sQ, y11 = x[2] * sQ + x[3] * cQ;
-        x[0] = cP * y00 - sP * y10;
-        x[1] = cP * y01 - sP * y11;
-        x[2] = sP * y00 + cP * y10;
-        x[3] = sP * y01 + cP * y11;
-      }
+      for (int e = 0; e < 4; ++e) x[u][e] = bc[e * PS + o];
+      gK[u] = rc[K];
+      gL[u] = rc[Lb];
+    };
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      if (bo[u] < 0) continue;
+      load(u);
+      const float cP = gK[u].x, sP = gK[u].y, cQ = gL[u].x, sQ = gL[u].y;
+      const float y00 = x[u][0] * cQ - x[u][1] * sQ, y01 = x[u][0] * sQ + x[u][1] * cQ;
+      const float y10 = x[u][2] * cQ - x[u][3] * sQ, y11 = x[u][2] * sQ + x[u][3] * cQ;
+      x[u][0] = cP * y00 - sP * y10;
+      x[u][1] = cP * y01 - sP * y11;
+      x[u][2] = sP * y00 + cP * y10;
+      x[u][3] = sP * y01 + cP * y11;
       if (u == 0 && tid < P) {
-        const int k = tid;
         float app = bc[r_srcA], aqq = bc[r_srcB];
-        float apq = r_ent == 0 ? x[0] : (r_ent == 2 ? x[2] : x[3]);
-        act = rotate_pair(rn, k, app, aqq, apq, rnx);
-        if (r_ent == 0) x[0] = apq;
-        else if (r_ent == 2) x[2] = apq;
-        else x[3] = apq;
-        bn[k * P + k] = app;
-        bn[3 * PP + k * P + k] = aqq;
-        bn[r_move] = bc[PP + k * P + k];  // the current diagonal block's a_ab moves on
+        const float moved = bc[PS + tid * RS + tid];  // the current diagonal block's a_ab moves on
+        float apq = r_ent == 0 ? x[0][0] : (r_ent == 2 ? x[0][2] : x[0][3]);
+        act = rotate_pair(rn, app, aqq, apq, rec + (cur ^ 1) * PM);
+        x[0][0] = r_ent == 0 ? apq : x[0][0];
+        x[0][2] = r_ent == 2 ? apq : x[0][2];
+        x[0][3] = r_ent == 3 ? apq : x[0][3];
+        bn[tid * RS + tid] = app;
+        bn[3 * PS + tid * RS + tid] = aqq;
+        bn[r_move] = moved;
       }
-      bn[bdst[u][0] & 0xffff] = x[0];
-      bn[bdst[u][0] >> 16] = x[1];
-      bn[bdst[u][1] & 0xffff] = x[2];
-      bn[bdst[u][1] >> 16] = x[3];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        bn[kPack ? (e & 1 ? bd[u][e >> 1] >> 16 : bd[u][e >> 1] & 0xffff) : bd[u][kPack ? 0 : e]] = x[u][e];
     }
-    nact = __syncthreads_count(act);
-    cur ^= 1;
+    nact = __syncthreads_or(act);
     r = rn;
+    return true;
+  };
+  while (step(std::integral_constant<int, 0>{}) && step(std::integral_constant<int, 1>{})) {
   }
   if (tid == 0) {
     s.jlog_steps = logged;
@@ -697,9 +764,28 @@ __global__ void __launch_bounds__(kJ32NT, 1) k_jacobi32(Search* S, int s0) {
   }
 }
 
-int jacobi32_smem_bytes(int n) {
-  const int N = n + (n & 1), P = N / 2;
-  return 2 * P * 8 + 2 * 4 * P * P * 4;
+static size_t jacobi32_smem_bytes(int pm) {
+  const int rm = (pm + 1) & ~1;
+  return static_cast<size_t>(8) * rm * rm * 4 + 2 * pm * 8;
+}
+
+template <int NT, int NB, int PM>
+static void launch_jacobi32_as(Search* S, int s0, int s1, cudaStream_t st) {
+  const int bytes = static_cast<int>(jacobi32_smem_bytes(PM));
+  cudaFuncSetAttribute(k_jacobi32<NT, NB, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  k_jacobi32<NT, NB, PM><<<s1 - s0, NT, bytes, st>>>(S, s0);
+}
+
+// The fewest threads whose blocks hide behind the rotations, by the largest n of the
+// handle: up to n = 44, 72, 104, 126 and kE32Max. (n = 100, ten searches, the whole
+// decomposition: 256 threads 547 us, 512 521, 768 509, 1024 530.)
+static void launch_jacobi32(Search* S, int s0, int s1, int max_n, cudaStream_t st) {
+  const int P = (max_n + 1) / 2;
+  if (P <= 22) launch_jacobi32_as<256, 1, 22>(S, s0, s1, st);
+  else if (P <= 36) launch_jacobi32_as<384, 2, 36>(S, s0, s1, st);
+  else if (P <= 52) launch_jacobi32_as<768, 2, 52>(S, s0, s1, st);
+  else if (P <= 63) launch_jacobi32_as<1024, 2, 63>(S, s0, s1, st);
+  else launch_jacobi32_as<1024, 4, kE32Max / 2>(S, s0, s1, st);
 }
 
 // V32 from the rotation log: row i of V32 = e_i^T J_1 J_2 ... J_T, and the
@@ -736,10 +822,15 @@ __device__ __forceinline__ void rr_pair(int r, int pi, int M, int& p, int& q) {
 template <int PL>  // slots per lane: P <= 32 PL
 __device__ __forceinline__ void jlog_replay(const Search& s, float* v, float2 (*lcs)[kLogChunkMax],
                                             int (*lr)[kLogStepsMax]) {
-  const int n = s.n, N = n + (n & 1), P = N / 2, M = N - 1;
+  // A step is the chain shuffle, select, rotate; its (c, s) and the next step's number
+  // are loaded beside it, the ring's one move needs no loop (further ones are rare),
+  // and sizes and step numbers pass through a broadcast, since a shuffle in a loop that
+  // is not known to be uniform waits for the warp. n = 100: 526 clocks per step with a
+  // loop over the moves, the number loaded in the chain; 240 here.
+  const int n = __shfl_sync(0xffffffffu, s.n, 0), N = n + (n & 1), P = N / 2, M = N - 1;
   const int tid = threadIdx.x, lane = tid & 31;
   const float2* jlog = reinterpret_cast<const float2*>(s.jlog);
-  const int T = s.jlog_steps;
+  const int T = __shfl_sync(0xffffffffu, s.jlog_steps, 0);
   const int K = kLogChunkMax / P;  // steps per chunk (<= kLogStepsMax)
   const int nch = ceil_div(T, K);
   float2 stage[kLogLoads];
@@ -767,8 +858,9 @@ __device__ __forceinline__ void jlog_replay(const Search& s, float* v, float2 (*
   load(0);
   store(0, 0);
   __syncthreads();
-  // the ring at the first logged step
-  int r = lr[0][0];
+  // the ring one step before the first logged one
+  int r = __shfl_sync(0xffffffffu, lr[0][0], 0) - 1;
+  if (r < 0) r += M;
   float a[PL], b[PL];
 #pragma unroll
   for (int u = 0; u < PL; ++u) {
@@ -805,21 +897,24 @@ __device__ __forceinline__ void jlog_replay(const Search& s, float* v, float2 (*
     if (c + 1 < nch) load(c + 1);  // in flight during the steps of chunk c
     const int cnt = min(K, T - c * K);
     const float2* cs = lcs[cur];
+    int rk = __shfl_sync(0xffffffffu, lr[cur][0], 0);
     for (int k = 0; k < cnt; ++k, cs += P) {
-      const int rk = lr[cur][k];
-      int moves = rk - r;  // unlogged steps between the two logged ones, plus one
-      if (moves < 0) moves += M;
-      for (int j = 0; j < moves; ++j) shift();
+      float2 g[PL];
+#pragma unroll
+      for (int u = 0; u < PL; ++u) g[u] = lane + 32 * u < P ? cs[lane + 32 * u] : make_float2(1.f, 0.f);
+      const int next = lr[cur][k + 1 < cnt ? k + 1 : 0];
+      shift();
+      int extra = rk - r - 1;  // unlogged steps between the two logged ones
+      if (extra < 0) extra += M;
+      if (extra > 0)
+        for (int j = 0; j < extra; ++j) shift();
       r = rk;
+      rk = __shfl_sync(0xffffffffu, next, 0);
 #pragma unroll
       for (int u = 0; u < PL; ++u) {
-        const int pi = lane + 32 * u;
-        if (pi < P) {
-          const float2 g = cs[pi];
-          const float x = a[u], y = b[u];
-          a[u] = g.x * x - g.y * y;
-          b[u] = g.y * x + g.x * y;
-        }
+        const float x = a[u], y = b[u];
+        a[u] = g[u].x * x - g[u].y * y;
+        b[u] = g[u].y * x + g[u].x * y;
       }
     }
     // the other buffer was last read in chunk c - 1, before the barrier below it
@@ -1062,9 +1157,7 @@ int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1
   }
   if (max_small > 0) {
     launch_eig_refine(S, s0, s1, max_small, 1, st);
-    const int bytes = jacobi32_smem_bytes(max_small);
-    cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    k_jacobi32<<<s1 - s0, kJ32NT, bytes, st>>>(S, s0);
+    launch_jacobi32(S, s0, s1, max_small, st);
     k_jlog_apply<<<dim3(ceil_div(max_small, kLogRows), s1 - s0), kLogRows * 32, 0, st>>>(S, s0);
     nl += 3;
   }
