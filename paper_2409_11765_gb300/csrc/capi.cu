@@ -41,6 +41,7 @@ struct cmaes_s {
   char* arena = nullptr;
   size_t arena_bytes = 0;
   int* d_off = nullptr;  // TK_COUNT x (count + 1)
+  double* state_buf = nullptr;  // pinned: a search's state on its way (get_state, set_state)
   int* d_err = nullptr;  // device status word (bit 0: a bounded wait timed out)
   bool mixed = false;
   std::vector<int> h_off;
@@ -165,16 +166,17 @@ static cmaes_status check_device_status(cmaes_t h) {
   return CMAES_OK;
 }
 
+// The state's way through the handle's pinned buffer: one kernel for the scalars, the
+// vectors and, up to kStateMaxN, the matrices (kernels_state.cu).
+static size_t state_bytes(const Search& x) {
+  return state_layout(x.n, x.hist_cap, x.n <= kStateMaxN).total * sizeof(double);
+}
+
 static cmaes_status read_search(cmaes_t h, int s, Search* out) {
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   cmaes_status r = check_device_status(h);
   if (r != CMAES_OK) return r;
   CUDA_TRY(h, cudaMemcpy(out, h->dS + s, sizeof(Search), cudaMemcpyDeviceToHost));
-  return CMAES_OK;
-}
-
-static cmaes_status write_search(cmaes_t h, int s, const Search* in) {
-  CUDA_TRY(h, cudaMemcpy(h->dS + s, in, sizeof(Search), cudaMemcpyHostToDevice));
   return CMAES_OK;
 }
 
@@ -564,6 +566,7 @@ void cmaes_destroy(cmaes_t h) {
   if (h->dS) cudaFree(h->dS);
   if (h->d_off) cudaFree(h->d_off);
   if (h->d_err) cudaFree(h->d_err);
+  if (h->state_buf) cudaFreeHost(h->state_buf);
   if (h->d_trd_grp) cudaFree(h->d_trd_grp);
   for (cudaEvent_t e : h->trd_pool) cudaEventDestroy(e);
   if (h->d_trd_bar) cudaFree(h->d_trd_bar);
@@ -714,6 +717,9 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
   } while (0)
   small_set_attributes();
   CREATE_TRY(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
+  size_t state_max = 0;
+  for (const Search& x : h->hs) state_max = std::max(state_max, state_bytes(x));
+  CREATE_TRY(cudaHostAlloc(reinterpret_cast<void**>(&h->state_buf), state_max, cudaHostAllocPortable));
   CREATE_TRY(cudaMemsetAsync(h->arena, 0, total, h->stream));
   for (int s = 0; s < count; ++s) {
     Search& x = h->hs[s];
@@ -1208,11 +1214,18 @@ cmaes_status cmaes_get_state(cmaes_t h, int s, cmaes_state* st) {
   CHECK_HANDLE(h);
   CHECK_SEARCH(h, s);
   if (!st) return set_error(h, CMAES_EINVAL, "state is NULL");
-  Search cur;
-  cmaes_status r = read_search(h, s, &cur);
-  if (r != CMAES_OK) return r;
   const Search& x = h->hs[s];
   const size_t n = x.n, ldn = x.ldn;
+  const bool staged = x.n <= kStateMaxN && (st->C || st->B);
+  const StateLayout l = state_layout(x.n, x.hist_cap, staged);
+  const double* buf = h->state_buf;
+  launch_state_get(h->dS, s, x.n, h->state_buf, l, h->stream);
+  cmaes_status r = launch_check(h, "get_state");
+  if (r != CMAES_OK) return r;
+  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  StateHead cur;
+  memcpy(&cur, buf, sizeof(cur));
+  if (cur.err && (r = check_device_status(h)) != CMAES_OK) return r;
   st->n = x.n;
   st->lambda = cur.lam;
   st->gen = cur.gen;
@@ -1223,16 +1236,20 @@ cmaes_status cmaes_get_state(cmaes_t h, int s, cmaes_state* st) {
   st->best_f = cur.best_f;
   const int cnt = cur.hist_count < cur.hist_len ? cur.hist_count : cur.hist_len;
   st->hist_count = cnt;
-  if (st->m) CUDA_TRY(h, cudaMemcpy(st->m, x.m, n * 8, cudaMemcpyDeviceToHost));
-  if (st->ps) CUDA_TRY(h, cudaMemcpy(st->ps, x.ps, n * 8, cudaMemcpyDeviceToHost));
-  if (st->pc) CUDA_TRY(h, cudaMemcpy(st->pc, x.pc, n * 8, cudaMemcpyDeviceToHost));
-  if (st->D) CUDA_TRY(h, cudaMemcpy(st->D, x.D, n * 8, cudaMemcpyDeviceToHost));
-  if (st->best_x) CUDA_TRY(h, cudaMemcpy(st->best_x, x.best_x, n * 8, cudaMemcpyDeviceToHost));
-  if (st->C) CUDA_TRY(h, cudaMemcpy2D(st->C, n * 8, x.C, ldn * 8, n * 8, n, cudaMemcpyDeviceToHost));
-  if (st->B) CUDA_TRY(h, cudaMemcpy2D(st->B, n * 8, x.B, ldn * 8, n * 8, n, cudaMemcpyDeviceToHost));
+  if (st->m) memcpy(st->m, buf + l.m, n * 8);
+  if (st->ps) memcpy(st->ps, buf + l.ps, n * 8);
+  if (st->pc) memcpy(st->pc, buf + l.pc, n * 8);
+  if (st->D) memcpy(st->D, buf + l.D, n * 8);
+  if (st->best_x) memcpy(st->best_x, buf + l.best_x, n * 8);
+  if (staged) {
+    if (st->C) memcpy(st->C, buf + l.C, n * n * 8);
+    if (st->B) memcpy(st->B, buf + l.B, n * n * 8);
+  } else {
+    if (st->C) CUDA_TRY(h, cudaMemcpy2D(st->C, n * 8, x.C, ldn * 8, n * 8, n, cudaMemcpyDeviceToHost));
+    if (st->B) CUDA_TRY(h, cudaMemcpy2D(st->B, n * 8, x.B, ldn * 8, n * 8, n, cudaMemcpyDeviceToHost));
+  }
   if (st->hist && cnt > 0) {
-    std::vector<double> ring(cur.hist_len);
-    CUDA_TRY(h, cudaMemcpy(ring.data(), x.hist, static_cast<size_t>(cur.hist_len) * 8, cudaMemcpyDeviceToHost));
+    const double* ring = buf + l.hist;
     const int start = cur.hist_count <= cur.hist_len ? 0 : cur.hist_count % cur.hist_len;
     for (int q = 0; q < cnt; ++q) st->hist[q] = ring[(start + q) % cur.hist_len];
   }
@@ -1255,45 +1272,58 @@ cmaes_status cmaes_set_state(cmaes_t h, int s, const cmaes_state* st) {
   const int hist_len = 10 + static_cast<int>(std::ceil(30.0 * x.n / st->lambda));
   if (st->hist_count < 0 || (st->hist_count > 0 && !st->hist))
     return set_error(h, CMAES_EINVAL, "bad hist");
-  Search cur;
-  cmaes_status r = read_search(h, s, &cur);
-  if (r != CMAES_OK) return r;
   const size_t n = x.n, ldn = x.ldn;
-  cur.lam = st->lambda;
-  cur.gen = st->gen;
-  cur.restart = st->restart;
-  cur.done = st->done;
-  cur.flags = st->flags;
-  cur.sigma = st->sigma;
-  cur.best_f = st->best_f;
-  cur.eig_due = 0;
+  const bool staged = x.n <= kStateMaxN;
+  const StateLayout l = state_layout(x.n, x.hist_cap, staged);
+  double* buf = h->state_buf;
   const int keep = st->hist_count < hist_len ? st->hist_count : hist_len;
-  cur.hist_count = keep;
-  // the snapshot holds no evaluation errors: a restored window counts them as 0
-  CUDA_TRY(h, cudaMemset(x.hist + x.hist_cap, 0, static_cast<size_t>(x.hist_cap) * 8));
-  if (keep > 0) {
-    CUDA_TRY(h, cudaMemcpy(x.hist, st->hist + (st->hist_count - keep), static_cast<size_t>(keep) * 8,
-                           cudaMemcpyHostToDevice));
+  StateHead head{};
+  head.lam = st->lambda;
+  head.gen = st->gen;
+  head.restart = st->restart;
+  head.done = st->done;
+  head.flags = st->flags;
+  head.sigma = st->sigma;
+  head.best_f = st->best_f;
+  head.hist_count = keep;
+  int has = 0;
+  auto put = [&](int field, size_t at, const double* src, size_t count) {
+    if (!src) return;
+    memcpy(buf + at, src, count * 8);
+    has |= 1 << field;
+  };
+  // (the buffer is free: every call that uses it ends with a synchronisation)
+  put(kStM, l.m, st->m, n);
+  put(kStPs, l.ps, st->ps, n);
+  put(kStPc, l.pc, st->pc, n);
+  put(kStD, l.D, st->D, n);
+  put(kStBest, l.best_x, st->best_x, n);
+  if (keep > 0) memcpy(buf + l.hist, st->hist + (st->hist_count - keep), static_cast<size_t>(keep) * 8);
+  if (staged) {
+    put(kStC, l.C, st->C, n * n);
+    put(kStB, l.B, st->B, n * n);
   }
-  if ((r = write_search(h, s, &cur)) != CMAES_OK) return r;
-  if (st->m) CUDA_TRY(h, cudaMemcpy(x.m, st->m, n * 8, cudaMemcpyHostToDevice));
-  if (st->ps) CUDA_TRY(h, cudaMemcpy(x.ps, st->ps, n * 8, cudaMemcpyHostToDevice));
-  if (st->pc) CUDA_TRY(h, cudaMemcpy(x.pc, st->pc, n * 8, cudaMemcpyHostToDevice));
-  if (st->D) CUDA_TRY(h, cudaMemcpy(x.D, st->D, n * 8, cudaMemcpyHostToDevice));
-  if (st->best_x) CUDA_TRY(h, cudaMemcpy(x.best_x, st->best_x, n * 8, cudaMemcpyHostToDevice));
-  if (st->C) CUDA_TRY(h, cudaMemcpy2D(x.C, ldn * 8, st->C, n * 8, n * 8, n, cudaMemcpyHostToDevice));
-  if (st->B) CUDA_TRY(h, cudaMemcpy2D(x.B, ldn * 8, st->B, n * 8, n * 8, n, cudaMemcpyHostToDevice));
-  launch_init_params(h->dS, s, s + 1, h->dopt, 0, h->stream);
+  launch_state_put(h->dS, s, x.n, h->dopt, buf, l, head, has, h->stream);
   h->launches += 1;
-  TileMap sq = h->tiles(TK_SQUARE, s, s + 1);
-  launch_set_bd_force(h->dS, sq, h->stream);
-  h->launches += 1;
-  if (h->mixed) {
-    launch_tc_set_bdt(h->dS, sq, h->opt.precision, 1, h->stream);
-    h->launches += 1;
-  }
-  if ((r = launch_check(h, "set_state")) != CMAES_OK) return r;
+  cmaes_status r = launch_check(h, "set_state");
+  if (r != CMAES_OK) return r;
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  StateHead back;
+  memcpy(&back, buf, sizeof(back));
+  if (back.err && (r = check_device_status(h)) != CMAES_OK) return r;
+  if (!staged) {
+    if (st->C) CUDA_TRY(h, cudaMemcpy2D(x.C, ldn * 8, st->C, n * 8, n * 8, n, cudaMemcpyHostToDevice));
+    if (st->B) CUDA_TRY(h, cudaMemcpy2D(x.B, ldn * 8, st->B, n * 8, n * 8, n, cudaMemcpyHostToDevice));
+    TileMap sq = h->tiles(TK_SQUARE, s, s + 1);
+    launch_set_bd_force(h->dS, sq, h->stream);
+    h->launches += 1;
+    if (h->mixed) {
+      launch_tc_set_bdt(h->dS, sq, h->opt.precision, 1, h->stream);
+      h->launches += 1;
+    }
+    if ((r = launch_check(h, "set_state")) != CMAES_OK) return r;
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  }
   return CMAES_OK;
 }
 

@@ -19,11 +19,15 @@ __device__ void compute_params(Search& s, const DevOptions& o, double* sh) {
   const int n = s.n, lam = s.lam, mu = lam / 2;
   const double lw = log((lam + 1) / 2.0);
   double part = 0.0;
-  for (int i = threadIdx.x; i < mu; i += NT) part += lw - log(static_cast<double>(i + 1));
+  for (int i = threadIdx.x; i < mu; i += NT) {  // (a logarithm is ~30 FP64 operations: each is taken once)
+    const double v = lw - log(static_cast<double>(i + 1));
+    s.w[i] = v;
+    part += v;
+  }
   const double sum = block_sum<NT>(part, sh);
   double sq = 0.0;
   for (int i = threadIdx.x; i < mu; i += NT) {
-    const double wi = (lw - log(static_cast<double>(i + 1))) / sum;
+    const double wi = s.w[i] / sum;
     s.w[i] = wi;
     if (s.mixed) s.w32[i] = static_cast<float>(wi);
     sq += wi * wi;

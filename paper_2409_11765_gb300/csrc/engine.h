@@ -144,6 +144,24 @@ void launch_cov_partial(Search* S, TileMap tm, cudaStream_t st);
 void launch_cov_reduce(Search* S, TileMap tm, cudaStream_t st);
 void launch_stop(Search* S, int s0, int s1, DevOptions o, cudaStream_t st);
 void launch_force_restart(Search* S, int s, DevOptions o, cudaStream_t st);
+// a search's state through a pinned buffer (kernels_state.cu): one launch for all of it
+// up to kStateMaxN, above it for all but C and B: the host's pass over the matrices then
+// takes longer than two more copies (n = 200: 66 us to restore and 34 to read through the
+// buffer, n = 333: 131 and 107 against ~125 and ~50, n = 500: 239 and 263 against ~130 and 57)
+constexpr int kStateMaxN = 256;
+struct StateHead {
+  double sigma, best_f;
+  int lam, gen, restart, done, flags, hist_count, hist_len, err;
+};
+enum StateField { kStM = 0, kStPs, kStPc, kStD, kStBest, kStC, kStB };
+struct StateLayout {
+  size_t m, ps, pc, D, best_x, hist, C, B, total;
+  bool matrices;
+};
+StateLayout state_layout(int n, int hist_cap, bool matrices);
+void launch_state_get(const Search* S, int s, int n, double* buf, const StateLayout& l, cudaStream_t st);
+void launch_state_put(Search* S, int s, int n, DevOptions o, double* buf, const StateLayout& l, const StateHead& h,
+                      int has, cudaStream_t st);
 // launchers (kernels_eig.cu)
 void launch_eig_gemm_CB(Search* S, TileMap tm, cudaStream_t st);
 void launch_eig_gemm_BtT(Search* S, TileMap tm, cudaStream_t st);
