@@ -330,7 +330,7 @@ static void enqueue_eig(cmaes_t h, int s0, int s1, cudaStream_t st) {
     TileMap tsy = h->tiles(TK_FLATSYM, s0, s1);
     int nl = launch_eig_mixed_head(h->dS, tfl, tsy, s0, s1, h->max_n_refine, st);
     if (h->max_n_big > 0) nl += enqueue_jacobi32_big(h, s0, s1, st);
-    nl += launch_eig_mixed_tail(h->dS, tfl, tsy, s0, s1, h->max_n_refine, st);
+    nl += launch_eig_mixed_tail(h->dS, tfl, tsy, s0, s1, h->max_n_refine, h->mixed, st);
     h->launches += nl;
     h->phase_launch[kPhaseEig] += nl;
   }

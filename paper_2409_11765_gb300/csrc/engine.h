@@ -229,7 +229,8 @@ int tiles_flat_sym(int n);
 // the refined route in two parts around the many-CTA FP32 Jacobi: the
 // warm-start products (and the one-CTA FP32 Jacobi), then the refinement
 int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, cudaStream_t st);
-int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, cudaStream_t st);
+int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, bool mixed,
+                          cudaStream_t st);
 // the products of that route for n <= kEigMixedMaxN (kernels_eig_refine.cu)
 void launch_eig_refine(Search* S, int s0, int s1, int max_n, int head, cudaStream_t st);
 // launchers (kernels_eig_big.cu)

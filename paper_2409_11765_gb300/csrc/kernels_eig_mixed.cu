@@ -30,8 +30,8 @@
 //   4. One Newton-Schulz step X <- X + X (I - X^T X) / 2 removes the
 //      second-order loss of orthogonality that large first-order corrections
 //      leave (error e -> 1.5 e^2).
-//   5. A = X^T C X in FP64, B <- X; on mixed-precision handles a few rounds of
-//      targeted rotations (k_pair_rounds) take the pairs the refinement left;
+//   5. A = X^T C X in FP64, B <- X; a few rounds of targeted rotations
+//      (k_pair_rounds; n <= kEigMixedMaxN) take the pairs the refinement left;
 //      the FP64 Jacobi then runs on (A, B) as in
 //      the FP64 path: it rotates what step 3 left (pairs of close eigenvalues),
 //      normally ends at its first quiet step, and delivers the eigenvalues, the
@@ -975,8 +975,13 @@ __global__ void __launch_bounds__(kLogNT) k_jlog_apply(Search* S, int s0) {
 // A lives in shared memory for the whole kernel (leading dimension n + 1, up to
 // 161 x 160 doubles) and goes back to EA only if a rotation was applied: a
 // round then costs shared-memory passes instead of a scan of A through L2.
-// Mixed-precision handles only: the FP64 handles' stricter floor leaves tens
-// of noise-level pairs, which the cluster's 8 SMs rotate faster than one CTA.
+// FP64 handles take part from n = kRoundsMinN: their floor is four times lower, but A's
+// products round well below it, so that what passes the test are pairs of close
+// eigenvalues, a few per decomposition, for which the cyclic sweeps took one to two
+// hundred steps of two cluster barriers (the decomposition of ten searches of n = 100
+// 744 -> 600 us, of three of n = 160 1290 -> 963, of four of n = 64 185 -> 183; six of
+// n = 40, with nothing to rotate, 146 -> 151).
+constexpr int kRoundsMinN = 64;
 constexpr int kRoundsNT = 512;
 constexpr int kRoundsMax = 16;
 constexpr int kRoundsList = 512;
@@ -995,7 +1000,7 @@ __global__ void __launch_bounds__(kRoundsNT) k_pair_rounds(Search* S, int s0) {
   __shared__ double papp[kRoundsPick], paqq[kRoundsPick], papq[kRoundsPick];
   __shared__ double shr[kRoundsNT / 32];
   Search& s = S[s0 + blockIdx.x];
-  if (!small_route_due(s) || !s.mixed) return;
+  if (!small_route_due(s) || (!s.mixed && s.n < kRoundsMinN)) return;
   const int n = s.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long L = s.ldn;
   double* Ag = s.EA;
@@ -1021,7 +1026,7 @@ __global__ void __launch_bounds__(kRoundsNT) k_pair_rounds(Search* S, int s0) {
   double am = 0.0;
   for (int i = tid; i < n; i += kRoundsNT) am = fmax(am, fabs(A[i + la * i]));
   const double amax = block_max<kRoundsNT>(am, shr);
-  const double floor_abs = 4.0 * n * 0x1p-53 * amax;  // the cleanup's floor on mixed handles
+  const double floor_abs = (s.mixed ? 4.0 : 1.0) * n * 0x1p-53 * amax;  // the cleanup's floor
   const long long floor_bits = __double_as_longlong(floor_abs);
   long long rot_total = 0;
   for (int round = 0; round < kRoundsMax; ++round) {
@@ -1164,7 +1169,8 @@ int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1
   return nl;
 }
 
-int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, cudaStream_t st) {
+int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, bool mixed,
+                          cudaStream_t st) {
   int nl = 0;
   if (s1 <= s0) return nl;
   if (tflat.total > 0) {
@@ -1192,10 +1198,12 @@ int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1
   }
   if (max_small > 0) {
     launch_eig_refine(S, s0, s1, max_small, 0, st);
+    ++nl;
+    if (!mixed && max_small < kRoundsMinN) return nl;
     const int rbytes = pair_rounds_smem_bytes(max_small);
     cudaFuncSetAttribute(k_pair_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, rbytes);
     k_pair_rounds<<<s1 - s0, kRoundsNT, rbytes, st>>>(S, s0);
-    nl += 2;
+    ++nl;
   }
   return nl;
 }
