@@ -1,6 +1,8 @@
 // kernels_ozaki.cu -- the general FP64-accurate product C = alpha A B + beta C
 // on the BF16 tensor cores (digit planes and bucket sums of ozaki.cuh), used
 // by include/cmaes_ozaki.h and by the eigensolver's Gram products.
+#include <algorithm>
+#include <mutex>
 #include <cuda_runtime.h>
 #include "../../include/cmaes_ozaki.h"
 #include "engine.h"
@@ -15,16 +17,58 @@ struct OzPackJob {
   int R, K, nks;
   unsigned char* out;
   int* e;
-  int block0;  // first CTA of this job in the launch
+  int blocks;  // 64-row blocks
 };
 
-__global__ void __launch_bounds__(kOzNT) k_oz_pack(const OzPackJob* jobs, int njobs) {
+// Packing both operands with one CTA per 64 rows was a serial pass of K / 32 steps on a
+// few CTAs (1000 x 1024 x 2000: 32 CTAs, 240 us). Here CTAs take 64 rows by kOzPackK,
+// first for the rows' exponents (e starts below kOzZeroExp), then, with those complete,
+// for the digits; the second pass finds the operands in L2. Bound by the digits' 14
+// bytes per element on their way to L2: 13 + 28 us for the same operands.
+constexpr int kOzPackKC = 4, kOzPackK = kOzPackKC * kOzKS;
+
+template <class F>
+__device__ __forceinline__ void oz_pack_job(const OzPackJob& a, const OzPackJob& b, const F& f) {
+  int rb = static_cast<int>(blockIdx.x);
+  const OzPackJob& J = rb < a.blocks ? a : b;
+  if (rb >= a.blocks) rb -= a.blocks;
+  f(J, [&](int r, int k) { return J.src[static_cast<long long>(r) * J.sr + static_cast<long long>(k) * J.sk]; }, rb);
+}
+
+__global__ void __launch_bounds__(kOzNT) k_oz_exponents(OzPackJob a, OzPackJob b) {
   __shared__ int sh_e[64];
-  int j = 0;
-  while (j + 1 < njobs && jobs[j + 1].block0 <= static_cast<int>(blockIdx.x)) ++j;
-  const OzPackJob J = jobs[j];
-  const int rb = static_cast<int>(blockIdx.x) - J.block0;
-  oz_pack_block(J.src, J.sr, J.sk, J.R, J.K, rb, J.nks, J.out, J.e, sh_e);
+  if (threadIdx.x < 64) sh_e[threadIdx.x] = kOzZeroExp;
+  __syncthreads();
+  oz_pack_job(a, b, [&](const OzPackJob& J, auto get, int rb) {
+    const bool kfast = J.sk == 1;
+    int rl, oc;
+    oz_pack_place(kfast, rl, oc);
+    int e = kOzZeroExp;
+    for (int k0 = blockIdx.y * kOzPackK; k0 < J.K; k0 += gridDim.y * kOzPackK)
+      e = max(e, oz_pack_exponent(get, kfast, J.R, k0, min(J.K, k0 + kOzPackK), rb));
+    atomicMax(&sh_e[rl], e);
+    __syncthreads();
+    if (oc == 0) atomicMax(&J.e[rb * 64 + rl], sh_e[rl]);
+  });
+}
+
+// One step of K in one pass (64 x 64 x 64: 60 us a call, 70 in two).
+__global__ void __launch_bounds__(kOzNT) k_oz_pack_short(OzPackJob a, OzPackJob b) {
+  __shared__ int sh_e[64];
+  oz_pack_job(a, b, [&](const OzPackJob& J, auto get, int rb) {
+    oz_pack_block_get(get, J.sk == 1, J.R, J.K, rb, J.nks, J.out, J.e, sh_e);
+  });
+}
+
+__global__ void __launch_bounds__(kOzNT) k_oz_pack(OzPackJob a, OzPackJob b) {
+  oz_pack_job(a, b, [&](const OzPackJob& J, auto get, int rb) {
+    const bool kfast = J.sk == 1;
+    int rl, oc;
+    oz_pack_place(kfast, rl, oc);
+    const int e = J.e[rb * 64 + rl];
+    for (int kc0 = blockIdx.y * kOzPackKC; kc0 < J.nks; kc0 += gridDim.y * kOzPackKC)
+      oz_pack_digits(get, kfast, J.R, J.K, rb, J.nks, kc0, min(J.nks, kc0 + kOzPackKC), e, J.out);
+  });
 }
 
 // C (M x N, column-major, ldc) = alpha * A B + beta * C from packed A (M rows)
@@ -40,11 +84,10 @@ struct OzGemmJob {
   double alpha, beta;
 };
 
-__global__ void __launch_bounds__(kOzNT, 1) k_oz_gemm(const OzGemmJob* job, int* err) {
+__global__ void __launch_bounds__(kOzNT, 1) k_oz_gemm(OzGemmJob J, int* err) {
   extern __shared__ unsigned char dyn[];
   __shared__ uint64_t bar[5];
   __shared__ uint32_t tslot;
-  const OzGemmJob J = *job;
   const int tn_count = (J.N + kOzBN - 1) / kOzBN;
   const int tm = static_cast<int>(blockIdx.x) / tn_count, tn = static_cast<int>(blockIdx.x) % tn_count;
   OzCtx cx;
@@ -77,6 +120,64 @@ __global__ void __launch_bounds__(kOzNT, 1) k_oz_gemm(const OzGemmJob* job, int*
 
 using namespace cmaes_gb300;
 
+// Workspace up to kOzKeep from a stream-ordered pool of the engine's own, so that a call
+// neither maps nor unmaps memory: cudaMalloc and cudaFree take up to 150 us of a call
+// (500 x 500 x 500: 251 us with them, 112 from the pool) and synchronise the device. The
+// pool keeps at most kOzKeep bytes per device between calls; what several threads took
+// beyond that goes back at the next synchronisation, and an allocation that fails gives
+// everything back first. Pools are safe from every thread and stream. A larger
+// workspace, or one where there is no pool, is cudaMalloc's: the pool would map and
+// unmap it on every call (3000 x 3000 x 3000: 2630 us, 2870 from the pool).
+namespace {
+constexpr uint64_t kOzKeep = 64ull << 20;
+constexpr int kOzMaxDevices = 64;
+std::mutex g_oz_mutex;
+cudaMemPool_t g_oz_pool[kOzMaxDevices] = {nullptr};
+
+cudaMemPool_t oz_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kOzMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_oz_mutex);
+  if (!g_oz_pool[dev]) {
+    int ok = 0;
+    if (cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, dev) != cudaSuccess || !ok) return nullptr;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = kOzKeep;
+    cudaMemPool_t p = nullptr;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
+    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return nullptr;
+    }
+    g_oz_pool[dev] = p;
+  }
+  return g_oz_pool[dev];
+}
+
+struct OzWorkspace {
+  unsigned char* p = nullptr;
+  bool pooled = false;
+  bool get(size_t bytes, cudaStream_t st) {
+    if (cudaMemPool_t pool = bytes <= kOzKeep ? oz_pool() : nullptr) {
+      if (cudaMallocFromPoolAsync(reinterpret_cast<void**>(&p), bytes, pool, st) == cudaSuccess) return pooled = true;
+      cudaGetLastError();
+      cudaMemPoolTrimTo(pool, 0);
+    }
+    p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+  }
+  void give_back(cudaStream_t st) {
+    if (pooled) cudaFreeAsync(p, st);
+    else cudaFree(p);
+  }
+};
+}  // namespace
+
 extern "C" int cmaes_ozaki_dgemm(int M, int N, int K, double alpha, const double* A, long long lda,
                                  const double* B, long long ldb, double beta, double* C, long long ldc,
                                  void* stream) {
@@ -84,47 +185,49 @@ extern "C" int cmaes_ozaki_dgemm(int M, int N, int K, double alpha, const double
   if (M == 0 || N == 0) return 0;
   if (!A || !B || !C || lda < M || ldb < K || ldc < M) return 1;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int nks = oz_nks(K);
-  const size_t abytes = oz_bytes(M, K), bbytes = oz_bytes(N, K);
-  const int mpad = oz_rows_padded(M), npad = oz_rows_padded(N);
-  unsigned char* ws = nullptr;
-  const size_t jobs_off = abytes + bbytes + sizeof(int) * (mpad + npad);
-  const size_t jobs_at = (jobs_off + 255) / 256 * 256;
-  const size_t total = jobs_at + sizeof(OzPackJob) * 2 + sizeof(OzGemmJob) + sizeof(int);
-  if (cudaMalloc(&ws, total) != cudaSuccess) {
+  // a call ends with a synchronisation, so a stream under capture cannot take it
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return 2;
   }
-  unsigned char* pa = ws;
-  unsigned char* pb = ws + abytes;
-  int* ea = reinterpret_cast<int*>(ws + abytes + bbytes);
+  const int nks = oz_nks(K);
+  const size_t abytes = oz_bytes(M, K), bbytes = oz_bytes(N, K);
+  const int mpad = oz_rows_padded(M), npad = oz_rows_padded(N);
+  const size_t ebytes = sizeof(int) * (static_cast<size_t>(mpad) + npad);
+  OzWorkspace ws;
+  if (!ws.get(abytes + bbytes + ebytes + sizeof(int), st)) return 2;
+  unsigned char* pa = ws.p;
+  unsigned char* pb = pa + abytes;
+  int* ea = reinterpret_cast<int*>(pb + bbytes);
   int* eb = ea + mpad;
-  OzPackJob pj[2];
+  int* d_err = eb + npad;
   // A: row i, K index k at A[i + lda k]; B: row j (a column of B), k at B[k + ldb j]
-  pj[0] = OzPackJob{A, 1, lda, M, K, nks, pa, ea, 0};
-  pj[1] = OzPackJob{B, ldb, 1, N, K, nks, pb, eb, mpad / 64};
-  OzGemmJob gj{pa, ea, pb, eb, M, N, nks, C, ldc, alpha, beta};
-  OzPackJob* d_pj = reinterpret_cast<OzPackJob*>(ws + jobs_at);
-  OzGemmJob* d_gj = reinterpret_cast<OzGemmJob*>(d_pj + 2);
-  int* d_err = reinterpret_cast<int*>(d_gj + 1);
+  const OzPackJob ja{A, 1, lda, M, K, nks, pa, ea, mpad / 64};
+  const OzPackJob jb{B, ldb, 1, N, K, nks, pb, eb, npad / 64};
+  const OzGemmJob gj{pa, ea, pb, eb, M, N, nks, C, ldc, alpha, beta};
   int rc = 0;
   int herr = 0;
-  if (cudaMemcpyAsync(d_pj, pj, sizeof(pj), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(d_gj, &gj, sizeof(gj), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemsetAsync(d_err, 0, sizeof(int), st) != cudaSuccess) {
+  // one fill for the exponents (0x80808080 is below kOzZeroExp) and the status word
+  // (whose timeout bit it leaves clear)
+  if (cudaMemsetAsync(ea, 0x80, ebytes + sizeof(int), st) != cudaSuccess) {
     rc = 3;
   } else {
-    k_oz_pack<<<mpad / 64 + npad / 64, kOzNT, 0, st>>>(d_pj, 2);
+    const dim3 grid(mpad / 64 + npad / 64, std::min(65535, (nks + kOzPackKC - 1) / kOzPackKC));
+    if (nks > 0 && nks <= kOzPackKC) {
+      k_oz_pack_short<<<grid.x, kOzNT, 0, st>>>(ja, jb);
+    } else if (nks > 0) {
+      k_oz_exponents<<<grid, kOzNT, 0, st>>>(ja, jb);
+      k_oz_pack<<<grid, kOzNT, 0, st>>>(ja, jb);
+    }
     cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSmem);
     const int tiles = (mpad / kOzBM) * ((N + kOzBN - 1) / kOzBN);
-    k_oz_gemm<<<tiles, kOzNT, kOzSmem, st>>>(d_gj, d_err);
-    if (cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      rc = 3;
-    else if (herr)
-      rc = 4;
+    k_oz_gemm<<<tiles, kOzNT, kOzSmem, st>>>(gj, d_err);
+    if (cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = 3;
   }
+  ws.give_back(st);
+  if (cudaStreamSynchronize(st) != cudaSuccess) rc = 3;
+  else if (rc == 0 && (herr & kDevErrTimeout)) rc = 4;
   if (cudaGetLastError() != cudaSuccess) rc = 3;
-  cudaFree(ws);
   return rc;
 }

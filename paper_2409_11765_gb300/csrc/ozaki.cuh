@@ -113,30 +113,39 @@ __device__ __forceinline__ int oz_off(int r, int k) {
 // call it; sh_e holds 64 ints. Writes the row exponents to e_out[r] (r < the
 // padded row count).
 // --------------------------------------------------------------------------
-template <class Get>
-__device__ __forceinline__ void oz_pack_block_get(const Get& get, bool kfast, int R, int K, int rb, int nks,
-                                                  unsigned char* __restrict__ out, int* __restrict__ e_out,
-                                                  int* sh_e) {
+// This thread's row and octet of K within a 64-row block.
+__device__ __forceinline__ void oz_pack_place(bool kfast, int& rl, int& oc) {
   const int tid = threadIdx.x;
-  const int rl = kfast ? (tid >> 2) : (tid & 63);
-  const int oc = kfast ? (tid & 3) : (tid >> 6);
+  rl = kfast ? (tid >> 2) : (tid & 63);
+  oc = kfast ? (tid & 3) : (tid >> 6);
+}
+
+// Its part of the row's exponent over k0 <= k < k1 (k0 a multiple of 32).
+template <class Get>
+__device__ __forceinline__ int oz_pack_exponent(const Get& get, bool kfast, int R, int k0, int k1, int rb) {
+  int rl, oc;
+  oz_pack_place(kfast, rl, oc);
   const int r = rb * 64 + rl;
-  if (tid < 64) sh_e[tid] = kOzZeroExp;
-  __syncthreads();
   int emax = kOzZeroExp;
   if (r < R) {
-    for (int k = oc * 8; k < K; k += 32) {
+    for (int k = k0 + oc * 8; k < k1; k += 32) {
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (k + u < K) emax = max(emax, oz_exponent(get(r, k + u)));
+        if (k + u < k1) emax = max(emax, oz_exponent(get(r, k + u)));
     }
   }
-  atomicMax(&sh_e[rl], emax);
-  __syncthreads();
-  const int e = sh_e[rl];
-  if (oc == 0) e_out[r] = e;
+  return emax;
+}
+
+// Its digits of the K chunks kc0 .. kc1 - 1, for the row exponent e.
+template <class Get>
+__device__ __forceinline__ void oz_pack_digits(const Get& get, bool kfast, int R, int K, int rb, int nks, int kc0,
+                                               int kc1, int e, unsigned char* __restrict__ out) {
+  int rl, oc;
+  oz_pack_place(kfast, rl, oc);
+  const int r = rb * 64 + rl;
   unsigned char* base = out + static_cast<long long>(rb) * oz_pitch(nks);
-  for (int kc = 0; kc < nks; ++kc) {
+  for (int kc = kc0; kc < kc1; ++kc) {
     uint32_t pk[kOzS][4];
 #pragma unroll
     for (int u = 0; u < 8; u += 2) {
@@ -154,6 +163,22 @@ __device__ __forceinline__ void oz_pack_block_get(const Get& get, bool kfast, in
     for (int p = 0; p < kOzS; ++p)
       *reinterpret_cast<uint4*>(blk + p * kOzBlk) = make_uint4(pk[p][0], pk[p][1], pk[p][2], pk[p][3]);
   }
+}
+
+template <class Get>
+__device__ __forceinline__ void oz_pack_block_get(const Get& get, bool kfast, int R, int K, int rb, int nks,
+                                                  unsigned char* __restrict__ out, int* __restrict__ e_out,
+                                                  int* sh_e) {
+  const int tid = threadIdx.x;
+  int rl, oc;
+  oz_pack_place(kfast, rl, oc);
+  if (tid < 64) sh_e[tid] = kOzZeroExp;
+  __syncthreads();
+  atomicMax(&sh_e[rl], oz_pack_exponent(get, kfast, R, 0, K, rb));
+  __syncthreads();
+  const int e = sh_e[rl];
+  if (oc == 0) e_out[rb * 64 + rl] = e;
+  oz_pack_digits(get, kfast, R, K, rb, nks, 0, nks, e, out);
 }
 
 // The same for a strided view x(r, k) = src[r * sr + k * sk].
