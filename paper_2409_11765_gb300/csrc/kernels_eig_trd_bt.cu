@@ -23,6 +23,7 @@
 namespace cmaes_gb300 {
 
 constexpr int kBtFinCols = 8;  // columns per CTA of the final pass (one warp each)
+constexpr int kBtTfNT = 64, kBtTfTiles = kBtNb / (kBtTfNT / 32);  // T_p: two rows per CTA
 
 int tiles_bt_pack(int n) {
   if (!trd_bt_blocked(n)) return 0;
@@ -31,12 +32,11 @@ int tiles_bt_pack(int n) {
   return t;
 }
 int tiles_bt_gram(int n) { return trd_bt_blocked(n) ? 2 * trd_panels(n) : 0; }
-int tiles_bt_tfac(int n) { return trd_bt_blocked(n) ? trd_panels(n) : 0; }
+int tiles_bt_tfac(int n) { return trd_bt_blocked(n) ? trd_panels(n) * kBtTfTiles : 0; }
 int tiles_bt_rows(int n) { return trd_bt_blocked(n) ? oz_rows_padded(n) / 64 : 0; }
 int tiles_bt_cols(int n) { return trd_bt_blocked(n) ? ceil_div(n, kOzBN) : 0; }
 int tiles_bt_update(int n) { return trd_bt_blocked(n) ? ceil_div(n - 1, kOzBM) * ceil_div(n, kOzBN) : 0; }
 int tiles_bt_final(int n) { return trd_bt_blocked(n) ? ceil_div(n, kBtFinCols) : 0; }
-static size_t bt_tfac_smem() { return static_cast<size_t>(kBtNb) * kBtNb * 8; }
 
 // ---------------------------------------------------------------- setup ----
 // Tiles 0 .. 2P-1: the two 64-row blocks of Y_p^T (row c = reflector k0 + c,
@@ -102,42 +102,79 @@ __global__ void __launch_bounds__(kOzNT, 1) k_bt_gram(Search* S, TileMap tm) {
   oz_end(cx);
 }
 
-// T_p (column by column in shared memory; row r of every column is formed by
-// thread r from its own earlier entries) and its packed form.
-__global__ void __launch_bounds__(kOzNT) k_bt_tfac(Search* S, TileMap tm) {
-  extern __shared__ double Tsm[];  // 128 x 128, column-major
-  __shared__ int sh_e[64];
-  int p;
-  const int si = find_search(tm, p);
+// T_p and its packed form. Its rows are independent: with t = T(r, :),
+//   t_r = tau_r,  t_c = -tau_c sum_{l = r}^{c - 1} t_l G(l, c)   (c > r),
+// so a warp takes a row, lane l the columns 4 l .. 4 l + 3 of its sums, and each t_c is
+// broadcast and added into the later ones. A step is the chain product, broadcast,
+// multiply-add (~200 clocks; the four multiply-adds of a warp take the SM's FP64 pipe for
+// 76), with the rows of G (symmetric: G(l, c) is read as G(c, l), four consecutive values
+// per lane) loaded four steps ahead. One CTA per panel with a thread per row ran 128
+// columns of sums of up to 128 dependent multiply-adds: 460 us, whatever n; 64 CTAs of
+// two rows per panel: 32 us at n = 500. (The back-transformation: n = 333 945 -> 556 us,
+// n = 500 1212 -> 805, n = 1000 2337 -> 1926.)
+__global__ void __launch_bounds__(kBtTfNT) k_bt_tfac(Search* S, TileMap tm) {
+  static_assert(kBtNb == 128, "four columns per lane");
+  int t;
+  const int si = find_search(tm, t);
   const Search& s = S[si];
   if (!trd_due(s)) return;
+  const int lane = threadIdx.x & 31;
+  const int p = t / kBtTfTiles;
+  const int r = __shfl_sync(0xffffffffu, (t % kBtTfTiles) * (kBtTfNT / 32) + (static_cast<int>(threadIdx.x) >> 5), 0);
   const int n = s.n, k0 = kBtNb * p, nb = trd_panel_nb(n, p);
   const TrdOz lay = trd_oz_layout(n);
-  const double* G = reinterpret_cast<const double*>(s.ozp + lay.g) + static_cast<size_t>(p) * kBtNb * kBtNb;
-  double* Tg = reinterpret_cast<double*>(s.ozp + lay.tf) + static_cast<size_t>(p) * kBtNb * kBtNb;
-  const double* tau = tv(s, TV_TAU);
-  for (int e = threadIdx.x; e < kBtNb * kBtNb; e += kOzNT) Tsm[e] = 0.0;
-  __syncthreads();
-  const int r = threadIdx.x;
-  for (int c = 0; c < kBtNb; ++c) {
-    const double tc = c < nb ? tau[k0 + c] : 0.0;
-    if (r < c) {
-      double acc = 0.0;
-      for (int l = r; l < c; ++l) acc = fma(Tsm[r + kBtNb * l], G[l + kBtNb * c], acc);
-      Tsm[r + kBtNb * c] = -tc * acc;
-    } else if (r == c) {
-      Tsm[c + kBtNb * c] = tc;
+  const double* G = reinterpret_cast<const double*>(s.ozp + lay.g) + static_cast<size_t>(p) * kBtNb * kBtNb + 4 * lane;
+  const double* tau = tv(s, TV_TAU) + k0;
+  double tj[4], acc[4], x[4];  // tau, the sums and T(r, .) of columns 4 lane + u
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    tj[u] = 4 * lane + u < nb ? tau[4 * lane + u] : 0.0;
+    acc[u] = x[u] = 0.0;
+  }
+  double2 g[4][2], h[4][2];
+  auto load = [&](double2 (&v)[4][2], int c0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double2* src = reinterpret_cast<const double2*>(G + kBtNb * (c0 + q));
+      v[q][0] = src[0];
+      v[q][1] = src[1];
+    }
+  };
+  load(g, r & ~3);
+  for (int c0 = r & ~3; c0 < kBtNb; c0 += 4) {
+    if (c0 + 4 < kBtNb) load(h, c0 + 4);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = c0 + q;
+      if (c < r) continue;
+      const double mine = c == r ? tj[q] : -tj[q] * acc[q];
+      const double tc = __shfl_sync(0xffffffffu, mine, c0 >> 2);
+      if (lane == c0 >> 2) x[q] = tc;
+      acc[0] = fma(tc, g[q][0].x, acc[0]);
+      acc[1] = fma(tc, g[q][0].y, acc[1]);
+      acc[2] = fma(tc, g[q][1].x, acc[2]);
+      acc[3] = fma(tc, g[q][1].y, acc[3]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      g[q][0] = h[q][0];
+      g[q][1] = h[q][1];
     }
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kBtNb * kBtNb; e += kOzNT) Tg[e] = Tsm[e];
-  unsigned char* out = s.ozp + lay.t + static_cast<size_t>(p) * trd_align256(oz_bytes(kBtNb, kBtNb));
-  int* eo = s.oze + lay.et + kBtNb * p;
-  for (int rb = 0; rb < 2; ++rb) {
-    oz_pack_block_get([=] __device__(int i, int k) { return Tsm[i + kBtNb * k]; }, false, kBtNb, kBtNb, rb,
-                      oz_nks(kBtNb), out, eo, sh_e);
-    __syncthreads();
-  }
+  int e = kOzZeroExp;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) e = max(e, oz_exponent(x[u]));
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0) s.oze[lay.et + kBtNb * p + r] = e;
+  uint32_t d[4][kOzS];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) oz_digits(x[u], e, d[u]);
+  unsigned char* out = s.ozp + lay.t + static_cast<size_t>(p) * trd_align256(oz_bytes(kBtNb, kBtNb)) +
+                       static_cast<long long>(r >> 6) * oz_pitch(oz_nks(kBtNb)) +
+                       static_cast<long long>(lane >> 3) * kOzS * kOzBlk + oz_off(r & 63, 4 * (lane & 7));
+#pragma unroll
+  for (int q = 0; q < kOzS; ++q)
+    *reinterpret_cast<uint2*>(out + q * kOzBlk) = make_uint2(d[0][q] | d[1][q] << 16, d[2][q] | d[3][q] << 16);
 }
 
 // ------------------------------------------------------------ one panel ----
@@ -315,7 +352,6 @@ void bt_set_attributes() {
   cudaFuncSetAttribute(k_bt_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSmem);
   cudaFuncSetAttribute(k_bt_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSmem);
   cudaFuncSetAttribute(k_bt_update, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSmem);
-  cudaFuncSetAttribute(k_bt_tfac, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bt_tfac_smem()));
 }
 
 int launch_bt(Search* S, const TrdMaps& m, int max_n, cudaStream_t st) {
@@ -323,7 +359,7 @@ int launch_bt(Search* S, const TrdMaps& m, int max_n, cudaStream_t st) {
   auto go = [&](const TileMap& t) { return t.total > 0 ? (++nl, true) : false; };
   if (go(m.btpack)) k_bt_pack_y<<<m.btpack.total, kOzNT, 0, st>>>(S, m.btpack);
   if (go(m.btgram)) k_bt_gram<<<m.btgram.total, kOzNT, kOzSmem, st>>>(S, m.btgram);
-  if (go(m.bttfac)) k_bt_tfac<<<m.bttfac.total, kOzNT, bt_tfac_smem(), st>>>(S, m.bttfac);
+  if (go(m.bttfac)) k_bt_tfac<<<m.bttfac.total, kBtTfNT, 0, st>>>(S, m.bttfac);
   const int steps = trd_bt_blocked(max_n) ? trd_panels(max_n) : 0;
   for (int r = 0; r < steps; ++r) {
     if (go(m.btrows)) k_bt_pack_v<<<m.btrows.total, kOzNT, 0, st>>>(S, m.btrows, r);

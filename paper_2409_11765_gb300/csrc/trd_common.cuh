@@ -64,7 +64,7 @@ __device__ __forceinline__ int* ti(const Search& s, int which) {
 //   y   per panel, the rows of its reflector block (K = 128)
 //   t   per panel, the rows of its triangular factor T_p (K = 128)
 //   w   the columns of W = Y_p^T V (or T_p W) as a packed operand (K = 128)
-//   g, tf  per panel, Y_p^T Y_p and T_p in FP64 (128 x 128, column-major)
+//   g       per panel, Y_p^T Y_p in FP64 (128 x 128, column-major)
 //   wf  W in FP64 (128 x n, column-major)
 // Search::oze, int offsets: v [0, np), w [np, 2 np), yt 2 np + 128 p,
 // y 2 np + 128 P + (padded rows of the earlier panels), t after y (128 per
@@ -89,7 +89,7 @@ __host__ __device__ inline int trd_panel_nb(int n, int p) {
 }
 
 struct TrdOz {
-  size_t v, yt, y, t, w, g, tf, wf, total;  // bytes
+  size_t v, yt, y, t, w, g, wf, total;  // bytes
   int ev, ew, eyt, ey, et, etotal;         // ints
 };
 
@@ -108,8 +108,6 @@ __host__ __device__ inline TrdOz trd_oz_layout(int n) {
   L.w = o;
   o += trd_align256(oz_bytes(n, kBtNb));
   L.g = o;
-  o += static_cast<size_t>(P) * kBtNb * kBtNb * 8;
-  L.tf = o;
   o += static_cast<size_t>(P) * kBtNb * kBtNb * 8;
   L.wf = o;
   o += trd_align256(static_cast<size_t>(kBtNb) * n * 8);
