@@ -975,13 +975,17 @@ __global__ void __launch_bounds__(kLogNT) k_jlog_apply(Search* S, int s0) {
 // A lives in shared memory for the whole kernel (leading dimension n + 1, up to
 // 161 x 160 doubles) and goes back to EA only if a rotation was applied: a
 // round then costs shared-memory passes instead of a scan of A through L2.
-// FP64 handles take part from n = kRoundsMinN: their floor is four times lower, but A's
-// products round well below it, so that what passes the test are pairs of close
-// eigenvalues, a few per decomposition, for which the cyclic sweeps took one to two
-// hundred steps of two cluster barriers (the decomposition of ten searches of n = 100
-// 744 -> 600 us, of three of n = 160 1290 -> 963, of four of n = 64 185 -> 183; six of
-// n = 40, with nothing to rotate, 146 -> 151).
+// FP64 handles take part from n = kRoundsMinN and with up to kRoundsFew pairs pending:
+// their floor is four times lower, but A's products round well below it, so that what
+// passes the test early in a descent are a few pairs of close eigenvalues, for which the
+// cyclic sweeps took one to two hundred steps of two cluster barriers (the decomposition
+// of ten searches of n = 100 744 -> 600 us, of three of n = 160 1290 -> 963, of four of
+// n = 64 185 -> 183; six of n = 40, with nothing to rotate, 146 -> 151). Late in a
+// descent on an ill-conditioned function hundreds are left, and the cluster's eight SMs
+// rotate those faster (three searches of n = 85, a generation: 6 rotations each 509 us
+// with the rounds and 564 without, 31 each 713 and 735, 100 each 912 and 805).
 constexpr int kRoundsMinN = 64;
+constexpr int kRoundsFew = 32;
 constexpr int kRoundsNT = 512;
 constexpr int kRoundsMax = 16;
 constexpr int kRoundsList = 512;
@@ -1057,7 +1061,7 @@ __global__ void __launch_bounds__(kRoundsNT) k_pair_rounds(Search* S, int s0) {
     }
     __syncthreads();
     const int c = cnt;
-    if (c == 0 || c > kRoundsList) break;  // done, or too many: the cyclic sweeps take them
+    if (c == 0 || c > (s.mixed ? kRoundsList : kRoundsFew)) break;  // done, or too many: the cyclic sweeps take them
     // bitonic sort of the candidate keys (padded to a power of two)
     int cap = 1;
     while (cap < c) cap <<= 1;
