@@ -813,23 +813,26 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     // as fit and the columns in HBM.
     constexpr int kTrdCols = 4;
     std::vector<int> G(count, 0);
+    std::vector<std::vector<int>> parts(1);  // the searches of each launch
+    for (int s = 0; s < count; ++s)
+      if (h->hs[s].trd) parts[0].push_back(s);
+    const size_t nact = parts[0].size();
     auto share = [&](long long budget) {
-      double wsum = 0.0;
-      long long nact = 0, caps = 0;
-      for (int s = 0; s < count; ++s) {
-        if (!h->hs[s].trd) continue;
-        const double n = h->hs[s].n;
-        wsum += n * n * n;
-        ++nact;
-        caps += std::min<long long>(h->hs[s].n / kTrdCols, sms);
-      }
-      for (int s = 0; s < count; ++s) {
-        if (!h->hs[s].trd) continue;
-        const double n = h->hs[s].n;
-        const long long cap = std::min<long long>(h->hs[s].n / kTrdCols, sms);
-        const long long spare = budget > nact ? budget - nact : 0;
-        G[s] = caps <= budget ? static_cast<int>(cap)
-                              : static_cast<int>(std::min(cap, 1 + static_cast<long long>(spare * (n * n * n / wsum))));
+      for (const std::vector<int>& part : parts) {
+        double wsum = 0.0;
+        long long caps = 0;
+        for (int s : part) {
+          const double n = h->hs[s].n;
+          wsum += n * n * n;
+          caps += std::min<long long>(h->hs[s].n / kTrdCols, sms);
+        }
+        const long long spare = std::max<long long>(0, budget - static_cast<long long>(part.size()));
+        for (int s : part) {
+          const double n = h->hs[s].n;
+          const long long cap = std::min<long long>(h->hs[s].n / kTrdCols, sms);
+          G[s] = caps <= budget ? static_cast<int>(cap)
+                                : static_cast<int>(std::min(cap, 1 + static_cast<long long>(spare * (n * n * n / wsum))));
+        }
       }
     };
     auto smem_of = [&](int in_smem) {
@@ -849,6 +852,25 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
       if (ctas > sms || trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 512) < 1) h->trd_plan.threads = 256;
     }
     if (h->trd_plan.threads == 256) {
+      // Where so many searches share the GPU that the large ones get a CTA or two, a few
+      // CTAs would still be at those when the rest has finished. Then launches of at most
+      // an eighth as many searches as there are CTAs follow one another, largest
+      // searches first: together they keep every SM busy to the end. (256 searches of
+      // n = 50 .. 2000: 3453 ms in one launch, 572 in several. Searches small enough
+      // that a step's exchange takes longer than its CTA's columns stay in one.)
+      share(2 * sms);
+      double most = 0.0;
+      for (int s : parts[0]) most = std::max(most, static_cast<double>(h->hs[s].n) * h->hs[s].n / G[s]);
+      if (nact > static_cast<size_t>(sms) / 2 && most > 65536.0) {
+        std::vector<int> order = parts[0];
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return h->hs[x].n > h->hs[y].n; });
+        parts.clear();
+        const size_t each = std::max<size_t>(1, static_cast<size_t>(sms) / 4);
+        for (size_t i = 0; i < order.size(); i += each)
+          parts.emplace_back(order.begin() + i, order.begin() + std::min(order.size(), i + each));
+        share(2 * sms);
+        h->trd_plan.smem = smem_of(0);
+      }
       // (the accumulators' size depends on the shares)
       int per_sm = trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 256);
       for (int pass = 0; pass < 2; ++pass) {
@@ -866,16 +888,19 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     std::vector<int4> grp;  // launches of at most `budget` CTAs never split a group
     h->trd_chunks.clear();
     int chunk_start = 0;
-    for (int s = 0; s < count; ++s) {
-      if (!h->hs[s].trd) continue;
-      const int Gs = static_cast<int>(std::min<long long>(G[s], budget));
-      if (static_cast<long long>(grp.size()) + Gs - chunk_start > budget) {
+    auto close = [&] {
+      if (static_cast<int>(grp.size()) > chunk_start)
         h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start});
-        chunk_start = static_cast<int>(grp.size());
+      chunk_start = static_cast<int>(grp.size());
+    };
+    for (const std::vector<int>& part : parts) {
+      for (int s : part) {
+        const int Gs = static_cast<int>(std::min<long long>(G[s], budget));
+        if (static_cast<long long>(grp.size()) + Gs - chunk_start > budget) close();
+        for (int r = 0; r < Gs; ++r) grp.push_back(make_int4(s, r, Gs, 0));
       }
-      for (int r = 0; r < Gs; ++r) grp.push_back(make_int4(s, r, Gs, 0));
+      close();
     }
-    h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start});
     h->trd_grp_blocks = static_cast<int>(grp.size());
     long long eig_total = 0;
     for (int s = 0; s < count; ++s)
