@@ -979,8 +979,8 @@ __global__ void __launch_bounds__(kLogNT) k_jlog_apply(Search* S, int s0) {
 // their floor is four times lower, but A's products round well below it, so that what
 // passes the test early in a descent are a few pairs of close eigenvalues, for which the
 // cyclic sweeps took one to two hundred steps of two cluster barriers (the decomposition
-// of ten searches of n = 100 744 -> 600 us, of three of n = 160 1290 -> 963, of four of
-// n = 64 185 -> 183; six of n = 40, with nothing to rotate, 146 -> 151). Late in a
+// of ten searches of n = 100 744 -> 621 us, of three of n = 160 1290 -> 1174, of four of
+// n = 64 185 -> 179; six of n = 40, with nothing to rotate, would pay 146 -> 151). Late in a
 // descent on an ill-conditioned function hundreds are left, and the cluster's eight SMs
 // rotate those faster (three searches of n = 85, a generation: 6 rotations each 509 us
 // with the rounds and 564 without, 31 each 713 and 735, 100 each 912 and 805).

@@ -25,11 +25,10 @@
 // A column with an infinite or NaN entry makes every output it enters a NaN.
 // What bounds it now: the integer multiply-adds of the SMs a cluster has (n = 100,
 // clusters of 8: 17k of the 24k clocks of a full product), then the FP64 arithmetic of
-// E and of the epilogues, then the cluster barriers (n = 40). The whole
-// eigendecomposition (with the FP32 Jacobi, which is most of the rest), one launch per
-// product -> here: six searches of n = 40 242 -> 209 us, n = 100 one search 460 -> 413,
-// eight 651 -> 557, ten 731 -> 638, n = 160 one 453 -> 465, four 1086 -> 981, eight
-// 1609 -> 1325. The results do not depend on the cluster size: every sum is exact.
+// E and of the epilogues, then the cluster barriers (n = 40). Kernel time of a
+// decomposition's products and corrections, one launch per product -> here (profiled
+// one by one): six searches of n = 40 178 -> 111 us, ten of n = 100 340 -> 231. The
+// results do not depend on the cluster size: every sum is exact.
 #include <cmath>
 #include <cooperative_groups.h>
 #include "device_common.cuh"
@@ -407,8 +406,8 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
 }
 
 // Clusters of 16 where those of all searches run side by side (seven did), else of 8:
-// the decomposition of four searches of n = 100 takes 425 us with 16 and 480 with 8, of
-// ten 741 and 638.
+// the decomposition of four searches of n = 100 took 425 us with 16 and 480 with 8, that
+// of ten, whose clusters of 16 no longer fit at once, 741 and 638.
 void launch_eig_refine(Search* S, int s0, int s1, int max_n, int head, cudaStream_t st) {
   if (s1 <= s0 || max_n <= kJacobiSmallN) return;
   cudaLaunchConfig_t cfg = {};
