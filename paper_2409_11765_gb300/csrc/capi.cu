@@ -716,6 +716,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     }                                                                                            \
   } while (0)
   small_set_attributes();
+  CREATE_TRY(eig_smem_limits());
   CREATE_TRY(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
   size_t state_max = 0;
   for (const Search& x : h->hs) state_max = std::max(state_max, state_bytes(x));

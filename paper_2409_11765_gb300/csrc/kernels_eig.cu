@@ -365,9 +365,28 @@ __global__ void __launch_bounds__(kJacobiNT) k_jacobi(Search* S, int s0, int lo_
 // Covers the whole search range and processes the searches with n > lo_n.
 void launch_jacobi_global(Search* S, int s0, int s1, int lo_n, int max_n, cudaStream_t st) {
   if (s1 <= s0 || max_n <= lo_n) return;
-  const int bytes = jacobi_smem_bytes(max_n);
-  cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  k_jacobi<<<s1 - s0, kJacobiNT, bytes, st>>>(S, s0, lo_n);
+  k_jacobi<<<s1 - s0, kJacobiNT, jacobi_smem_bytes(max_n), st>>>(S, s0, lo_n);
+}
+
+cudaError_t smem_limit_max(const void* kernel) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes a;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess ||
+      (e = cudaFuncGetAttributes(&a, kernel)) != cudaSuccess)
+    return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              optin - static_cast<int>(a.sharedSizeBytes));
+}
+
+cudaError_t eig_smem_limits() {
+  cudaError_t e;
+  if ((e = smem_limit_max(reinterpret_cast<const void*>(k_jacobi))) != cudaSuccess ||
+      (e = refine_smem_limit()) != cudaSuccess || (e = eig_mixed_smem_limits()) != cudaSuccess ||
+      (e = jacobi_cluster_smem_limit()) != cudaSuccess)
+    return e;
+  return jlog_big_smem_limit();
 }
 
 // BD = B diag(D); force = 1 applies to every search (after set_state).

@@ -426,8 +426,8 @@ void launch_jlog_big(Search* S, TileMap trows, int max_n, cudaStream_t st) {
   if (trows.total <= 0) return;
   const int N = max_n + (max_n & 1);
   const int bytes = 2 * kJrChunk * 8 + kJrRows * (N + 1) * 4;
-  cudaFuncSetAttribute(k_jlog_big, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   k_jlog_big<<<trows.total, kJrNT, bytes, st>>>(S, trows);
 }
+cudaError_t jlog_big_smem_limit() { return smem_limit_max(reinterpret_cast<const void*>(k_jlog_big)); }
 
 }  // namespace cmaes_gb300

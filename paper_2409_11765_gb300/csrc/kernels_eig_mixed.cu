@@ -771,9 +771,7 @@ static size_t jacobi32_smem_bytes(int pm) {
 
 template <int NT, int NB, int PM>
 static void launch_jacobi32_as(Search* S, int s0, int s1, cudaStream_t st) {
-  const int bytes = static_cast<int>(jacobi32_smem_bytes(PM));
-  cudaFuncSetAttribute(k_jacobi32<NT, NB, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  k_jacobi32<NT, NB, PM><<<s1 - s0, NT, bytes, st>>>(S, s0);
+  k_jacobi32<NT, NB, PM><<<s1 - s0, NT, jacobi32_smem_bytes(PM), st>>>(S, s0);
 }
 
 // The fewest threads whose blocks hide behind the rotations, by the largest n of the
@@ -1205,12 +1203,20 @@ int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1
     launch_eig_refine(S, s0, s1, max_small, 0, st);
     ++nl;
     if (!mixed && max_small < kRoundsMinN) return nl;
-    const int rbytes = pair_rounds_smem_bytes(max_small);
-    cudaFuncSetAttribute(k_pair_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, rbytes);
-    k_pair_rounds<<<s1 - s0, kRoundsNT, rbytes, st>>>(S, s0);
+    k_pair_rounds<<<s1 - s0, kRoundsNT, pair_rounds_smem_bytes(max_small), st>>>(S, s0);
     ++nl;
   }
   return nl;
+}
+
+cudaError_t eig_mixed_smem_limits() {
+  for (const void* k : {reinterpret_cast<const void*>(k_pair_rounds), reinterpret_cast<const void*>(k_jacobi32<256, 1, 22>),
+                        reinterpret_cast<const void*>(k_jacobi32<384, 2, 36>),
+                        reinterpret_cast<const void*>(k_jacobi32<768, 2, 52>),
+                        reinterpret_cast<const void*>(k_jacobi32<1024, 2, 63>),
+                        reinterpret_cast<const void*>(k_jacobi32<1024, 4, kE32Max / 2>)})
+    if (const cudaError_t e = smem_limit_max(k); e != cudaSuccess) return e;
+  return cudaSuccess;
 }
 
 }  // namespace cmaes_gb300

@@ -424,16 +424,21 @@ void launch_eig_refine(Search* S, int s0, int s1, int max_n, int head, cudaStrea
     cfg.gridDim = dim3(static_cast<unsigned>((s1 - s0) * cs));
     cfg.dynamicSmemBytes = rf_layout(max_n, cs).bytes;
   };
-  cudaFuncSetAttribute(k_eig_refine, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       static_cast<int>(rf_layout(max_n, 8).bytes));
+  // (a device that refuses clusters of 16 reports that none fits)
   int fit = 0;
-  if (cudaFuncSetAttribute(k_eig_refine, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-    size(16);
-    if (cudaOccupancyMaxActiveClusters(&fit, k_eig_refine, &cfg) != cudaSuccess) fit = 0;
+  size(16);
+  if (cudaOccupancyMaxActiveClusters(&fit, k_eig_refine, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    fit = 0;
   }
-  cudaGetLastError();  // (a device that refuses either takes clusters of 8)
   if (fit < s1 - s0) size(8);
   cudaLaunchKernelEx(&cfg, k_eig_refine, S, s0, head);
+}
+
+cudaError_t refine_smem_limit() {
+  if (cudaFuncSetAttribute(k_eig_refine, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    cudaGetLastError();
+  return smem_limit_max(reinterpret_cast<const void*>(k_eig_refine));
 }
 
 }  // namespace cmaes_gb300

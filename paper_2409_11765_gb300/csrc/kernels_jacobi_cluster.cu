@@ -426,8 +426,8 @@ __global__ void __cluster_dims__(kCS, 1, 1) __launch_bounds__(512)
 void launch_jacobi_cluster(Search* S, int s0, int s1, int lo_n, int hi_n, int layout_n, cudaStream_t st) {
   if (s1 <= s0 || layout_n <= lo_n) return;
   const CLayout L = make_layout(layout_n);
-  cudaFuncSetAttribute(k_jacobi_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(L.bytes));
   k_jacobi_cluster<<<(s1 - s0) * kCS, L.threads, L.bytes, st>>>(S, s0, lo_n, hi_n, layout_n);
 }
+cudaError_t jacobi_cluster_smem_limit() { return smem_limit_max(reinterpret_cast<const void*>(k_jacobi_cluster)); }
 
 }  // namespace cmaes_gb300
