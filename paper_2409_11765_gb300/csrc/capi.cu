@@ -711,8 +711,10 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
   do {                                                                                           \
     cudaError_t e_ = (call);                                                                     \
     if (e_ != cudaSuccess) {                                                                     \
-      set_error(h, CMAES_ECUDA, "%s failed: %s", #call, cudaGetErrorString(e_));                \
-      return fail(CMAES_ECUDA);                                                                  \
+      cudaGetLastError();                                                                        \
+      const cmaes_status r_ = e_ == cudaErrorMemoryAllocation ? CMAES_ENOMEM : CMAES_ECUDA;      \
+      set_error(h, r_, "%s failed: %s", #call, cudaGetErrorString(e_));                         \
+      return fail(r_);                                                                           \
     }                                                                                            \
   } while (0)
   small_set_attributes();
