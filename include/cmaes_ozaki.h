@@ -25,9 +25,12 @@ extern "C" {
  * B: device pointer, K x N, column-major, ldb >= K.
  * C: device pointer, M x N, column-major, ldc >= M; read only if beta != 0.
  * stream: a cudaStream_t (NULL = the legacy default stream).
- * The caller owns all three arrays. The call allocates and frees its own
- * workspace (about 14 bytes per element of A and B) and returns after the
- * product is complete.
+ * The caller owns all three arrays. The call takes a workspace of
+ * about 14 bytes per element of A and B and returns after the product is
+ * complete. Workspaces up to 64 MiB come from a memory pool of the library's
+ * own, which keeps at most 64 MiB per context between calls and ends with the
+ * context (the call works again after cudaDeviceReset); larger ones are
+ * allocated and freed by the call.
  *
  * Accuracy: with 2^a the power of two bounding row i of A (2^a < 2 x its
  * largest magnitude) and 2^b the one bounding column j of B, every entry is
@@ -38,7 +41,9 @@ extern "C" {
  * count as zero.
  *
  * Returns 0 on success, 1 on a bad argument, 2 if the workspace cannot be
- * allocated, 3 on a CUDA error, 4 if a device wait ran out (about 1 s). */
+ * allocated or the stream is being captured (the call synchronises, so a
+ * graph cannot hold it; the capture goes on), 3 on a CUDA error, 4 if a device
+ * wait ran out (about 1 s). */
 int cmaes_ozaki_dgemm(int M, int N, int K, double alpha, const double* A, long long lda,
                       const double* B, long long ldb, double beta, double* C, long long ldc,
                       void* stream);

@@ -123,38 +123,66 @@ using namespace cmaes_gb300;
 // Workspace up to kOzKeep from a stream-ordered pool of the engine's own, so that a call
 // neither maps nor unmaps memory: cudaMalloc and cudaFree take up to 150 us of a call
 // (500 x 500 x 500: 251 us with them, 112 from the pool) and synchronise the device. The
-// pool keeps at most kOzKeep bytes per device between calls; what several threads took
+// pool keeps at most kOzKeep bytes per context between calls; what several threads took
 // beyond that goes back at the next synchronisation, and an allocation that fails gives
 // everything back first. Pools are safe from every thread and stream. A larger
 // workspace, or one where there is no pool, is cudaMalloc's: the pool would map and
 // unmap it on every call (3000 x 3000 x 3000: 2630 us, 2870 from the pool).
+// A pool ends with its context (cudaDeviceReset), and a context's number is never given
+// twice, so a pool is kept under the number of the context that made it; a number that
+// does not come again costs its entry, and beyond kOzMaxPools there is no pool.
 namespace {
 constexpr uint64_t kOzKeep = 64ull << 20;
-constexpr int kOzMaxDevices = 64;
+constexpr int kOzMaxPools = 64;
+struct OzPool {
+  unsigned long long context;
+  cudaMemPool_t pool;
+};
 std::mutex g_oz_mutex;
-cudaMemPool_t g_oz_pool[kOzMaxDevices] = {nullptr};
+OzPool g_oz_pool[kOzMaxPools];
+int g_oz_pools = 0;
 
-cudaMemPool_t oz_pool() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kOzMaxDevices) return nullptr;
-  std::lock_guard<std::mutex> lock(g_oz_mutex);
-  if (!g_oz_pool[dev]) {
-    int ok = 0;
-    if (cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, dev) != cudaSuccess || !ok) return nullptr;
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    uint64_t keep = kOzKeep;
-    cudaMemPool_t p = nullptr;
-    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
-    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-      cudaMemPoolDestroy(p);
-      return nullptr;
+// The current context's number (0: not to be had); the runtime API does not give it.
+unsigned long long context_number() {
+  using Fn = int (*)(void*, unsigned long long*);  // cuCtxGetId
+  static const Fn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      p = nullptr;
     }
-    g_oz_pool[dev] = p;
+    return reinterpret_cast<Fn>(p);
+  }();
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == 0 ? id : 0;
+}
+
+// (called with a current context: the call has asked for its stream's state)
+cudaMemPool_t oz_pool() {
+  const unsigned long long id = context_number();
+  if (id == 0) return nullptr;
+  std::lock_guard<std::mutex> lock(g_oz_mutex);
+  for (int i = 0; i < g_oz_pools; ++i)
+    if (g_oz_pool[i].context == id) return g_oz_pool[i].pool;
+  int dev = 0, ok = 0;
+  if (g_oz_pools == kOzMaxPools || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, dev) != cudaSuccess || !ok)
+    return nullptr;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  uint64_t keep = kOzKeep;
+  cudaMemPool_t p = nullptr;
+  if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
+  if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaMemPoolDestroy(p);
+    return nullptr;
   }
-  return g_oz_pool[dev];
+  g_oz_pool[g_oz_pools++] = OzPool{id, p};
+  return p;
 }
 
 struct OzWorkspace {
