@@ -158,10 +158,13 @@ __global__ void __launch_bounds__(kTrdNT) k_trd_blocks(Search* S, int s0) {
 }
 
 // --------------------------------------------------------------------------
-// 3. Multisection: a group of LANES lanes finds eigenvalue t - b0 (ascending)
-// of its block; each round the lanes take the Sturm counts at LANES interior
-// points of the bracket, which shrinks it (LANES + 1)-fold: fewer sequential
-// rounds for more counts in all.
+// 3. Bisection: a group of LANES lanes finds eigenvalue t - b0 (ascending) of its
+// block; each round the lanes take the Sturm counts at the LANES - 1 points (one
+// point where a lane is alone) of the next log2(LANES) halvings and then walk those
+// halvings on the counts: fewer sequential rounds for more counts in all. A
+// precision's points lie on one grid, its last halving's, so the walk meets the same
+// points and counts with any number of lanes: the number, which the whole handle
+// decides, does not show in the bits.
 //
 // A Sturm count is the number of sign changes of the leading minors of T - x I,
 //   p_j = (d_j - x) p_{j-1} - e_{j-1}^2 p_{j-2},
@@ -178,8 +181,8 @@ constexpr int kTrdTT = 32;
 int tiles_trd(int n) { return ceil_div(n, kTrdTT); }
 int tiles_trd_bis(int n, int lanes) { return ceil_div(n * lanes, kTrdTT); }
 
-// Lanes per eigenvalue by the number of eigenvalues of the handle's searches:
-// the rounds' latency against the counts' FP64 work (three operations of ~19
+// Lanes per eigenvalue (a power of two) by the number of eigenvalues of the handle's
+// searches: the rounds' latency against the counts' FP64 work (three operations of ~19
 // clocks per warp and row on each SM).
 int trd_bis_lanes(long long eigenvalues) {
   return eigenvalues <= 700 ? 16 : eigenvalues <= 2500 ? 8 : eigenvalues <= 7000 ? 4 : 1;
@@ -329,8 +332,7 @@ __device__ __forceinline__ int sturm_df(const float* __restrict__ dh, const floa
   return cnt;
 }
 
-// Eigenvalue t of its block by bisection (LANES = 1) or multisection with
-// LANES points per step, in three precisions, on the scaled copies: FP32 down to
+// Eigenvalue t of its block by bisection in three precisions on the scaled copies: FP32 down to
 // a width of 2^-19 ||T||, widened by 2^-18 ||T|| (eight times the backward
 // error of an FP32 Sturm count, ~10 eps32 ||T||); double-float down to
 // 2^-42 ||T||, widened by 2^-41 ||T|| (several times that of a double-float
@@ -369,16 +371,30 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
   const double fudge = 2.0 * kTrdEps * tn * (b1 - b0) + 0x1p-1000;
   double lo = -tn - fudge, hi = tn + fudge;
   const int idx = t - b0;
-  // one multisection step on [lo, hi] from the counts of the LANES points
-  auto narrow = [&](auto& lo_, auto& hi_, int cnt, auto w) -> bool {
-    const unsigned le = __ballot_sync(gmask, cnt <= idx) & gmask;
-    const int qlo = le ? (31 - __clz(le)) - base : -1;
-    const auto nlo = qlo >= 0 ? lo_ + w * (qlo + 1) : lo_;
-    const auto nhi = qlo + 1 < LANES ? lo_ + w * (qlo + 2) : hi_;
-    if (!(nlo < nhi) || (nlo == lo_ && nhi == hi_)) return false;
-    lo_ = nlo;
-    hi_ = nhi;
-    return true;
+  // halves [lo_, hi_] to a width of at most tol; cnt(x): the Sturm count at x
+  auto halve = [&](auto& lo_, auto& hi_, auto tol, auto cnt) {
+    using V = std::remove_reference_t<decltype(lo_)>;
+    constexpr int kBits = LANES == 1 ? 1 : LANES == 4 ? 2 : LANES == 8 ? 3 : 4;
+    const V width = hi_ - lo_;
+    if (!(width > tol) || !(tol > V(0))) return;
+    int left = ilogb(width) - ilogb(tol) + 1;  // halvings: at most 54
+    if (ldexp(width, 1 - left) <= tol) --left;
+    const V w = ldexp(width, -left);  // the grid's spacing
+    long long at = 0;                 // the bracket's left end on the grid
+    while (left > 0) {
+      const int b = min(kBits, left);
+      left -= b;
+      const long long p = min(q + 1, (1 << b) - 1);
+      const int c = cnt(fma(w, static_cast<V>(at + (p << left)), lo_));
+      const unsigned le = (__ballot_sync(gmask, c <= idx) & gmask) >> base;
+      int pos = 0;
+#pragma unroll
+      for (int h = kBits - 1; h >= 0; --h)
+        if (h < b && (le >> (pos + (1 << h) - 1) & 1u)) pos += 1 << h;
+      at += static_cast<long long>(pos) << left;
+    }
+    hi_ = fma(w, static_cast<V>(at + 1), lo_);
+    lo_ = fma(w, static_cast<V>(at), lo_);
   };
   // the two ends of a candidate bracket checked by the counts `cnt` (lane 0
   // the left end, lane 1 the right one; one lane does both)
@@ -392,10 +408,7 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
     const long long L2 = s.ldn;
     // FP32
     float lo32 = static_cast<float>(lo), hi32 = static_cast<float>(hi);
-    for (int it = 0; it < 40 && hi32 - lo32 > 0x1p-19f; ++it) {
-      const float w = (hi32 - lo32) / (LANES + 1);
-      if (!narrow(lo32, hi32, sturm32(d32, e32, b0, b1, lo32 + w * (q + 1)), w)) break;
-    }
+    halve(lo32, hi32, 0x1p-19f, [&](float x) { return sturm32(d32, e32, b0, b1, x); });
     auto cnt_df = [&](double xs) {
       const float xh = static_cast<float>(xs);
       return sturm_df(d32, d32 + L2, e32, e32 + L2, b0, b1, xh, static_cast<float>(xs - static_cast<double>(xh)));
@@ -409,20 +422,14 @@ __global__ void __launch_bounds__(kTrdTT) k_trd_bisect(Search* S, TileMap tm) {
       }
     }
     // double-float
-    for (int it = 0; it < 60 && his - los > 0x1p-42; ++it) {
-      const double w = (his - los) * (1.0 / (LANES + 1));
-      if (!narrow(los, his, cnt_df(los + w * (q + 1)), w)) break;
-    }
+    halve(los, his, 0x1p-42, cnt_df);
     const double lo2 = fmax(lo, los - 0x1p-41), hi2 = fmin(hi, his + 0x1p-41);
     if (lo2 < hi2 && check([&](double x) { return sturm64(d, e2, b0, b1, x); }, lo2, hi2)) {
       lo = lo2;
       hi = hi2;
     }
   }
-  for (int it = 0; it < 160 && hi - lo > atol; ++it) {
-    const double w = (hi - lo) * (1.0 / (LANES + 1));
-    if (!narrow(lo, hi, sturm64(d, e2, b0, b1, lo + w * (q + 1)), w)) break;
-  }
+  halve(lo, hi, atol, [&](double x) { return sturm64(d, e2, b0, b1, x); });
   if (q == 0) lamb[t] = 0.5 * (lo + hi) / scl;
 }
 
