@@ -148,21 +148,46 @@ __device__ __forceinline__ int block_or(int v, int* sh) {
 // h l + l h are summed exactly (below 2^61 and 2^62 over 32 k), and the step's
 // sum, to within 2^-57 of the two scales, is added to the FP64 accumulator: three
 // integer multiply-adds per term instead of one FP64 FMA, two FP64 operations per
-// output and step. An entry is off by 2^-58 of its row's largest and a step's sum
-// is rounded once, where 32 FP64 FMAs round 32 partial sums: against 113-bit
-// arithmetic the objectives come out 1.2 to 3 times closer than with FMAs (n = 100,
-// rastrigin: 1.1e-16 rms, was 2.3e-16; n = 1000: 7.8e-17, was 2.5e-16). A step with
-// an infinite or NaN entry is summed in FP64. (The rotation of 17391 points,
-// n = 100: 462 -> 179 us; its integer multiply-adds alone, tile padding included,
-// take ~80.)
+// output and step.
+//
+// The step's error, ~2^-57 of the product of the scales (rms), is small against
+// sum |a b| only where large entries of the row meet large ones of the column; an
+// axis-aligned rotation, or a row graded over many orders, has outputs where they
+// do not. So sum |a b| is also formed to 8 bits a factor (eight dp4a per output and
+// step), and an output where it is below 2^-4 of the scales' product, so that the
+// error could pass an FP64 rounding of sum |a b|, takes the step's FMAs in FP64 from
+// the entries themselves; so does one whose row or column has an infinite or NaN
+// entry or scales near the ends of the exponent range. No output depends on which
+// others share its tile. Rotated and evenly scaled operands have no such output:
+// against 113-bit arithmetic the objectives come out 1.2 to 3 times closer than with
+// FMAs (n = 100, rastrigin: 1.1e-16 rms, was 2.3e-16; n = 1000: 7.8e-17, was
+// 2.5e-16). The steps split K evenly: a last step of a few k would meet them by chance.
+// Bound by the integer multiply-adds and, beside them, by staging, which two CTAs per
+// SM overlap (128 registers; one of 172: 166 us). Evaluating 8704 points of n = 100:
+// 305 us in FP64 FMAs, 143 here (its multiply-adds alone, tile padding included, take
+// ~40), 270 if every output were to go to FP64.
 // ---------------------------------------------------------------------------
-constexpr int kGBM = 64, kGBN = 64, kGBK = 32, kGNT = 256;
+constexpr int kGBM = 64, kGBN = 64, kGBK = 32, kGNT = 256, kGPerSM = 2;
 
 struct GemmSmem {
   int2 As[kGBK][kGBM + 1];  // limbs (h, l), or the doubles themselves
   int2 Bs[kGBK][kGBN + 1];
+  unsigned ma[kGBK / 4][kGBM + 1];  // the entries' magnitudes to 8 bits, four k a word
+  unsigned mb[kGBK / 4][kGBN + 1];
   int ea[kGBM], eb[kGBN];
 };
+
+// k per step: K split evenly into as few steps as there can be.
+__host__ __device__ inline int gemm_step(int K) {
+  const int steps = (K + kGBK - 1) / kGBK;
+  return steps > 0 ? (K + steps - 1) / steps : kGBK;
+}
+
+// The biased exponent of x for the scales (1 for a subnormal number).
+__device__ __forceinline__ int gemm_exponent(double x) {
+  const int hi = __double2hiint(x), be = (hi >> 20) & 0x7ff;
+  return be | static_cast<int>(be == 0 && ((hi << 1) | __double2loint(x)) != 0);
+}
 
 // The limbs of x for a scale with biased exponent E (|x| < 2^(E - 1022)): x rounded
 // to 2 H - 1 bits of it, x = (h 2^H + l) 2^(E - 1022 - (2 H - 1)), |h|, |l| <= 2^(H - 1).
@@ -177,6 +202,17 @@ __device__ __forceinline__ int2 gemm_limbs(double x, int E) {
   if (hi < 0) m = -m;
   const int h = static_cast<int>((m + (1LL << (H - 1))) >> H);
   return make_int2(h, static_cast<int>(m - (static_cast<long long>(h) << H)));
+}
+
+// 8 bits of the magnitude of an entry with limb h (of gemm_limbs<29>), 2^-8 of the
+// scale each.
+__device__ __forceinline__ unsigned gemm_byte(int h) { return min(static_cast<unsigned>(abs(h)) >> 20, 255u); }
+
+// Whether a step's output goes to FP64: `sum` is the dot product of those bytes, ea and
+// eb the scales' biased exponents (0: only zeros there).
+__device__ __forceinline__ bool gemm_in_f64(unsigned sum, int ea, int eb) {
+  constexpr unsigned kLeast = 1u << 12;  // 2^-4 of the scales' product
+  return ea != 0 && eb != 0 && (sum < kLeast || min(ea, eb) < 64 || max(ea, eb) == 0x7ff);
 }
 
 // The value of sum (h h) + sum (h l + l h) / 2^H over two operands of that form
@@ -208,29 +244,32 @@ __device__ __forceinline__ void gemm_tile_f64(int M, int N, int K, int i0, int j
   auto ak = [&](int q) { return A_I_CONTIG ? (tid >> 6) + 4 * q : (tid & 31); };
   auto bj = [&](int q) { return B_K_CONTIG ? (tid >> 5) + 8 * q : (tid & 63); };
   auto bk = [&](int q) { return B_K_CONTIG ? (tid & 31) : (tid >> 6) + 4 * q; };
-  for (int k0 = 0; k0 < K; k0 += kGBK) {
+  const int step = gemm_step(K);
+  for (int k0 = 0; k0 < K; k0 += step) {
+    const int kn = min(step, K - k0);
     double av[Q], bv[Q];
+    auto load = [&] {
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int gi = i0 + ai(q), gk = k0 + ak(q);
-      av[q] = (gi < M && gk < K) ? la(gi, gk) : 0.0;
-    }
+      for (int q = 0; q < Q; ++q) {
+        const int gi = i0 + ai(q), k = ak(q);
+        av[q] = (gi < M && k < kn) ? la(gi, k0 + k) : 0.0;
+      }
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int gk = k0 + bk(q), gj = j0 + bj(q);
-      bv[q] = (gk < K && gj < N) ? lb(gk, gj) : 0.0;
-    }
+      for (int q = 0; q < Q; ++q) {
+        const int k = bk(q), gj = j0 + bj(q);
+        bv[q] = (k < kn && gj < N) ? lb(k0 + k, gj) : 0.0;
+      }
+    };
+    load();
     if (tid < kGBM) sm.ea[tid] = 0;
     else if (tid < kGBM + kGBN) sm.eb[tid - kGBM] = 0;
     __syncthreads();
     // scales: the largest biased exponent of every row of A and column of B
-    int special = 0;
     auto scale = [&](const double (&v)[Q], bool column_per_warp, int* e, auto index) {
       int mx = 0;
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        const int be = (__double2hiint(v[q]) >> 20) & 0x7ff;
-        special |= be == 0x7ff;
+        const int be = gemm_exponent(v[q]);
         if (column_per_warp) {
           const int m = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(be)));
           if ((tid & 31) == 0) e[index(q)] = m;
@@ -242,35 +281,42 @@ __device__ __forceinline__ void gemm_tile_f64(int M, int N, int K, int i0, int j
     };
     scale(av, !A_I_CONTIG, sm.ea, ai);
     scale(bv, B_K_CONTIG, sm.eb, bj);
-    if (__syncthreads_or(special)) {
+    __syncthreads();
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        *reinterpret_cast<double*>(&sm.As[ak(q)][ai(q)]) = av[q];
-        *reinterpret_cast<double*>(&sm.Bs[bk(q)][bj(q)]) = bv[q];
-      }
-      __syncthreads();
-      for (int kk = 0; kk < min(kGBK, K - k0); ++kk)
+    for (int q = 0; q < Q; ++q) {
+      const int2 a = gemm_limbs<29>(av[q], sm.ea[ai(q)]), b = gemm_limbs<29>(bv[q], sm.eb[bj(q)]);
+      sm.As[ak(q)][ai(q)] = a;
+      sm.Bs[bk(q)][bj(q)] = b;
+      reinterpret_cast<unsigned char*>(&sm.ma[ak(q) >> 2][ai(q)])[ak(q) & 3] = static_cast<unsigned char>(gemm_byte(a.x));
+      reinterpret_cast<unsigned char*>(&sm.mb[bk(q) >> 2][bj(q)])[bk(q) & 3] = static_cast<unsigned char>(gemm_byte(b.x));
+    }
+    __syncthreads();
+    unsigned f64 = 0;  // bit 4 r + c: this output's step is summed in FP64
+    {
+      unsigned sum[4][4] = {};
+#pragma unroll 2
+      for (int w = 0; w < kGBK / 4; ++w) {
+        unsigned a[4], b[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) a[r] = sm.ma[w][tr + 16 * r];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) b[c] = sm.mb[w][tc + 16 * c];
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            acc[r][c] = fma(*reinterpret_cast<const double*>(&sm.As[kk][tr + 16 * r]),
-                            *reinterpret_cast<const double*>(&sm.Bs[kk][tc + 16 * c]), acc[r][c]);
-      __syncthreads();
-      continue;
-    }
+          for (int c = 0; c < 4; ++c) sum[r][c] = __dp4a(a[r], b[c], sum[r][c]);
+      }
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      sm.As[ak(q)][ai(q)] = gemm_limbs<29>(av[q], sm.ea[ai(q)]);
-      sm.Bs[bk(q)][bj(q)] = gemm_limbs<29>(bv[q], sm.eb[bj(q)]);
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          f64 |= static_cast<unsigned>(gemm_in_f64(sum[r][c], sm.ea[tr + 16 * r], sm.eb[tc + 16 * c])) << (4 * r + c);
     }
-    __syncthreads();
     long long hh[4][4], mid[4][4];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int c = 0; c < 4; ++c) hh[r][c] = mid[r][c] = 0;
-    const int kn = min(kGBK, K - k0);
 #pragma unroll 2
     for (int kk = 0; kk < kn; ++kk) {
       int2 a[4], b[4];
@@ -291,7 +337,26 @@ __device__ __forceinline__ void gemm_tile_f64(int M, int N, int K, int i0, int j
     for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        acc[r][c] += gemm_scaled<29>(hh[r][c], mid[r][c], sm.ea[tr + 16 * r] + sm.eb[tc + 16 * c]);
+        if (!(f64 >> (4 * r + c) & 1u))
+          acc[r][c] += gemm_scaled<29>(hh[r][c], mid[r][c], sm.ea[tr + 16 * r] + sm.eb[tc + 16 * c]);
+    if (!__syncthreads_or(static_cast<int>(f64))) continue;
+    load();
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      *reinterpret_cast<double*>(&sm.As[ak(q)][ai(q)]) = av[q];
+      *reinterpret_cast<double*>(&sm.Bs[bk(q)][bj(q)]) = bv[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (!(f64 >> (4 * r + c) & 1u)) continue;
+#pragma unroll 4
+        for (int kk = 0; kk < kn; ++kk)
+          acc[r][c] = fma(*reinterpret_cast<const double*>(&sm.As[kk][tr + 16 * r]),
+                          *reinterpret_cast<const double*>(&sm.Bs[kk][tc + 16 * c]), acc[r][c]);
+      }
     __syncthreads();
   }
 #pragma unroll

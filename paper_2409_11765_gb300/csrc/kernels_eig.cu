@@ -47,7 +47,7 @@ int jacobi_smem_bytes(int n) {
 __device__ __forceinline__ bool mixed_route(const Search& s) { return s.n <= kEigBigMaxN; }
 
 // ET = C B (square tiles; only searches whose decomposition is due).
-__global__ void __launch_bounds__(256) k_eig_gemm_CB(Search* S, TileMap tm) {
+__global__ void __launch_bounds__(kGNT, kGPerSM) k_eig_gemm_CB(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(256) k_eig_gemm_CB(Search* S, TileMap tm) {
 }
 
 // EA = B^T ET = B^T C B.
-__global__ void __launch_bounds__(256) k_eig_gemm_BtT(Search* S, TileMap tm) {
+__global__ void __launch_bounds__(kGNT, kGPerSM) k_eig_gemm_BtT(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);

@@ -124,7 +124,7 @@ void launch_sample_z(Search* S, TileMap tm, DevOptions o, cudaStream_t st) {
 }
 
 // Eq. (1) for all candidates (§3.1): Y = (B diag(D)) Z, X = m 1^T + sigma Y.
-__global__ void __launch_bounds__(256) k_gemm_sample(Search* S, TileMap tm) {
+__global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_sample(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -158,7 +158,7 @@ void launch_gemm_sample(Search* S, TileMap tm, cudaStream_t st) {
 
 // ------------------------------- objective ----------------------------------
 // Rotated objectives: U = Q (X - x*), with x - x* formed in FP64.
-__global__ void __launch_bounds__(256) k_gemm_objective(Search* S, TileMap tm) {
+__global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_objective(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -470,7 +470,7 @@ __device__ __forceinline__ void sym_tile(int t, int n, int& ti, int& tj) {
   tj = ti + rem;
 }
 
-__global__ void __launch_bounds__(256) k_cov_partial(Search* S, TileMap tm) {
+__global__ void __launch_bounds__(kGNT, kGPerSM) k_cov_partial(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);

@@ -28,7 +28,7 @@ __device__ __align__(256) double g_eval_scratch[kEvalScratchDoubles];
 constexpr int kMaxDevices = 64;
 double* g_scratch_addr[kMaxDevices] = {nullptr};
 
-__global__ void __launch_bounds__(256) k_noalloc_rotate(int n, int lam, int ld, const double* X,
+__global__ void __launch_bounds__(kGNT, kGPerSM) k_noalloc_rotate(int n, int lam, int ld, const double* X,
                                                         const double* Q, int ldq,
                                                         const double* xstar, double* U) {
   __shared__ GemmSmem sm;
