@@ -199,7 +199,7 @@ constexpr int kSmallPanel = 2048;
 void launch_small_eig(Search* S, int s0, int s1, int max_n, cudaStream_t st);
 bool small_generation(int n, int lam_cap);
 size_t small_generation_smem(int n, int lam_cap);
-void small_set_attributes();
+cudaError_t small_smem_limits();
 void launch_small_generations(Search* S, int count, DevOptions o, int gens, size_t smem, cudaStream_t st);
 void launch_jacobi_cluster(Search* S, int s0, int s1, int lo_n, int hi_n, int layout_n, cudaStream_t st);
 void launch_set_bd(Search* S, TileMap tm, cudaStream_t st);
@@ -207,11 +207,14 @@ void launch_set_bd(Search* S, TileMap tm, cudaStream_t st);
 // that the device gives the kernel, when a handle is created, and never to a handle's
 // own need, which a launch of another thread's handle could still be above.
 cudaError_t smem_limit_max(const void* kernel);
-cudaError_t eig_smem_limits();         // kernels_eig.cu, which calls the others
+cudaError_t set_smem_limits();         // all of them, once per context (capi.cu)
+unsigned long long context_number();   // the current context's (0: not to be had), never given twice
+cudaError_t eig_smem_limits();         // kernels_eig.cu, which calls the next four
 cudaError_t refine_smem_limit();       // kernels_eig_refine.cu
 cudaError_t eig_mixed_smem_limits();   // kernels_eig_mixed.cu
 cudaError_t jacobi_cluster_smem_limit();
 cudaError_t jlog_big_smem_limit();
+cudaError_t tc_smem_limits();          // kernels_mixed.cu
 void launch_set_bd_force(Search* S, TileMap tm, cudaStream_t st);
 int jacobi_smem_bytes(int n);
 

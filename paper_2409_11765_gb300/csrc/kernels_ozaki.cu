@@ -142,23 +142,6 @@ std::mutex g_oz_mutex;
 OzPool g_oz_pool[kOzMaxPools];
 int g_oz_pools = 0;
 
-// The current context's number (0: not to be had); the runtime API does not give it.
-unsigned long long context_number() {
-  using Fn = int (*)(void*, unsigned long long*);  // cuCtxGetId
-  static const Fn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult r;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &r) != cudaSuccess ||
-        r != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      p = nullptr;
-    }
-    return reinterpret_cast<Fn>(p);
-  }();
-  unsigned long long id = 0;
-  return fn && fn(nullptr, &id) == 0 ? id : 0;
-}
-
 // (called with a current context: the call has asked for its stream's state)
 cudaMemPool_t oz_pool() {
   const unsigned long long id = context_number();

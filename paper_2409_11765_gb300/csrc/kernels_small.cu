@@ -835,10 +835,9 @@ bool small_generation(int n, int lam_cap) {
 
 size_t small_generation_smem(int n, int lam_cap) { return sm_gen_doubles(n, lam_cap) * sizeof(double); }
 
-void small_set_attributes() {
-  const int top = 200 * 1024;  // above any search's need; the attribute belongs to the process
-  cudaFuncSetAttribute(k_small_generations, cudaFuncAttributeMaxDynamicSharedMemorySize, top);
-  cudaFuncSetAttribute(k_small_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, top);
+cudaError_t small_smem_limits() {
+  const cudaError_t e = smem_limit_max(reinterpret_cast<const void*>(k_small_generations));
+  return e != cudaSuccess ? e : smem_limit_max(reinterpret_cast<const void*>(k_small_eig));
 }
 
 void launch_small_generations(Search* S, int count, DevOptions o, int gens, size_t smem, cudaStream_t st) {
