@@ -183,9 +183,14 @@ int tiles_trd_bis(int n, int lanes) { return ceil_div(n * lanes, kTrdTT); }
 
 // Lanes per eigenvalue (a power of two) by the number of eigenvalues of the handle's
 // searches: the rounds' latency against the counts' FP64 work (three operations of ~19
-// clocks per warp and row on each SM).
+// clocks per warp and row on each SM). The eigenvalue stage with 16 / 8 / 4 / 1 lanes, us:
+//   1000 (1 search) 1203 / 1459 / 2020 / 3915, 1800 (2) 1270 / 1332 / 1837 / 3534,
+//   2000 (8) 459 / 446 / 581 / 1097, 4000 (4) 2488 / 1873 / 2056 / 3910,
+//   5000 (20) 906 / 683 / 649 / 1099, 12000 (12) 5519 / 4023 / 3361 / 3968,
+//   14000 (4) 22277 / 15817 / 13249 / 13611, 15000 (15) 6893 / 4864 / 4252 / 4006,
+//   38000 (76) 7909 / 5228 / 4088 / 2829.
 int trd_bis_lanes(long long eigenvalues) {
-  return eigenvalues <= 700 ? 16 : eigenvalues <= 2500 ? 8 : eigenvalues <= 7000 ? 4 : 1;
+  return eigenvalues <= 1900 ? 16 : eigenvalues <= 4500 ? 8 : eigenvalues <= 14000 ? 4 : 1;
 }
 
 // Eigenvalues of block [b0, b1) below x; d and e2 the scaled copies (|d| <= 1).
