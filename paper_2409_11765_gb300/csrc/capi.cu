@@ -88,6 +88,7 @@ struct cmaes_s {
   bool any_plain_eig = false;  // a search above every other route (warm start B^T C B by k_eig_gemm_*)
   bool all_small = true;       // whole generations run in one CTA per search (FP64 handles of small searches)
   size_t small_smem = 0;
+  bool small_dense = false;    // more such searches than wide CTAs fit
   int max_n_refine = 0;        // largest n <= kEigMixedMaxN on the refined Jacobi route
   int max_n_big = 0;           // largest n of the searches whose FP32 Jacobi runs over many CTAs
   // tridiagonal route: largest n, the CTA -> (search, member, group size) table
@@ -752,6 +753,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     }                                                                                            \
   } while (0)
   CREATE_TRY(set_smem_limits());
+  if (h->all_small) CREATE_TRY(small_generations_dense(count, h->small_smem, &h->small_dense));
   CREATE_TRY(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
   size_t state_max = 0;
   for (const Search& x : h->hs) state_max = std::max(state_max, state_bytes(x));
@@ -1081,7 +1083,8 @@ cmaes_status cmaes_step_batch(cmaes_t h, int generations, void* stream) {
     // (with profiling on, the phases are timed: the phase kernels)
     constexpr int kPerLaunch = 1 << 10;  // bounds a launch's time
     for (int g = 0; g < generations; g += kPerLaunch) {
-      launch_small_generations(h->dS, h->count, h->dopt, std::min(kPerLaunch, generations - g), h->small_smem, st);
+      launch_small_generations(h->dS, h->count, h->dopt, std::min(kPerLaunch, generations - g), h->small_smem,
+                               h->small_dense, st);
       h->launches += 1;
     }
     cmaes_status r = launch_check(h, "small generations");

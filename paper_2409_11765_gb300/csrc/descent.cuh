@@ -105,6 +105,27 @@ __device__ void restart_descent(Search& s, const DevOptions& o, double* sh) {
   compute_params<NT>(s, o, sh);
 }
 
+// The formulas that the phase kernels, the one-CTA generations and the allocation-free
+// evaluation share, with the rounding of each operation written out: the same state
+// gives the same bits through any of them.
+__device__ __forceinline__ double objective_term(int obj, double lam, double u) {
+  return obj == 1 ? __dmul_rn(__dmul_rn(lam, u), u) : fma(u, u, __dmul_rn(-10.0, cospi(2.0 * u)));
+}
+// x = m + sigma y, also the mean's step
+__device__ __forceinline__ double step_from(double m, double sigma, double y) { return fma(sigma, y, m); }
+// (1 - c) p + coef v of the two paths
+__device__ __forceinline__ double path_step(double c, double p, double coef, double v) {
+  return fma(coef, v, __dmul_rn(1.0 - c, p));
+}
+// Eq. (2): the weight of the old C, and an entry of the new one
+__device__ __forceinline__ double cov_keep(double c1, double cmu, double cc, double hsig) {
+  return fma(__dmul_rn(__dmul_rn(c1, 1.0 - hsig), cc), 2.0 - cc, 1.0 - c1 - cmu);
+}
+__device__ __forceinline__ double cov_entry(double keep, double c, double c1, double pi, double pj, double cmu,
+                                            double acc) {
+  return fma(cmu, acc, fma(__dmul_rn(c1, pi), pj, __dmul_rn(keep, c)));
+}
+
 // Order-preserving 64-bit integer key of f: NaN -> +inf, -0 -> +0, then the
 // IEEE bit pattern with the sign folded so that unsigned order = numeric order.
 // (Comparing integers keeps the O(lambda^2) count off GB300's slow FP64 pipe.)

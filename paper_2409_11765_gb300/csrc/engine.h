@@ -195,12 +195,13 @@ void launch_jacobi_global(Search* S, int s0, int s1, int lo_n, int max_n, cudaSt
 // small searches (kernels_small.cu): the eigendecomposition up to kJacobiSmallN,
 // and whole generations of FP64 searches with n lambda_cap <= kSmallPanel
 // (above it one CTA's FP64 pipe takes longer than the phase kernels' launches)
-constexpr int kSmallPanel = 2048;
+constexpr int kSmallPanel = 2048, kSmallLambda = 1024;
 void launch_small_eig(Search* S, int s0, int s1, int max_n, cudaStream_t st);
 bool small_generation(int n, int lam_cap);
 size_t small_generation_smem(int n, int lam_cap);
 cudaError_t small_smem_limits();
-void launch_small_generations(Search* S, int count, DevOptions o, int gens, size_t smem, cudaStream_t st);
+cudaError_t small_generations_dense(int count, size_t smem, bool* dense);
+void launch_small_generations(Search* S, int count, DevOptions o, int gens, size_t smem, bool dense, cudaStream_t st);
 void launch_jacobi_cluster(Search* S, int s0, int s1, int lo_n, int hi_n, int layout_n, cudaStream_t st);
 void launch_set_bd(Search* S, TileMap tm, cudaStream_t st);
 // A kernel's dynamic shared-memory limit belongs to the process: it is set to the most

@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_sample(Search* S, TileMa
       [=] __device__(int i, int j, double acc) {
         const long long e = i + static_cast<long long>(ldn) * j;
         Y[e] = acc;
-        X[e] = m[i] + sigma * acc;
+        X[e] = step_from(m[i], sigma, acc);
       },
       sm);
 }
@@ -203,10 +203,10 @@ __global__ void __launch_bounds__(256) k_colreduce_f(Search* S, TileMap tm) {
     }
   } else if (s.obj == 1) {
     const double* u = s.U + static_cast<long long>(ldn) * k;
-    for (int i = lane; i < n; i += 32) acc += s.lamdiag[i] * u[i] * u[i];
+    for (int i = lane; i < n; i += 32) acc += objective_term(1, s.lamdiag[i], u[i]);
   } else {
     const double* u = s.U + static_cast<long long>(ldn) * k;
-    for (int i = lane; i < n; i += 32) acc += u[i] * u[i] - 10.0 * cospi(2.0 * u[i]);
+    for (int i = lane; i < n; i += 32) acc += objective_term(2, 0.0, u[i]);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(256) k_psigma_final(Search* S, TileMap tm) {
   double v = 0.0;
   for (int ch = 0; ch < nch; ++ch) v += s.part[static_cast<long long>(ch) * s.ldn + i];
   const double coef = sqrt(s.cs * (2.0 - s.cs) * s.mueff);
-  s.ps[i] = (1.0 - s.cs) * s.ps[i] + coef * v;
+  s.ps[i] = path_step(s.cs, s.ps[i], coef, v);
 }
 
 void launch_psigma_partial(Search* S, TileMap tm, cudaStream_t st) {
@@ -404,8 +404,8 @@ __global__ void __launch_bounds__(256) k_finalize(Search* S, int s0) {
   const double sigma = s.sigma;
   for (int i = threadIdx.x; i < n; i += 256) {
     const double y = s.yw[i];
-    s.pc[i] = (1.0 - s.cc) * s.pc[i] + pc_coef * y;
-    s.m[i] = s.m[i] + sigma * y;
+    s.pc[i] = path_step(s.cc, s.pc[i], pc_coef, y);
+    s.m[i] = step_from(s.m[i], sigma, y);
   }
   const int i0 = s.order[0];
   double f0 = s.f[i0];
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_cov_partial(Search* S, TileMa
     double* C = s.C;
     const double* pc = s.pc;
     const double c1 = s.c1, cmu = s.cmu;
-    const double a = 1.0 - c1 - cmu + c1 * (1.0 - s.hsig) * s.cc * (2.0 - s.cc);
+    const double a = cov_keep(c1, cmu, s.cc, s.hsig);
     gemm_tile_f64<true, false>(
         n, n, k_hi - k_lo, ti * kGBM, tj * kGBN,
         [=] __device__(int i, int r) { return w[r] * Y[i + static_cast<long long>(ldn) * order[r]]; },
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_cov_partial(Search* S, TileMa
         [=] __device__(int i, int j, double acc) {
           if (i > j) return;
           const long long e = i + static_cast<long long>(ldn) * j;
-          const double v = a * C[e] + c1 * pc[i] * pc[j] + cmu * acc;
+          const double v = cov_entry(a, C[e], c1, pc[i], pc[j], cmu, acc);
           C[e] = v;
           C[j + static_cast<long long>(ldn) * i] = v;
         },
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256) k_cov_reduce(Search* S, TileMap tm) {
   int ti, tj;
   sym_tile(t, n, ti, tj);
   const double c1 = s.c1, cmu = s.cmu;
-  const double a = 1.0 - c1 - cmu + c1 * (1.0 - s.hsig) * s.cc * (2.0 - s.cc);
+  const double a = cov_keep(c1, cmu, s.cc, s.hsig);
   const double* part = s.covpart + static_cast<long long>(t) * nch * (kGBM * kGBN);
   for (int e = sub * 1024 + threadIdx.x; e < (sub + 1) * 1024; e += 256) {
     const int ii = e & (kGBM - 1), jj = e >> 6;
@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(256) k_cov_reduce(Search* S, TileMap tm) {
     double acc = 0.0;
     for (int c = 0; c < used; ++c) acc += part[static_cast<long long>(c) * (kGBM * kGBN) + e];
     const long long x = i + static_cast<long long>(ldn) * j;
-    const double v = a * s.C[x] + c1 * s.pc[i] * s.pc[j] + cmu * acc;
+    const double v = cov_entry(a, s.C[x], c1, s.pc[i], s.pc[j], cmu, acc);
     s.C[x] = v;
     s.C[j + static_cast<long long>(ldn) * i] = v;
   }

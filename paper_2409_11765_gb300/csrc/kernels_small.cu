@@ -7,14 +7,22 @@
 //                        population panel is small too, one CTA per search,
 //                        any number of generations in one launch.
 //
-// What bounds them: at n = 10, lambda = 10 a generation is ~10^4 FP64
-// operations, so its time is launches and chains. As 18 launches of the phase
-// kernels it took 277 us: 2 - 8 us each for a kernel's start and its loads, ~20 us
-// for each product (a 64 x 64 x 16 tile of FP64 FMAs at 1.7 a clock, almost all
-// padding) and 100 us for the Jacobi sweeps. Here the state stays in shared
-// memory from generation to generation, the phases are one block barrier
-// apart and work only the entries there are, and a Jacobi step's chain is ~1000
-// clocks instead of ~2500.
+// What bounds them: at n = 10, lambda = 10 a generation is ~10^4 operations, so its time
+// is chains and launches. As 18 launches of the phase kernels it took 277 us: 2 - 8 us
+// each for a kernel's start and its loads, and 100 us for the Jacobi sweeps. Here the
+// state stays in shared memory from generation to generation, the phases are one block
+// barrier apart and work only the entries there are, and a Jacobi step's chain is ~1000
+// clocks instead of ~2500: 49 us, of which 32 are the decomposition.
+//
+// A generation's sums have the operands and the order of the phase kernels': the
+// products are those of gemm_tile_f64 on integers, the rest follows each kernel's
+// partial sums. So a search has the same bits here and there -- beside a larger search,
+// under profiling, between ask and tell -- and f is that of the allocation-free
+// evaluation. (Plain FP64 sums of another order: 53 us.)
+//
+// A generation's code passes through the instruction cache every time: written out as
+// the compiler does by itself it was 391 KB, and every phase began with ~3000 clocks of
+// misses. The loops over a CTA's work and over a sum are therefore not unrolled (192 KB).
 #include "descent.cuh"
 
 namespace cmaes_gb300 {
@@ -40,6 +48,7 @@ template <class Y>
 __device__ __forceinline__ double sm_dot(int n, const double* x, int sx, const Y* y) {
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
   int k = 0;
+#pragma unroll 1
   for (; k + 4 <= n; k += 4, x += 4 * sx, y += 4) {
     const double x0 = x[0], x1 = x[sx], x2 = x[2 * sx], x3 = x[3 * sx];
     a0 = fma(x0, static_cast<double>(y[0]), a0);
@@ -53,9 +62,9 @@ __device__ __forceinline__ double sm_dot(int n, const double* x, int sx, const Y
   return (a0 + a1) + (a2 + a3);
 }
 
-// Shared memory of the eigensolver, N = n rounded up to even, matrices with
-// leading dimension N + 1: A, T, E, X, the FP32 pair, then a step's rotations
-// and the index tables of the two triangles.
+// Shared memory of the eigensolver, N = n rounded up to even: the matrices (leading
+// dimension N + 1: A, T, E, X, the FP32 pair), which nothing outlives, and a step's
+// rotations with the index tables of the two triangles.
 struct SmEig {
   double *A, *T, *E, *X, *c, *s, *t, *ev;
   float *A32, *V32;
@@ -66,21 +75,22 @@ struct SmEig {
 
 __host__ __device__ inline int sm_even(int n) { return n + (n & 1); }
 __host__ __device__ inline size_t sm_mat(int n) { return static_cast<size_t>(sm_even(n) + 1) * sm_even(n); }
-__host__ __device__ inline size_t sm_eig_doubles(int n) {
+__host__ __device__ inline size_t sm_eig_mats(int n) { return 5 * sm_mat(n); }
+__host__ __device__ inline size_t sm_eig_rest(int n) {
   const size_t N = sm_even(n), P = N / 2;
-  return 5 * sm_mat(n) + 3 * P + N + (2 * P + N + 1) / 2 + (P * (P + 1) + N * (N + 1) + 7) / 8 + 2;
+  return 3 * P + N + (2 * P + N + 1) / 2 + (P * (P + 1) + N * (N + 1) + 7) / 8 + 2;
 }
 
-__device__ SmEig sm_eig_carve(double* base, int n) {
+__device__ SmEig sm_eig_carve(double* mats, double* rest, int n) {
   const int N = sm_even(n), P = N / 2;
   SmEig w;
-  w.A = base;
+  w.A = mats;
   w.T = w.A + sm_mat(n);
   w.E = w.T + sm_mat(n);
   w.X = w.E + sm_mat(n);
   w.A32 = reinterpret_cast<float*>(w.X + sm_mat(n));
   w.V32 = w.A32 + sm_mat(n);
-  w.c = w.X + 2 * sm_mat(n);
+  w.c = rest;
   w.s = w.c + P;
   w.t = w.s + P;
   w.ev = w.t + P;
@@ -171,6 +181,7 @@ __device__ int sm_jacobi(int n, T* A, T* V, const SmEig& w, int max_sweeps, int*
         ++quiet;
         if (quiet == 1 || quiet % 16 == 0) {
           int pend = 0;
+#pragma unroll 1
           for (int e = tid; e < n * (n + 1) / 2; e += kSmNT) {
             const int i = w.ui[e], j = w.uj[e];
             if (i < j)
@@ -190,6 +201,7 @@ __device__ int sm_jacobi(int n, T* A, T* V, const SmEig& w, int max_sweeps, int*
       quiet = 0;
       // A <- J^T A J by 2 x 2 blocks of pairs (upper triangle, mirrored), and
       // V <- V J, an entry pair per thread
+#pragma unroll 1
       for (int e = tid; e < nblk + P * n; e += kSmNT) {
         if (e >= nblk) {
           const int k = quotient(e - nblk, rn), row = (e - nblk) - k * n;
@@ -244,6 +256,7 @@ __device__ __forceinline__ void sm_product(int n, int ld, const SmEig& w, double
   const int count = SYM ? n * (n + 1) / 2 : n * n;
   const int sx = TN ? 1 : ld;
   const float rn = 1.0f / n;
+#pragma unroll 1
   for (int e = threadIdx.x; e < count; e += kSmNT) {
     const int j = SYM ? w.uj[e] : quotient(e, rn), i = SYM ? w.ui[e] : e - j * n;
     const double v = epi(i, j, sm_dot(n, x + (TN ? ld * i : i), sx, y + ld * j));
@@ -271,12 +284,14 @@ constexpr double kSmSep = 0x1p-10;
 // The index tables, once per launch.
 __device__ void small_eig_tables(int n, const SmEig& w) {
   const int P = sm_even(n) / 2, tid = threadIdx.x;
+#pragma unroll 1
   for (int b = tid; b < P * (P + 1) / 2; b += kSmNT) {
     int Q = 0;
     while ((Q + 1) * (Q + 2) / 2 <= b) ++Q;
     w.bq[b] = static_cast<unsigned char>(Q);
     w.bp[b] = static_cast<unsigned char>(b - Q * (Q + 1) / 2);
   }
+#pragma unroll 1
   for (int b = tid; b < n * (n + 1) / 2; b += kSmNT) {
     int j = 0;
     while ((j + 1) * (j + 2) / 2 <= b) ++j;
@@ -291,6 +306,7 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
   const int N = sm_even(n), ld = N + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = uniform(tid >> 5);
   double *A = w.A, *T = w.T, *E = w.E, *X = w.X;
+#pragma unroll 1
   for (int e = tid; e < N * N; e += kSmNT) {  // (the dummy row and column of an odd n stay zero)
     A[e % N + ld * (e / N)] = 0.0;
     w.A32[e % N + ld * (e / N)] = 0.0f;
@@ -322,6 +338,7 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
   }
   __syncthreads();
   const float shift = sh_shift;
+#pragma unroll 1
   for (int e = tid; e < n * n; e += kSmNT) {
     const int j = e / n, i = e - j * n;
     w.A32[i + ld * j] = static_cast<float>(A[i + ld * j] - (i == j ? static_cast<double>(shift) : 0.0));
@@ -340,6 +357,7 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
     __syncthreads();
     sm_product<true, true>(n, ld, w, A, X, T, [](int, int, double v) { return v; });  // S
     __syncthreads();
+#pragma unroll 1
     for (int e = tid; e < n * (n + 1) / 2; e += kSmNT) {
       const int i = w.ui[e], j = w.uj[e];
       const double gij = B[i + ld * j];
@@ -420,6 +438,7 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
     if (lane < n) T[lane + ld * w.rk[j]] = neg ? -v : v;
   }
   __syncthreads();
+#pragma unroll 1
   for (int e = tid; e < n * n; e += kSmNT) {
     const int j = e / n, i = e - j * n;
     B[i + ld * j] = T[i + ld * j];
@@ -439,8 +458,9 @@ __global__ void __launch_bounds__(kSmNT) k_small_eig(Search* S, int s0) {
   const int n = s.n, ldn = s.ldn, N = sm_even(n), ld = N + 1, tid = threadIdx.x;
   double* C = sdyn;
   double* B = C + sm_mat(n);
-  const SmEig w = sm_eig_carve(B + sm_mat(n), n);
+  const SmEig w = sm_eig_carve(B + sm_mat(n), B + sm_mat(n) + sm_eig_mats(n), n);
   small_eig_tables(n, w);
+#pragma unroll 1
   for (int e = tid; e < N * N; e += kSmNT) {
     const int i = e % N, j = e / N;
     const bool in = i < n && j < n;
@@ -449,7 +469,9 @@ __global__ void __launch_bounds__(kSmNT) k_small_eig(Search* S, int s0) {
   }
   __syncthreads();
   const int sweeps = small_eig(n, C, B, w, &sh_rot);
+#pragma unroll 1
   for (int e = tid; e < n * n; e += kSmNT) s.B[e % n + ldn * (e / n)] = B[e % n + ld * (e / n)];
+#pragma unroll 1
   for (int i = tid; i < n; i += kSmNT) {
     s.D[i] = sqrt(w.ev[i]);
     s.C[i + ldn * i] = C[i + ld * i];
@@ -462,7 +484,7 @@ __global__ void __launch_bounds__(kSmNT) k_small_eig(Search* S, int s0) {
   }
 }
 
-static size_t small_eig_smem(int n) { return (2 * sm_mat(n) + sm_eig_doubles(n)) * sizeof(double); }
+static size_t small_eig_smem(int n) { return (2 * sm_mat(n) + sm_eig_mats(n) + sm_eig_rest(n)) * sizeof(double); }
 
 void launch_small_eig(Search* S, int s0, int s1, int max_n, cudaStream_t st) {
   if (s1 > s0) k_small_eig<<<s1 - s0, kSmNT, small_eig_smem(max_n), st>>>(S, s0);
@@ -479,15 +501,21 @@ __device__ __forceinline__ long long order_bits(double x) {
 }
 
 struct SmGen {
-  double *C, *B, *BD, *Q, *D, *m, *ps, *pc, *xs, *ld_, *yw, *zw, *w, *Z, *Y, *R, *U, *f;
+  double *C, *B, *BD, *D, *m, *ps, *pc, *xs, *ld_, *yw, *zw, *w, *Z, *Y, *R, *U, *f;
+  int2 *BDl, *Ql, *L;  // integer operands of the products: B D, Q, and the panel's
+  int *eBD, *eQ, *eL;  // their scales: of a row, a row, a candidate
   unsigned long long* key;
   int* order;
-  double* eig;
+  double *mats, *rest;  // of the eigensolver; the panels Z .. L lie where its matrices do
 };
 
+__host__ __device__ inline size_t sm_gen_panels(int n, int lam) {
+  const size_t panels = 5 * static_cast<size_t>(n) * lam;
+  return panels > sm_eig_mats(n) ? panels : sm_eig_mats(n);
+}
 __host__ __device__ inline size_t sm_gen_doubles(int n, int lam) {
-  return 4 * sm_mat(n) + 8 * static_cast<size_t>(n) + lam / 2 + 1 + 4 * static_cast<size_t>(n) * lam + 2 * lam +
-         (lam + 1) / 2 + sm_eig_doubles(n);
+  return 5 * sm_mat(n) + 9 * static_cast<size_t>(n) + lam / 2 + 1 + 2 * lam + 2 * ((lam + 1) / 2) + sm_eig_rest(n) +
+         sm_gen_panels(n, lam);
 }
 
 __device__ SmGen sm_gen_carve(double* p, int n, int lam) {
@@ -500,7 +528,8 @@ __device__ SmGen sm_gen_carve(double* p, int n, int lam) {
   g.C = take(sm_mat(n));
   g.B = take(sm_mat(n));
   g.BD = take(sm_mat(n));
-  g.Q = take(sm_mat(n));
+  g.BDl = reinterpret_cast<int2*>(take(sm_mat(n)));
+  g.Ql = reinterpret_cast<int2*>(take(sm_mat(n)));
   g.D = take(n);
   g.m = take(n);
   g.ps = take(n);
@@ -509,16 +538,72 @@ __device__ SmGen sm_gen_carve(double* p, int n, int lam) {
   g.ld_ = take(n);
   g.yw = take(n);
   g.zw = take(n);
+  g.eBD = reinterpret_cast<int*>(take(n));
+  g.eQ = g.eBD + n;
   g.w = take(lam / 2 + 1);
+  g.f = take(lam);
+  g.key = reinterpret_cast<unsigned long long*>(take(lam));
+  g.order = reinterpret_cast<int*>(take((lam + 1) / 2));
+  g.eL = reinterpret_cast<int*>(take((lam + 1) / 2));
+  g.rest = take(sm_eig_rest(n));
+  g.mats = p;
   g.Z = take(static_cast<size_t>(n) * lam);
   g.Y = take(static_cast<size_t>(n) * lam);
   g.R = take(static_cast<size_t>(n) * lam);
   g.U = take(static_cast<size_t>(n) * lam);
-  g.f = take(lam);
-  g.key = reinterpret_cast<unsigned long long*>(take(lam));
-  g.order = reinterpret_cast<int*>(take((lam + 1) / 2));
-  g.eig = p;
+  g.L = reinterpret_cast<int2*>(take(static_cast<size_t>(n) * lam));
   return g;
+}
+
+// One K step of an output of gemm_tile_f64 added to acc: limbs a[sa k], b[sb k] with the
+// scales ea, eb; the entries themselves A[sA k] and B[sB k], or B[sB order[k]]. (Not
+// inlined, as the two below: a generation's code passes through the instruction cache
+// each time, and these are called from three places.)
+__device__ __noinline__ double sm_step(double acc, int kn, const int2* a, int sa, const int2* b, int sb, int ea,
+                                       int eb, const double* A, int sA, const double* B, int sB, const int* order) {
+  long long hh = 0, mid = 0;
+  unsigned sum = 0;
+#pragma unroll 2
+  for (int k = 0; k < kn; ++k) {
+    const int2 x = a[sa * k], y = b[sb * k];
+    hh += static_cast<long long>(x.x) * y.x;
+    mid += static_cast<long long>(x.x) * y.y;
+    mid += static_cast<long long>(x.y) * y.x;
+    sum += gemm_byte(x.x) * gemm_byte(y.x);
+  }
+  if (!gemm_in_f64(sum, ea, eb)) return acc + gemm_scaled<29>(hh, mid, ea + eb);
+#pragma unroll 1
+  for (int k = 0; k < kn; ++k) acc = fma(A[sA * k], B[sB * (order ? order[k] : k)], acc);
+  return acc;
+}
+
+// The largest biased exponent of x[s k], k < n.
+__device__ __forceinline__ int sm_scale(const double* x, int s, int n) {
+  int e = 0;
+  for (int k = 0; k < n; ++k) e = max(e, gemm_exponent(x[s * k]));
+  return e;
+}
+
+// The n x n matrix x (entry (i, j) at x[i + lx j]) as integers by rows.
+__device__ __noinline__ void sm_rows_as_integers(int n, int ld, const double* x, long long lx, int2* out, int* eo) {
+#pragma unroll 1
+  for (int e = threadIdx.x; e < n * n; e += kSmNT) {
+    const int j = e / n, i = e - j * n;
+    const int E = sm_scale(x + i, static_cast<int>(lx), n);
+    out[i + ld * j] = gemm_limbs<29>(x[i + lx * j], E);
+    if (j == 0) eo[i] = E;
+  }
+}
+
+// The panel x (n x lam) as integers by columns.
+__device__ __noinline__ void sm_panel_as_integers(int n, int lam, float rn, const double* x, int2* out, int* eo) {
+#pragma unroll 1
+  for (int e = threadIdx.x; e < n * lam; e += kSmNT) {
+    const int k = quotient(e, rn), i = e - k * n;
+    const int E = sm_scale(x + n * k, 1, n);
+    out[e] = gemm_limbs<29>(x[e], E);
+    if (i == 0) eo[k] = E;
+  }
 }
 
 __device__ __forceinline__ double sm_sum(double v) {
@@ -529,7 +614,12 @@ __device__ __forceinline__ double sm_sum(double v) {
 
 }  // namespace
 
-__global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, DevOptions o, int gens) {
+// PER_SM: the CTAs per SM that the registers are cut for. One search runs 15 % faster
+// with a whole SM's; where more searches than SMs would wait, four side by side do more
+// (20 generations of n = 10, lambda = 10: 965 and 1135 us; ten of 1000 such searches, two
+// CTAs and four per SM: 2.08 and 1.56 ms; of 2000 with n = 20, lambda = 12: 9.6 and 7.8).
+template <int PER_SM>
+__global__ void __launch_bounds__(kSmNT, PER_SM) k_small_generations(Search* S, int s0, DevOptions o, int gens) {
   extern __shared__ double sdyn[];
   __shared__ double sh[32];
   __shared__ double sh_den, sh_psn, sh_hsig, sh_sigma, sh_best;
@@ -539,24 +629,28 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
   const int n = s.n, ldn = s.ldn, N = sm_even(n), ld = N + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = uniform(tid >> 5);
   const SmGen g = sm_gen_carve(sdyn, n, s.lam_cap);
-  const SmEig we = sm_eig_carve(g.eig, n);
+  const SmEig we = sm_eig_carve(g.mats, g.rest, n);
   small_eig_tables(n, we);
   const int obj = s.obj, npairs = (n + 1) >> 1;
   const float rn = 1.0f / n, rp = 1.0f / npairs;
+  const int tree_top = n > 16 ? 16 : n > 8 ? 8 : n > 4 ? 4 : n > 2 ? 2 : n - 1;  // f's first level with a pair
 
   for (int done_gens = 0; done_gens < gens;) {
     // ---- the state of this descent ----
     const int lam = s.lam, mu = s.mu, g_eig = s.g_eig, hist_len = s.hist_len, max_iter = s.max_iter;
     const double cs = s.cs, ds = s.ds, cc = s.cc, c1 = s.c1, cmu = s.cmu, chin = s.chin, mueff = s.mueff;
     int gen = s.gen, hist_count = s.hist_count;
+#pragma unroll 1
     for (int e = tid; e < N * N; e += kSmNT) {
       const int i = e % N, j = e / N;
       const bool in = i < n && j < n;
       g.C[i + ld * j] = in ? s.C[i + ldn * j] : 0.0;
       g.B[i + ld * j] = in ? s.B[i + ldn * j] : 0.0;
       g.BD[i + ld * j] = in ? s.BD[i + ldn * j] : 0.0;
-      g.Q[i + ld * j] = in && obj != 3 ? s.Q[i + ldn * j] : 0.0;
     }
+    sm_rows_as_integers(n, ld, s.BD, ldn, g.BDl, g.eBD);
+    if (obj != 3) sm_rows_as_integers(n, ld, s.Q, ldn, g.Ql, g.eQ);
+#pragma unroll 1
     for (int i = tid; i < n; i += kSmNT) {
       g.D[i] = s.D[i];
       g.m[i] = s.m[i];
@@ -565,6 +659,7 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
       g.xs[i] = s.xstar[i];
       g.ld_[i] = obj == 1 ? s.lamdiag[i] : 0.0;
     }
+#pragma unroll 1
     for (int r = tid; r < mu; r += kSmNT) g.w[r] = s.w[r];
     if (tid == 0) {
       sh_sigma = s.sigma;
@@ -576,6 +671,7 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
     // ---- generations until the block's count, a stop or a restart ----
     for (; done_gens < gens && !flags; ++done_gens) {
       // z; the denominator of the h_sigma test beside it
+#pragma unroll 1
       for (int e = tid; e < npairs * lam; e += kSmNT) {
         const int k = quotient(e, rp), j = e - k * npairs;
         double z0, z1;
@@ -590,45 +686,63 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
       }
       __syncthreads();
       const double sigma = sh_sigma;
+      sm_panel_as_integers(n, lam, rn, g.Z, g.L, g.eL);
+      __syncthreads();
       // y = B D z, x = m + sigma y
+#pragma unroll 1
       for (int e = tid; e < n * lam; e += kSmNT) {
         const int k = quotient(e, rn), i = e - k * n;
-        const double y = sm_dot(n, g.BD + i, ld, g.Z + n * k), x = g.m[i] + sigma * y;
+        const double y = sm_step(0.0, n, g.BDl + i, ld, g.L + n * k, 1, g.eBD[i], g.eL[k], g.BD + i, ld, g.Z + n * k, 1,
+                                 nullptr);
+        const double x = step_from(g.m[i], sigma, y);
         g.Y[n * k + i] = y;
         g.R[n * k + i] = x - g.xs[i];
         s.X[i + static_cast<long long>(ldn) * k] = x;
       }
       __syncthreads();
+      if (obj != 3) {
+        sm_panel_as_integers(n, lam, rn, g.R, g.L, g.eL);
+        __syncthreads();
+      }
       // the objective's terms
+#pragma unroll 1
       for (int e = tid; e < n * lam; e += kSmNT) {
         const int k = quotient(e, rn), i = e - k * n;
-        const double* rr = g.R + n * k;
         double term;
         if (obj == 3) {
-          term = rr[i] * rr[i];
+          term = g.R[e] * g.R[e];
         } else {
-          const double u = sm_dot(n, g.Q + i, ld, rr);
-          term = obj == 1 ? g.ld_[i] * u * u : u * u - 10.0 * cospi(2.0 * u);
+          const double u = sm_step(0.0, n, g.Ql + i, ld, g.L + n * k, 1, g.eQ[i], g.eL[k], s.Q + i, ldn, g.R + n * k, 1,
+                                   nullptr);
+          term = objective_term(obj, g.ld_[i], u);
         }
-        g.U[n * k + i] = term;
+        g.U[e] = term;
       }
       __syncthreads();
+      // f: the shuffle tree of k_colreduce_f over 32 lanes
+#pragma unroll 1
       for (int k = tid; k < lam; k += kSmNT) {
-        const double* u = g.U + n * k;
-        double a0 = 0.0, a1 = 0.0;
-        int i = 0;
-        for (; i + 1 < n; i += 2) {
-          a0 += u[i];
-          a1 += u[i + 1];
-        }
-        if (i < n) a0 += u[i];
-        const double f = (obj == 2) ? 10.0 * n + (a0 + a1) : a0 + a1;
+        double* u = g.U + n * k;
+#pragma unroll 1
+        for (int off = tree_top; off > 0; off >>= 1)
+#pragma unroll 1
+          for (int i = 0; i < min(off, n - off); i += 4) {  // four independent sums at a time
+            double v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = i + q < min(off, n - off) ? u[i + q] + u[i + q + off] : 0.0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (i + q < min(off, n - off)) u[i + q] = v[q];
+          }
+        const double sum = n < 32 ? u[0] + 0.0 : u[0];
+        const double f = (obj == 2) ? 10.0 * n + sum : sum;
         g.f[k] = f;
         g.key[k] = rank_key(f);
         s.f[k] = f;
       }
       __syncthreads();
       // rank: ascending f, ties by index
+#pragma unroll 1
       for (int k = tid; k < lam; k += kSmNT) {
         const unsigned long long key = g.key[k];
         int r = 0;
@@ -638,24 +752,36 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
         s.order[r] = k;
       }
       __syncthreads();
-      // <y>_w and <z>_w: eight threads per entry
+      // <y>_w and <z>_w: eight threads per entry, for the eight warps of k_recomb_partial
+#pragma unroll 1
       for (int e = tid; e < ((2 * n * 8 + 31) & ~31); e += kSmNT) {
         const int id = e >> 3, i = id % n;
         const double* src = id < n ? g.Y : g.Z;
-        double a = 0.0;
-        if (id < 2 * n)
-          for (int r = e & 7; r < mu; r += 8) a = fma(g.w[r], src[n * g.order[r] + i], a);
-        a += __shfl_xor_sync(0xffffffffu, a, 1);
-        a += __shfl_xor_sync(0xffffffffu, a, 2);
-        a += __shfl_xor_sync(0xffffffffu, a, 4);
-        if ((e & 7) == 0 && id < 2 * n) (id < n ? g.yw : g.zw)[i] = a;
+        double total = 0.0;
+        for (int r0 = 0; r0 < mu; r0 += 256) {
+          double a = 0.0, v = 0.0;
+          if (id < 2 * n)
+            for (int r = r0 + (e & 7); r < min(mu, r0 + 256); r += 8) a = fma(g.w[r], src[n * g.order[r] + i], a);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v += __shfl_sync(0xffffffffu, a, (lane & 24) + q);
+          total += v;
+        }
+        if ((e & 7) == 0 && id < 2 * n) (id < n ? g.yw : g.zw)[i] = total;
       }
       __syncthreads();
       // p_sigma, its norm, h_sigma (warp 0); the mean (warp 1); the best point (warp 2)
       if (warp == 0) {
         double ps = 0.0;
         if (lane < n) {
-          ps = (1.0 - cs) * g.ps[lane] + sqrt(cs * (2.0 - cs) * mueff) * sm_dot(n, g.B + lane, ld, g.zw);
+          double part[8] = {}, v = 0.0;  // the eight warps of k_psigma_partial
+#pragma unroll 1
+          for (int j0 = 0; j0 < n; j0 += 8)
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              if (j0 + q < n) part[q] = fma(g.B[lane + ld * (j0 + q)], g.zw[j0 + q], part[q]);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v += part[q];
+          ps = path_step(cs, g.ps[lane], sqrt(cs * (2.0 - cs) * mueff), v);
           g.ps[lane] = ps;
         }
         const double psn = sqrt(sm_sum(ps * ps));
@@ -664,7 +790,7 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
           sh_hsig = (psn / sh_den < (1.4 + 2.0 / (n + 1.0)) * chin) ? 1.0 : 0.0;
         }
       } else if (warp == 1) {
-        if (lane < n) g.m[lane] = g.m[lane] + sigma * g.yw[lane];
+        if (lane < n) g.m[lane] = step_from(g.m[lane], sigma, g.yw[lane]);
       } else if (warp == 2) {
         const int i0 = g.order[0];
         const double f0 = g.f[i0];
@@ -682,29 +808,61 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
       __syncthreads();
       const double hsig = sh_hsig, psn = sh_psn;
       if (tid == kSmNT - 1) sh_sigma = sigma * exp((cs / ds) * (psn / chin - 1.0));
-      if (warp == 0 && lane < n) g.pc[lane] = (1.0 - cc) * g.pc[lane] + hsig * sqrt(cc * (2.0 - cc) * mueff) * g.yw[lane];
+      if (warp == 0 && lane < n) g.pc[lane] = path_step(cc, g.pc[lane], hsig * sqrt(cc * (2.0 - cc) * mueff), g.yw[lane]);
+      __syncthreads();
+      // the rank-mu product's operands as integers, in the chunks of k_cov_partial and the
+      // steps of its tile: w y at R and L, y at L + mu n, their scales at Z
+      const int kc = s.cov_kc, chunk_steps = ceil_div(kc, gemm_step(kc));
+      int *ea = reinterpret_cast<int*>(g.Z), *eb = ea + n * ceil_div(mu, kc) * chunk_steps;
+      // rank r's step and that step's range
+      auto step_of = [&](int r, int& r0, int& r1) {
+        const int c = r / kc, last = min(mu, (c + 1) * kc), len = gemm_step(last - c * kc), q = (r - c * kc) / len;
+        r0 = c * kc + q * len;
+        r1 = min(last, r0 + len);
+        return c * chunk_steps + q;
+      };
+#pragma unroll 1
+      for (int e = tid; e < mu * n; e += kSmNT) {
+        const int r = quotient(e, rn);
+        g.R[e] = g.w[r] * g.Y[n * g.order[r] + (e - r * n)];
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int e = tid; e < mu * n; e += kSmNT) {
+        const int r = quotient(e, rn), i = e - r * n;
+        int r0, r1, a = 0, b = 0;
+        const int st = step_of(r, r0, r1);
+        for (int q = r0; q < r1; ++q) {
+          a = max(a, gemm_exponent(g.R[n * q + i]));
+          b = max(b, gemm_exponent(g.Y[n * g.order[q] + i]));
+        }
+        if (r == r0) {
+          ea[n * st + i] = a;
+          eb[n * st + i] = b;
+        }
+        g.L[e] = gemm_limbs<29>(g.R[e], a);
+        g.L[mu * n + e] = gemm_limbs<29>(g.Y[n * g.order[r] + i], b);
+      }
       __syncthreads();
       // C, upper triangle with its mirror
       {
-        const double a = 1.0 - c1 - cmu + c1 * (1.0 - hsig) * cc * (2.0 - cc);
+        const double keep = cov_keep(c1, cmu, cc, hsig);
+#pragma unroll 1
         for (int e = tid; e < n * (n + 1) / 2; e += kSmNT) {
           const int i = we.ui[e], j = we.uj[e];
-          double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-          auto add = [&](int r, double& acc) {
-            const double* y = g.Y + n * g.order[r];
-            acc = fma(g.w[r] * y[i], y[j], acc);
-          };
-          int r = 0;
-          for (; r + 4 <= mu; r += 4) {
-            add(r, a0);
-            add(r + 1, a1);
-            add(r + 2, a2);
-            add(r + 3, a3);
+          double acc = 0.0, chunk = 0.0;
+          for (int r = 0; r < mu;) {
+            int r0, r1;
+            const int st = step_of(r, r0, r1);
+            chunk = sm_step(chunk, r1 - r0, g.L + n * r0 + i, n, g.L + n * (mu + r0) + j, n, ea[n * st + i],
+                            eb[n * st + j], g.R + n * r0 + i, n, g.Y + j, n, g.order + r0);
+            r = r1;
+            if (r % kc == 0 || r == mu) {
+              acc += chunk;
+              chunk = 0.0;
+            }
           }
-          if (r < mu) add(r, a0);
-          if (r + 1 < mu) add(r + 1, a1);
-          if (r + 2 < mu) add(r + 2, a2);
-          const double v = a * g.C[i + ld * j] + c1 * g.pc[i] * g.pc[j] + cmu * ((a0 + a1) + (a2 + a3));
+          const double v = cov_entry(keep, g.C[i + ld * j], c1, g.pc[i], g.pc[j], cmu, acc);
           g.C[i + ld * j] = v;
           g.C[j + ld * i] = v;
         }
@@ -714,6 +872,7 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
       __syncthreads();
       if (due) {
         const int sweeps = small_eig(n, g.C, g.B, we, &sh_rot);
+#pragma unroll 1
         for (int i = tid; i < n; i += kSmNT) g.D[i] = sqrt(we.ev[i]);
         if (tid == 0) {
           s.eig_sweeps = sweeps;
@@ -722,10 +881,13 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
           s.eig_rotations += sh_rot;
         }
         __syncthreads();
+#pragma unroll 1
         for (int e = tid; e < n * n; e += kSmNT) {
           const int i = e % n, j = e / n;
           g.BD[i + ld * j] = g.B[i + ld * j] * g.D[j];
         }
+        __syncthreads();
+        sm_rows_as_integers(n, ld, g.BD, ld, g.BDl, g.eBD);
       }
       // ---- stop tests: the axis, coordinate, TolX and finiteness ones in warp
       // 0 (a lane per coordinate), the history in warp 1 ----
@@ -791,12 +953,14 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
       __syncthreads();  // sh_bits is cleared in the next generation
     }
     // ---- the state back to its place ----
+#pragma unroll 1
     for (int e = tid; e < n * n; e += kSmNT) {
       const int i = e % n, j = e / n;
       s.C[i + ldn * j] = g.C[i + ld * j];
       s.B[i + ldn * j] = g.B[i + ld * j];
       s.BD[i + ldn * j] = g.BD[i + ld * j];
     }
+#pragma unroll 1
     for (int i = tid; i < n; i += kSmNT) {
       s.D[i] = g.D[i];
       s.m[i] = g.m[i];
@@ -830,18 +994,37 @@ __global__ void __launch_bounds__(kSmNT) k_small_generations(Search* S, int s0, 
 }
 
 bool small_generation(int n, int lam_cap) {
-  return n <= kJacobiSmallN && static_cast<long long>(n) * lam_cap <= kSmallPanel;
+  return n <= kJacobiSmallN && lam_cap <= kSmallLambda && static_cast<long long>(n) * lam_cap <= kSmallPanel;
 }
 
 size_t small_generation_smem(int n, int lam_cap) { return sm_gen_doubles(n, lam_cap) * sizeof(double); }
 
-cudaError_t small_smem_limits() {
-  const cudaError_t e = smem_limit_max(reinterpret_cast<const void*>(k_small_generations));
-  return e != cudaSuccess ? e : smem_limit_max(reinterpret_cast<const void*>(k_small_eig));
+static const void* small_fn(bool dense) {
+  return dense ? reinterpret_cast<const void*>(k_small_generations<4>) : reinterpret_cast<const void*>(k_small_generations<1>);
 }
 
-void launch_small_generations(Search* S, int count, DevOptions o, int gens, size_t smem, cudaStream_t st) {
-  k_small_generations<<<count, kSmNT, smem, st>>>(S, 0, o, gens);
+cudaError_t small_smem_limits() {
+  for (const void* k : {small_fn(false), small_fn(true), reinterpret_cast<const void*>(k_small_eig)})
+    if (const cudaError_t e = smem_limit_max(k); e != cudaSuccess) return e;
+  return cudaSuccess;
+}
+
+// Whether `count` searches overflow the CTAs of the kernel for few, and more fit of the other.
+cudaError_t small_generations_dense(int count, size_t smem, bool* dense) {
+  int dev = 0, sms = 0, few = 0, many = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&few, small_fn(false), kSmNT, smem)) != cudaSuccess ||
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&many, small_fn(true), kSmNT, smem)) != cudaSuccess)
+    return e;
+  *dense = many > few && count > static_cast<long long>(few) * sms;
+  return cudaSuccess;
+}
+
+void launch_small_generations(Search* S, int count, DevOptions o, int gens, size_t smem, bool dense, cudaStream_t st) {
+  if (dense) k_small_generations<4><<<count, kSmNT, smem, st>>>(S, 0, o, gens);
+  else k_small_generations<1><<<count, kSmNT, smem, st>>>(S, 0, o, gens);
 }
 
 }  // namespace cmaes_gb300

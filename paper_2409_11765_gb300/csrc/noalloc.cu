@@ -15,6 +15,7 @@
 #include <string>
 
 #include "../../include/cmaes.h"
+#include "descent.cuh"
 #include "device_common.cuh"
 
 namespace cmaes_gb300 {
@@ -57,10 +58,10 @@ __global__ void __launch_bounds__(256) k_noalloc_reduce(int kind, int n, int lam
     }
   } else if (kind == CMAES_OBJ_ELLIPSOID) {
     const double* u = U + static_cast<long long>(ld) * k;
-    for (int i = lane; i < n; i += 32) acc += lamdiag[i] * u[i] * u[i];
+    for (int i = lane; i < n; i += 32) acc += objective_term(1, lamdiag[i], u[i]);
   } else {
     const double* u = U + static_cast<long long>(ld) * k;
-    for (int i = lane; i < n; i += 32) acc += u[i] * u[i] - 10.0 * cospi(2.0 * u[i]);
+    for (int i = lane; i < n; i += 32) acc += objective_term(2, 0.0, u[i]);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);

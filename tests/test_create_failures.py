@@ -24,6 +24,7 @@ int cudaGetDevice(int* d) { *d = 0; return 0; }
 int cudaDeviceGetAttribute(int* v, int a, int d) { *v = 152; return 0; }
 int cudaFuncGetAttributes(void* a, const void* f) { memset(a, 0, 64); return 0; }
 int cudaFuncSetAttribute(const void* f, int a, int v) { return 0; }
+int cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* b, const void* f, int t, size_t n) { *b = 1; return 0; }
 int cudaStreamCreateWithFlags(void** s, unsigned f) { *s = (void*)8; return 0; }
 int cudaStreamDestroy(void* s) { return 0; }
 int cudaStreamSynchronize(void* s) { return 0; }
