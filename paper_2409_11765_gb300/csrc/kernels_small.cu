@@ -43,6 +43,13 @@ __device__ __forceinline__ int quotient(int e, float rd) {
   return __float2int_rz((static_cast<float>(e) + 0.5f) * rd);
 }
 
+// |x| in FP32, cut to 20 bits of mantissa, by the bits (a conversion takes the FP64
+// pipe); below 2^-126 it is zero.
+__device__ __forceinline__ unsigned sm_float_bits(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff, e = hi - (896 << 20);
+  return e < (1 << 20) ? 0u : static_cast<unsigned>(min(e, 0xff << 20)) << 3;
+}
+
 // sum_k x[sx k] y[k], k < n, in four chains
 template <class Y>
 __device__ __forceinline__ double sm_dot(int n, const double* x, int sx, const Y* y) {
@@ -117,7 +124,7 @@ __device__ __forceinline__ void sm_cos(float tf, float& c) { c = rsqrtf(fmaf(tf,
 
 // Cyclic Jacobi on the symmetric A (N x N, leading dimension ld, a zero row and
 // column beyond n), V <- V J over n rows. A pair turns when rotates(app, aqq,
-// apq) says so (FP32 values). Round-robin steps of N / 2 disjoint pairs; a
+// apq, p, q) says so (FP32 values). Round-robin steps of N / 2 disjoint pairs; a
 // step's t = tan(phi) is an FP32 value in either type (its error leaves 2^-23
 // of a_pq, which a later step takes). FP64 operations (66 clocks each, 19 of a
 // whole SM's pipe a warp) stay where the result needs them: d = a_qq - a_pp, c,
@@ -146,7 +153,7 @@ __device__ int sm_jacobi(int n, T* A, T* V, const SmEig& w, int max_sweeps, int*
             const T app = A[p + ld * p], aqq = A[q + ld * q], apq = A[p + ld * q];
             const T d = aqq - app;
             const float af = static_cast<float>(apq);
-            if (rotates(static_cast<float>(app), static_cast<float>(aqq), af)) {
+            if (rotates(static_cast<float>(app), static_cast<float>(aqq), af, p, q)) {
               act = true;
               const float df = static_cast<float>(d);
               float tf;
@@ -186,7 +193,7 @@ __device__ int sm_jacobi(int n, T* A, T* V, const SmEig& w, int max_sweeps, int*
             const int i = w.ui[e], j = w.uj[e];
             if (i < j)
               pend |= rotates(static_cast<float>(A[i + ld * i]), static_cast<float>(A[j + ld * j]),
-                              static_cast<float>(A[i + ld * j]));
+                              static_cast<float>(A[i + ld * j]), i, j);
           }
           if (!__syncthreads_or(pend)) quiet = M;
         } else {
@@ -274,12 +281,15 @@ __device__ __forceinline__ void sm_product(int n, int ld, const SmEig& w, double
 //   lambda_i = s_ii / g_ii, e_ij = (s_ij - lambda_j g_ij) / (lambda_j -
 //   lambda_i), X <- X + X E; pairs too close for first order get -g_ij / 2)
 //   and a Newton-Schulz step; A = X^T C X; FP64 Jacobi on what is left above
-//   the rounding level of that product.
+//   the rounding level of that product's entries.
 // A shift by tr(A) / n lets FP32 resolve a spectrum of nearly equal eigenvalues;
 // a graded A is left as it is, so that its small eigenvalues keep their FP32
-// relative accuracy. All kSmNT threads call it. Returns the FP64 sweeps; *rot
-// their rotations (thread 0).
+// relative accuracy. All kSmNT threads call it. Returns the sweeps of both; *rot the
+// FP64 ones' rotations (thread 0).
 constexpr double kSmSep = 0x1p-10;
+struct SmSweeps {
+  int f64, f32;
+};
 
 // The index tables, once per launch.
 __device__ void small_eig_tables(int n, const SmEig& w) {
@@ -300,7 +310,7 @@ __device__ void small_eig_tables(int n, const SmEig& w) {
   }
 }
 
-__device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) {
+__device__ SmSweeps small_eig(int n, double* C, double* B, const SmEig& w, int* rot) {
   __shared__ int sh_big, sh_rot32;
   __shared__ float sh_shift;
   const int N = sm_even(n), ld = N + 1;
@@ -315,7 +325,7 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
   if (tid == 0) {
     *rot = sh_rot32 = 0;
     sh_big = 0;
-      }
+  }
   __syncthreads();
   if (warp == 0 && lane < n) atomicMax(&sh_big, (__double2hiint(fabs(C[lane + ld * lane])) >> 20) & 0x7ff);
   sm_product<false, false>(n, ld, w, T, C, B, [](int, int, double v) { return v; });
@@ -345,7 +355,7 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
   }
   __syncthreads();
   const float floor32 = shift != 0.0f ? 16.0f * 0x1p-24f * 2.0f : 0.0f;
-  sm_jacobi<float>(n, w.A32, w.V32, w, 12, &sh_rot32, [=](float app, float aqq, float apq) {
+  const int sweeps32 = sm_jacobi<float>(n, w.A32, w.V32, w, 12, &sh_rot32, [=](float app, float aqq, float apq, int, int) {
     return fabsf(apq) > floor32 && fabsf(apq) * rsqrtf(fabsf(app)) * rsqrtf(fabsf(aqq)) > 1e-6f;
   });
   __syncthreads();
@@ -397,9 +407,25 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
   __syncthreads();
   if (warp == 0 && lane < n) atomicMax(&sh_big, __float_as_int(fabsf(static_cast<float>(A[lane + ld * lane]))));
   __syncthreads();
-  const float floor64 = static_cast<float>(n) * 0x1p-53f * __int_as_float(sh_big);
-  const int sweeps = sm_jacobi<double>(n, A, B, w, kSmMaxSweeps, rot, [=](float app, float aqq, float apq) {
-    return fabsf(apq) > floor64 && fabsf(apq) * rsqrtf(fabsf(app)) * rsqrtf(fabsf(aqq)) > kSmTol;
+  // The rounding of a_ij is within n eps of (|X|^T |C| |X|)_ij, and that of g_i g_j with
+  // g_i = sum_k |x_ki| sqrt(c_kk), C being positive semi-definite: an entry below is not
+  // turned. Where X mixes large and small c_kk this is the level of max a_ii; a graded
+  // C whose X is near I keeps the relative test, and so its small eigenvalues.
+  float *root = w.A32, *g = w.A32 + N;  // (the FP32 pair is done with)
+  if (warp == 0 && lane < n) root[lane] = sqrtf(fabsf(static_cast<float>(C[lane + ld * lane] * up)));
+  __syncwarp();
+  if (warp == 0 && lane < n) {
+    float sum = 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k)
+      sum = fmaf(__uint_as_float(sm_float_bits(B[k + ld * lane])), root[k], sum);
+    g[lane] = sum;
+  }
+  __syncthreads();
+  const float noise = static_cast<float>(n) * 0x1p-53f, top = __int_as_float(sh_big);
+  const int sweeps = sm_jacobi<double>(n, A, B, w, kSmMaxSweeps, rot, [=](float app, float aqq, float apq, int p, int q) {
+    return fabsf(apq) > noise * fminf(top, g[p] * g[q]) &&
+           fabsf(apq) * rsqrtf(fabsf(app)) * rsqrtf(fabsf(aqq)) > kSmTol;
   });
   // eigenvalues with the PD guard
   if (warp == 0) {
@@ -444,7 +470,7 @@ __device__ int small_eig(int n, double* C, double* B, const SmEig& w, int* rot) 
     B[i + ld * j] = T[i + ld * j];
   }
   __syncthreads();
-  return sweeps;
+  return SmSweeps{sweeps, sweeps32};
 }
 
 }  // namespace
@@ -468,7 +494,7 @@ __global__ void __launch_bounds__(kSmNT) k_small_eig(Search* S, int s0) {
     B[i + ld * j] = in ? s.B[i + ldn * j] : 0.0;
   }
   __syncthreads();
-  const int sweeps = small_eig(n, C, B, w, &sh_rot);
+  const SmSweeps sweeps = small_eig(n, C, B, w, &sh_rot);
 #pragma unroll 1
   for (int e = tid; e < n * n; e += kSmNT) s.B[e % n + ldn * (e / n)] = B[e % n + ld * (e / n)];
 #pragma unroll 1
@@ -477,9 +503,10 @@ __global__ void __launch_bounds__(kSmNT) k_small_eig(Search* S, int s0) {
     s.C[i + ldn * i] = C[i + ld * i];
   }
   if (tid == 0) {
-    s.eig_sweeps = sweeps;
+    s.eig_sweeps = sweeps.f64;
     s.eig_count += 1;
-    s.eig_sweeps_total += sweeps;
+    s.eig_sweeps_total += sweeps.f64;
+    s.eig_sweeps32 += sweeps.f32;
     s.eig_rotations += sh_rot;
   }
 }
@@ -871,13 +898,14 @@ __global__ void __launch_bounds__(kSmNT, PER_SM) k_small_generations(Search* S, 
       due = (gen % g_eig) == 0;
       __syncthreads();
       if (due) {
-        const int sweeps = small_eig(n, g.C, g.B, we, &sh_rot);
+        const SmSweeps sweeps = small_eig(n, g.C, g.B, we, &sh_rot);
 #pragma unroll 1
         for (int i = tid; i < n; i += kSmNT) g.D[i] = sqrt(we.ev[i]);
         if (tid == 0) {
-          s.eig_sweeps = sweeps;
+          s.eig_sweeps = sweeps.f64;
           s.eig_count += 1;
-          s.eig_sweeps_total += sweeps;
+          s.eig_sweeps_total += sweeps.f64;
+          s.eig_sweeps32 += sweeps.f32;
           s.eig_rotations += sh_rot;
         }
         __syncthreads();
