@@ -39,7 +39,7 @@ namespace cmaes_gb300 {
 
 constexpr int kRfNT = 512, kRfW = kRfNT / 32;
 constexpr int kRfK = 32;                                   // k per step of the left operand
-constexpr int kRfCols = 20;                                // columns of a CTA: ceil(kEigMixedMaxN / 8)
+constexpr int kRfCols = 20;                                // most columns of a CTA: ceil(kEigMixedMaxN / 8)
 constexpr int kRfRow = (kEigMixedMaxN + 31) / 32;          // elements of a column per lane
 constexpr int kRfPre = kRfK * kEigMixedMaxN / kRfNT;       // left elements per thread and step
 constexpr double kRfSep = 0x1p-10;                         // largest first-order correction
@@ -79,10 +79,11 @@ struct Rf {
 
 // One product over the cluster's columns. SYM: only i <= j. NA right operands
 // (R0 and R1) share the left one. rows: M(i, k) at M[i + L k], else M(k, i) at
-// M[k + L i]. CT columns and two rows per thread; epi(i, c, v0, v1). HI: h h only.
+// M[k + L i]. CT columns and two rows per thread; epi(i, c, v0, v1). HI: h h only,
+// as for every column of Ra whose scale is at most `tiny`.
 template <int CT, int NA, bool SYM, bool HI, class EPI>
 __device__ __forceinline__ void rf_product(const Rf& f, const int2* M, long long L, bool rows, const int2* Ra,
-                                           const int2* Rb, const int* el, const int* ea, const int* eb,
+                                           const int2* Rb, const int* el, const int* ea, const int* eb, int tiny,
                                            const EPI& epi) {
   const int n = f.n, tid = f.tid, lane = f.lane, warp = f.warp;
   // this thread's outputs: rows r and r + H of columns c0 .. c0 + CT - 1
@@ -198,7 +199,7 @@ __device__ __forceinline__ void rf_product(const Rf& f, const int2* M, long long
 #pragma unroll
       for (int c = 0; c < CT; ++c) {
         if (c0 + c >= f.ncl || (SYM && i > f.col(c0 + c))) continue;
-        epi(i, c0 + c, value(hh[0][u][c], mid[0][u][c], e, ea[c0 + c]),
+        epi(i, c0 + c, value(hh[0][u][c], HI || ea[c0 + c] <= tiny ? 0 : mid[0][u][c], e, ea[c0 + c]),
             NA == 2 ? value(hh[NA - 1][u][c], mid[NA - 1][u][c], e, eb[c0 + c]) : 0.0);
       }
     }
@@ -207,19 +208,19 @@ __device__ __forceinline__ void rf_product(const Rf& f, const int2* M, long long
 
 template <bool HI, class EPI>
 __device__ __forceinline__ void rf_full(const Rf& f, const int2* M, long long L, bool rows, const int2* R,
-                                        const int* el, const int* er, const EPI& epi) {
+                                        const int* el, const int* er, int tiny, const EPI& epi) {
   const int H = (f.n + 1) >> 1;
-  if (H * f.ncl <= kRfNT) rf_product<1, 1, false, HI>(f, M, L, rows, R, R, el, er, er, epi);
-  else if (H * ((f.ncl + 1) >> 1) <= kRfNT) rf_product<2, 1, false, HI>(f, M, L, rows, R, R, el, er, er, epi);
-  else rf_product<4, 1, false, HI>(f, M, L, rows, R, R, el, er, er, epi);
+  if (H * f.ncl <= kRfNT) rf_product<1, 1, false, HI>(f, M, L, rows, R, R, el, er, er, tiny, epi);
+  else if (H * ((f.ncl + 1) >> 1) <= kRfNT) rf_product<2, 1, false, HI>(f, M, L, rows, R, R, el, er, er, tiny, epi);
+  else rf_product<4, 1, false, HI>(f, M, L, rows, R, R, el, er, er, tiny, epi);
 }
 template <int NA, class EPI>
 __device__ __forceinline__ void rf_sym(const Rf& f, const int2* M, long long L, const int2* Ra, const int2* Rb,
                                        const int* el, const int* ea, const int* eb, const EPI& epi) {
   int items = 0;
   for (int c = 0; c < f.ncl; ++c) items += (f.col(c) + 2) >> 1;
-  if (items <= kRfNT) rf_product<1, NA, true, false>(f, M, L, false, Ra, Rb, el, ea, eb, epi);
-  else rf_product<2, NA, true, false>(f, M, L, false, Ra, Rb, el, ea, eb, epi);
+  if (items <= kRfNT) rf_product<1, NA, true, false>(f, M, L, false, Ra, Rb, el, ea, eb, 0, epi);
+  else rf_product<2, NA, true, false>(f, M, L, false, Ra, Rb, el, ea, eb, 0, epi);
 }
 
 // x 2^(E - 1022) by its exponent field; below the normal range it is zero, above it
@@ -323,12 +324,14 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
       rf_integers(f, f.T, f.ex + cur * n, f.R1, f.e1, nullptr, L, nullptr, cl);
       __syncthreads();
       // corrections this small (the second step's and Newton-Schulz's, as a rule): the
-      // products left out are below sqrt(n) 2^-63, an entry of X is rounded at 2^-56
+      // products left out are below sqrt(n) 2^-63, an entry of X is rounded at 2^-56. Each
+      // column decides for itself, so that which CTA has it does not show.
+      constexpr int tiny = 1022 - kRfTiny;
       auto add = [&](int i, int c, double v, double) { f.X[c * f.ns + i] += v; };
-      if (__syncthreads_or(f.tid < f.ncl && f.e1[f.tid] > 1022 - kRfTiny))
-        rf_full<false>(f, XL[cur], L, true, f.R1, nullptr, f.e1, add);
+      if (__syncthreads_or(f.tid < f.ncl && f.e1[f.tid] > tiny))
+        rf_full<false>(f, XL[cur], L, true, f.R1, nullptr, f.e1, tiny, add);
       else
-        rf_full<true>(f, XL[cur], L, true, f.R1, nullptr, f.e1, add);
+        rf_full<true>(f, XL[cur], L, true, f.R1, nullptr, f.e1, tiny, add);
       __syncthreads();
       cur ^= 1;
       rf_integers(f, f.X, nullptr, f.R0, f.e0, XL[cur], L, f.ex + cur * n, cl);
@@ -353,7 +356,7 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
       continue;
     }
     // T = C X
-    rf_full<false>(f, CL, L, false, f.R0, f.ec, f.e0, [&](int i, int c, double v, double) { f.T[c * f.ns + i] = v; });
+    rf_full<false>(f, CL, L, false, f.R0, f.ec, f.e0, 0, [&](int i, int c, double v, double) { f.T[c * f.ns + i] = v; });
     __syncthreads();
     rf_integers(f, f.T, nullptr, f.R1, f.e1, nullptr, L, nullptr, cl);
     __syncthreads();

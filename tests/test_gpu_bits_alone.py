@@ -130,3 +130,24 @@ def test_many_small_searches():
         finally:
             eng.cmaes_destroy(h)
     same(*got)
+
+
+@pytest.mark.parametrize("precision", [eng.FP64, eng.MIXED_TF32], ids=["fp64", "tf32"])
+@pytest.mark.parametrize("n,count", [(33, 100), (40, 12), (40, 200), (41, 60), (80, 100), (81, 20), (160, 30)])
+def test_jacobi_route(n, count, precision):
+    """With clusters of 16 CTAs alone, and of 8, 4 and 2 in a batch."""
+    d = W.random_state(n, SEED, 7, cond=30.0)
+    got = []
+    for searches in (1, count):
+        opt = eng.cmaes_default_options(eig_every=1, stop_mask=0, precision=precision)
+        h = eng.cmaes_create_batch([n] * searches, [12] * searches, [np.zeros(n)] * searches, [1.0] * searches, SEED, opt)
+        try:
+            for i in range(searches):
+                eng.cmaes_set_problem(h, i, eng.OBJ_SPHERE, xstar=np.ones(n))
+            eng.cmaes_set_state(h, 0, dict(n=n, lam=12, sigma=0.3, m=d["m"], ps=d["ps"], pc=d["pc"], C=d["C"],
+                                           B=d["B"], D=d["D"], gen=5))
+            eng.cmaes_step_batch(h, 3)
+            got.append((eng.cmaes_get_state(h, 0, n), eng.cmaes_get_generation(h, 0, n)))
+        finally:
+            eng.cmaes_destroy(h)
+    same(*got)
