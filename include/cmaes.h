@@ -92,18 +92,22 @@ typedef enum {
 #define CMAES_STOP_NONFINITE 128    /* m, sigma or diag C not finite           */
 #define CMAES_STOP_ALL 255
 
-/* Eigensolver of C = B D^2 B^T for 32 < n <= 4096 (smaller n always use a
- * one-CTA FP64 Jacobi; larger n a warm-started FP64 Jacobi on one CTA).
+/* Eigensolver of C = B D^2 B^T for 32 < n <= 4096 (smaller n always take the
+ * JACOBI method in one CTA; larger n a warm-started FP64 Jacobi on one CTA).
  *   JACOBI: warm-started from the previous basis; cyclic Jacobi sweeps in
  *     FP32, FP64 accuracy recovered by two Ogita-Aishima refinement steps
  *     and a Newton-Schulz step, then an FP64 Jacobi cleanup.
  *   TRIDIAGONAL: Householder reduction to tridiagonal form, the route of
  *     LAPACK's dsyev that the paper calls (§3.1): bisection for the
  *     eigenvalues, inverse iteration for the eigenvectors, Newton-Schulz
- *     steps for orthogonality, all in FP64.
+ *     steps for orthogonality. FP64-accurate; the reduction is in 64-bit
+ *     fixed point, the long products are exact sums on the tensor cores.
  *   AUTO (default): JACOBI up to n = 160 (its FP32 sweeps fit one CTA's
- *     shared memory and beat the reduction's n sequential FP64 steps there),
- *     TRIDIAGONAL above (the Jacobi sweeps' n steps each then span the GPU). */
+ *     shared memory and beat the reduction's n sequential steps there),
+ *     TRIDIAGONAL above (the Jacobi sweeps' n steps each then span the GPU).
+ * Either gives what LAPACK's dsyev does: B orthonormal to rounding and
+ * B D^2 B^T = C to rounding of ||C||; the smallest eigenvalues of a graded C
+ * are not promised to their own relative accuracy. */
 typedef enum {
     CMAES_EIG_AUTO = 0,
     CMAES_EIG_JACOBI = 1,
@@ -279,8 +283,8 @@ cmaes_status cmaes_phase_times(cmaes_t h, double* ms, long long* launches,
 
 /* Work done by the eigensolver of search s since creation: decompositions,
  * FP64 Jacobi sweeps, plane rotations applied by them, and the FP32 Jacobi
- * sweeps that precede them on the refined route (32 < n <= 4096, every handle
- * precision; zero for other n). Any pointer may be NULL. Synchronises. */
+ * sweeps that precede them (every handle precision; zero on the tridiagonal
+ * route and for n > 4096). Any pointer may be NULL. Synchronises. */
 cmaes_status cmaes_eig_stats(cmaes_t h, int s, long long* decompositions,
                              long long* sweeps, long long* rotations,
                              long long* sweeps32);
