@@ -90,6 +90,7 @@ struct cmaes_s {
   size_t small_smem = 0;
   bool small_dense = false;    // more such searches than wide CTAs fit
   int max_n_refine = 0;        // largest n <= kEigMixedMaxN on the refined Jacobi route
+  RefinePlan refine_plan;      // its clusters
   int max_n_big = 0;           // largest n of the searches whose FP32 Jacobi runs over many CTAs
   // tridiagonal route: largest n, the CTA -> (search, member, group size) table
   // of the cooperative reduction, and one barrier counter per search
@@ -363,9 +364,9 @@ static void enqueue_eig(cmaes_t h, int s0, int s1, cudaStream_t st) {
   {
     TileMap tfl = h->tiles(TK_FLAT, s0, s1);
     TileMap tsy = h->tiles(TK_FLATSYM, s0, s1);
-    int nl = launch_eig_mixed_head(h->dS, tfl, tsy, s0, s1, h->max_n_refine, st);
+    int nl = launch_eig_mixed_head(h->dS, tfl, tsy, s0, s1, h->max_n_refine, h->refine_plan, st);
     if (h->max_n_big > 0) nl += enqueue_jacobi32_big(h, s0, s1, st);
-    nl += launch_eig_mixed_tail(h->dS, tfl, tsy, s0, s1, h->max_n_refine, h->mixed, st);
+    nl += launch_eig_mixed_tail(h->dS, tfl, tsy, s0, s1, h->max_n_refine, h->refine_plan, h->mixed, st);
     h->launches += nl;
     h->phase_launch[kPhaseEig] += nl;
   }
@@ -753,6 +754,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     }                                                                                            \
   } while (0)
   CREATE_TRY(set_smem_limits());
+  if (h->max_n_refine > 0) h->refine_plan = refine_plan(h->max_n_refine);
   if (h->all_small) CREATE_TRY(small_generations_dense(count, h->small_smem, &h->small_dense));
   CREATE_TRY(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
   size_t state_max = 0;

@@ -239,13 +239,19 @@ int tiles_flat(int n);
 // 32-row blocks of the FP64 re-evaluation of the best point (one partial sum each)
 __host__ __device__ inline int tiles_reeval(int n) { return (n + 31) / 32; }
 int tiles_flat_sym(int n);
+struct RefinePlan {
+  static constexpr int kTop = 16, kSizes = 4;  // clusters of 16, 8, 4 and 2 CTAs
+  int fit[kSizes] = {0, 0, 0, 0}, least = 8;   // of each, how many at once; the smallest that holds n columns
+};
+RefinePlan refine_plan(int max_n);  // kernels_eig_refine.cu
 // the refined route in two parts around the many-CTA FP32 Jacobi: the
 // warm-start products (and the one-CTA FP32 Jacobi), then the refinement
-int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, cudaStream_t st);
-int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, bool mixed,
-                          cudaStream_t st);
+int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small,
+                          const RefinePlan& plan, cudaStream_t st);
+int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small,
+                          const RefinePlan& plan, bool mixed, cudaStream_t st);
 // the products of that route for n <= kEigMixedMaxN (kernels_eig_refine.cu)
-void launch_eig_refine(Search* S, int s0, int s1, int max_n, int head, cudaStream_t st);
+void launch_eig_refine(Search* S, int s0, int s1, int max_n, const RefinePlan& plan, int head, cudaStream_t st);
 // launchers (kernels_eig_big.cu)
 int tiles_jb_blocks(int n);
 int tiles_jb_load(int n);

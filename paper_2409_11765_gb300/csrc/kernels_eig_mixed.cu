@@ -1155,7 +1155,8 @@ int pair_rounds_smem_bytes(int n) { return (n + 1) * n * 8; }
 
 
 // max_small: the largest n <= kE32Max of this route (0: none).
-int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, cudaStream_t st) {
+int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small,
+                          const RefinePlan& plan, cudaStream_t st) {
   int nl = 0;
   if (s1 <= s0) return nl;
   if (tflat.total > 0) {
@@ -1164,7 +1165,7 @@ int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1
     nl += 2;
   }
   if (max_small > 0) {
-    launch_eig_refine(S, s0, s1, max_small, 1, st);
+    launch_eig_refine(S, s0, s1, max_small, plan, 1, st);
     launch_jacobi32(S, s0, s1, max_small, st);
     k_jlog_apply<<<dim3(ceil_div(max_small, kLogRows), s1 - s0), kLogRows * 32, 0, st>>>(S, s0);
     nl += 3;
@@ -1172,8 +1173,8 @@ int launch_eig_mixed_head(Search* S, TileMap tflat, TileMap tsym, int s0, int s1
   return nl;
 }
 
-int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small, bool mixed,
-                          cudaStream_t st) {
+int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1, int max_small,
+                          const RefinePlan& plan, bool mixed, cudaStream_t st) {
   int nl = 0;
   if (s1 <= s0) return nl;
   if (tflat.total > 0) {
@@ -1200,7 +1201,7 @@ int launch_eig_mixed_tail(Search* S, TileMap tflat, TileMap tsym, int s0, int s1
     sym(OA_A);
   }
   if (max_small > 0) {
-    launch_eig_refine(S, s0, s1, max_small, 0, st);
+    launch_eig_refine(S, s0, s1, max_small, plan, 0, st);
     ++nl;
     if (!mixed && max_small < kRoundsMinN) return nl;
     k_pair_rounds<<<s1 - s0, kRoundsNT, pair_rounds_smem_bytes(max_small), st>>>(S, s0);

@@ -408,33 +408,51 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
   }
 }
 
-// Clusters of 16 where those of all searches run side by side (seven did), else of 8:
-// the decomposition of four searches of n = 100 took 425 us with 16 and 480 with 8, that
-// of ten, whose clusters of 16 no longer fit at once, 741 and 638.
-void launch_eig_refine(Search* S, int s0, int s1, int max_n, int head, cudaStream_t st) {
-  if (s1 <= s0 || max_n <= kJacobiSmallN) return;
+static cudaLaunchConfig_t refine_config(int searches, int max_n, int cs, cudaLaunchAttribute* at) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = static_cast<unsigned>(cs);
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cfg.blockDim = dim3(kRfNT);
-  cfg.stream = st;
-  auto size = [&](int cs) {
-    at[0].val.clusterDim.x = static_cast<unsigned>(cs);
-    cfg.gridDim = dim3(static_cast<unsigned>((s1 - s0) * cs));
-    cfg.dynamicSmemBytes = rf_layout(max_n, cs).bytes;
-  };
-  // (a device that refuses clusters of 16 reports that none fits)
-  int fit = 0;
-  size(16);
-  if (cudaOccupancyMaxActiveClusters(&fit, k_eig_refine, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    fit = 0;
+  cfg.gridDim = dim3(static_cast<unsigned>(searches * cs));
+  cfg.dynamicSmemBytes = rf_layout(max_n, cs).bytes;
+  return cfg;
+}
+
+// How many clusters of each size run side by side (none of a size that the device
+// refuses); a CTA holds at most kRfCols columns.
+RefinePlan refine_plan(int max_n) {
+  RefinePlan plan;
+  cudaLaunchAttribute at[1];
+  for (int q = 0; q < RefinePlan::kSizes; ++q) {
+    const int cs = RefinePlan::kTop >> q;
+    plan.fit[q] = 0;
+    if (cs * kRfCols < max_n) break;
+    const cudaLaunchConfig_t cfg = refine_config(1, max_n, cs, at);
+    if (cudaOccupancyMaxActiveClusters(&plan.fit[q], k_eig_refine, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      plan.fit[q] = 0;
+    }
+    plan.least = cs;
   }
-  if (fit < s1 - s0) size(8);
+  return plan;
+}
+
+// The largest clusters of which those of all searches run side by side, else the
+// smallest that hold n columns, which pass the fewest barriers: the results do not depend
+// on it. Four searches of n = 100, the decomposition: clusters of 16 425 us, of 8 480;
+// ten, of which seven fit with 16: 741 and 638. Two generations of 300 searches of n = 40:
+// clusters of 8 3.74 ms, of 2 1.87; of 1000 of n = 33: 11.8 and 5.3.
+void launch_eig_refine(Search* S, int s0, int s1, int max_n, const RefinePlan& plan, int head, cudaStream_t st) {
+  if (s1 <= s0 || max_n <= kJacobiSmallN) return;
+  int cs = plan.least;
+  for (int q = RefinePlan::kSizes - 1; q >= 0; --q)
+    if (plan.fit[q] >= s1 - s0 && (RefinePlan::kTop >> q) > cs) cs = RefinePlan::kTop >> q;
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg = refine_config(s1 - s0, max_n, cs, at);
+  cfg.stream = st;
   cudaLaunchKernelEx(&cfg, k_eig_refine, S, s0, head);
 }
 
