@@ -555,8 +555,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_trd_reduce(Search* S, const in
         const bool pub = j1 == k + 1;
         long long h1 = 0, h2 = 0, mid1 = 0, mid2 = 0;
         int i0 = base + unit * ch + lane;
+        const int live = min(batches, (n - base - unit * ch + 127) >> 7);  // batches with a row below n
 #pragma unroll 1
-        for (int bt = 0; bt < batches; ++bt, i0 += 128) {
+        for (int bt = 0; bt < live; ++bt, i0 += 128) {
           long long a1[4], a2[4], ma1 = 0, mb1 = 0, ma2 = 0, mb2 = 0;
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
