@@ -551,6 +551,14 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_trd_reduce(Search* S, const in
         const bool two = NCOL == 2 && c1 + 1 < nc;
         long long* const A1 = column(m0 + c1);
         long long* const A2 = column(m0 + c1 + (two ? 1 : 0));
+        if (!SM && un + NW < groups * chunks) {
+          // the warp's next unit on its way to L2 (rows r0 .. below n of its columns; 16-byte
+          // pieces from a multiple of 32 rows): 40 searches of n = 2000 391 -> 366 ms
+          const int nu = un + NW, nch = nu / groups, nc1 = NCOL * (nu - nch * groups), r0 = base + unit * nch;
+          const unsigned bytes = static_cast<unsigned>(min(unit, n - r0) * 8) & ~15u;
+          if (lane < NCOL && nc1 + lane < nc && bytes != 0u)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(column(m0 + nc1 + lane) + r0), "r"(bytes) : "memory");
+        }
         const int4 x1 = vw[j1], x2 = vw[two ? j1 + G : j1];
         const bool pub = j1 == k + 1;
         long long h1 = 0, h2 = 0, mid1 = 0, mid2 = 0;
