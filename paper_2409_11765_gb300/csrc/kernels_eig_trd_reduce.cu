@@ -422,23 +422,27 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_trd_reduce(Search* S, const in
         tmx = max(tmx, static_cast<unsigned>((P < 0 ? -P : P) >> 32));
       }
       __syncwarp();
-      // p . v in 2 q, exact but for the cut of each thread's share
-      const u64 pv = warp_sum_u64(static_cast<u64>((thi << 7) + static_cast<long long>(tlo >> 44)));
+      // p . v in its high words and, cut for each row alone, its low ones: the sums do
+      // not depend on which thread has a row
+      const u64 pvh = warp_sum_u64(static_cast<u64>(thi)), pvl = warp_sum_u64(tlo);
       tmx = __reduce_max_sync(0xffffffffu, tmx);
       if (lane == 0) {
-        redi[0][warp] = pv;
+        redi[0][warp] = pvh;
+        redi[1][warp] = pvl;
         redm[warp] = tmx;
       }
       if (!__syncthreads_and(ok)) return;
     }
     if (warp == 0) {  // half = (tau / 2) p . v of p = tau A v; the scale of w from |w| <= tau max|A v| + |half|
-      long long pv = 0;
+      u64 pvh = 0ull, pvl = 0ull;
       unsigned mx = 0u;
 #pragma unroll
       for (int w = 0; w < NW; ++w) {
-        pv += static_cast<long long>(redi[0][w]);
+        pvh += redi[0][w];
+        pvl += redi[1][w];
         mx = max(mx, redm[w]);
       }
+      const long long pv = static_cast<long long>((pvh << 7) + (pvl >> 44));
       // p . v is in 2 q: half = tau^2 pv q, from pv 2^zp < 2^62 and tau^2 in 2^-60
       const u64 ap = static_cast<u64>(pv < 0 ? -pv : pv);
       const int zp = ap != 0ull ? __clzll(static_cast<long long>(ap)) - 2 : 61, eh = 66 - zp;

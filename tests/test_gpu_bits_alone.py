@@ -35,7 +35,9 @@ def first_search(ns, precision, kind):
 @pytest.mark.parametrize("n,kind", [(33, "spread"), (200, "spread"), (257, "wide"), (300, "rank-one")])
 def test_tridiagonal_route(n, kind, precision):
     alone = first_search([n], precision, kind)
-    for neighbours in ([400], [400] * 4, [400] * 11, [400] * 36):  # 16, 8, 4 lanes and 1 per eigenvalue
+    # 16, 8, 4 lanes and 1 per eigenvalue; the reduction's columns in shared memory and in HBM,
+    # CTAs of 512 and of 256 threads, one launch and several
+    for neighbours in ([400], [400] * 4, [400] * 11, [400] * 36, [64] * 140, [64] * 320, [600] * 100):
         batch = first_search([n] + neighbours, precision, kind)
         for key in ("m", "ps", "pc", "C", "B", "D"):
             assert np.array_equal(alone[key], batch[key]), (len(neighbours), key)
