@@ -208,6 +208,120 @@ static size_t state_bytes(const Search& x) {
   return state_layout(x.n, x.hist_cap, x.n <= kStateMaxN).total * sizeof(double);
 }
 
+// The cooperative launches of the tridiagonal reduction: which searches each has, with
+// how many CTAs.
+struct TrdShares {
+  TrdReducePlan launch;
+  std::vector<std::vector<int>> parts;  // launches that follow one another (a part of more CTAs than fit: several)
+  std::vector<int> G;                   // CTAs of a search
+  long long budget = 0;                 // CTAs of a launch (0: the form cannot be resident)
+  double time = INFINITY;               // modelled, ns
+
+  // f(searches) for every launch; a launch never splits a search's CTAs
+  template <class F>
+  void chunks(const F& f) const {
+    for (const std::vector<int>& part : parts) {
+      std::vector<int> now;
+      long long ctas = 0;
+      for (int s : part) {
+        if (ctas + G[s] > budget) {
+          f(now);
+          now.clear();
+          ctas = 0;
+        }
+        now.push_back(s);
+        ctas += G[s];
+      }
+      if (!now.empty()) f(now);
+    }
+  }
+};
+
+// CTAs of a launch are shared in proportion to the work n^3, so that its searches end
+// together, one at least and n / kTrdCols columns at most.
+static void share_ctas(const std::vector<Search>& hs, int sms, TrdShares* p) {
+  constexpr int kTrdCols = 4;
+  p->G.assign(hs.size(), 0);
+  for (const std::vector<int>& part : p->parts) {
+    double work = 0.0;
+    long long caps = 0;
+    for (int s : part) {
+      const double n = hs[s].n;
+      work += n * n * n;
+      caps += std::min(hs[s].n / kTrdCols, sms);
+    }
+    const double spare = static_cast<double>(std::max<long long>(0, p->budget - static_cast<long long>(part.size())));
+    for (int s : part) {
+      const double n = hs[s].n;
+      const int cap = std::min(hs[s].n / kTrdCols, sms);
+      p->G[s] = caps <= p->budget ? cap : std::min(cap, 1 + static_cast<int>(spare * (n * n * n / work) * (1.0 + 1e-12)));
+    }
+  }
+}
+
+// One launch with the columns in shared memory where every search has its CTAs with one
+// per SM and they hold them. Else the columns are in HBM, and of one CTA of 512 threads per
+// SM or two of 256, in one launch or in several of `each` searches, largest first, the
+// form with the least time by a model of it: a launch lasts as long as its longest search,
+// n^3 / 3 elements over G CTAs and n exchanges. (Together in one launch the large searches
+// of an uneven batch get a CTA or two and go on long after the others: the stage of 150
+// searches of n = 50 .. 2000 929 ms in one launch, 288 as chosen; of 300 searches of
+// n = 300 11.4 ms in one and 19.1 in eight.) The bits do not depend on any of it.
+static TrdShares plan_reduction(const std::vector<Search>& hs, int sms) {
+  std::vector<int> order;
+  for (int s = 0; s < static_cast<int>(hs.size()); ++s)
+    if (hs[s].trd) order.push_back(s);
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return hs[x].n > hs[y].n; });
+  auto smem_of = [&](const TrdShares& p, int in_smem) {
+    size_t b = 0;
+    for (int s : order) b = std::max(b, trd_reduce_smem(hs[s].n, p.G[s], in_smem));
+    return b;
+  };
+  TrdShares best;
+  best.parts = {order};
+  best.budget = sms;
+  share_ctas(hs, sms, &best);
+  best.launch.in_smem = 1;
+  best.launch.smem = smem_of(best, 1);
+  long long ctas = 0;
+  for (int s : order) ctas += best.G[s];
+  if (ctas <= sms && trd_reduce_blocks_per_sm(best.launch.smem, 1, 512) >= 1) return best;
+  best = TrdShares{};
+  for (const int threads : {512, 256}) {
+    for (const size_t each : {order.size(), static_cast<size_t>(sms), static_cast<size_t>(sms) / 2,
+                              static_cast<size_t>(sms) / 4, static_cast<size_t>(sms) / 8}) {
+      if (each == 0 || each > order.size()) continue;
+      TrdShares p;
+      for (size_t i = 0; i < order.size(); i += each)
+        p.parts.emplace_back(order.begin() + i, order.begin() + std::min(order.size(), i + each));
+      p.launch.threads = threads;
+      int per_sm = 512 / threads;
+      for (int fit = 0; per_sm > 0; per_sm = fit) {  // (the accumulators' size depends on the shares)
+        p.budget = static_cast<long long>(per_sm) * sms;
+        share_ctas(hs, sms, &p);
+        p.launch.smem = smem_of(p, 0);
+        fit = trd_reduce_blocks_per_sm(p.launch.smem, 0, threads);
+        if (fit >= per_sm) break;
+      }
+      if (per_sm < 1) continue;
+      // measured: ns an element of a CTA, with a whole SM or half of one, and an exchange
+      const double per_element = per_sm == 1 ? 0.52 : 0.96;
+      p.time = 0.0;
+      p.chunks([&](const std::vector<int>& searches) {
+        double longest = 0.0;
+        for (int s : searches) {
+          const double n = hs[s].n;
+          const double per_step = threads == 512 ? 2400.0 : 2600.0 + 1.9 * n;
+          longest = std::max(longest, n * n * n / 3.0 / p.G[s] * per_element + n * per_step);
+        }
+        p.time += longest;
+      });
+      if (p.time < best.time) best = p;
+    }
+  }
+  return best;
+}
+
 static cmaes_status read_search(cmaes_t h, int s, Search* out) {
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   cmaes_status r = check_device_status(h);
@@ -845,102 +959,20 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
     CREATE_TRY(cudaGetDevice(&dev));
     CREATE_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     trd_set_attributes();
-    // CTAs per search: at least kTrdCols columns each. When every search can
-    // have that many with one CTA per SM the columns stay in shared memory if
-    // they fit; otherwise the resident CTAs are shared in proportion to the
-    // work n^3 (so that the searches end together), one CTA at least, first
-    // with one CTA per SM and the columns in shared memory, then with as many
-    // as fit and the columns in HBM.
-    constexpr int kTrdCols = 4;
-    std::vector<int> G(count, 0);
-    std::vector<std::vector<int>> parts(1);  // the searches of each launch
-    for (int s = 0; s < count; ++s)
-      if (h->hs[s].trd) parts[0].push_back(s);
-    const size_t nact = parts[0].size();
-    auto share = [&](long long budget) {
-      for (const std::vector<int>& part : parts) {
-        double wsum = 0.0;
-        long long caps = 0;
-        for (int s : part) {
-          const double n = h->hs[s].n;
-          wsum += n * n * n;
-          caps += std::min<long long>(h->hs[s].n / kTrdCols, sms);
-        }
-        const long long spare = std::max<long long>(0, budget - static_cast<long long>(part.size()));
-        for (int s : part) {
-          const double n = h->hs[s].n;
-          const long long cap = std::min<long long>(h->hs[s].n / kTrdCols, sms);
-          G[s] = caps <= budget ? static_cast<int>(cap)
-                                : static_cast<int>(std::min(cap, 1 + static_cast<long long>(spare * (n * n * n / wsum))));
-        }
-      }
-    };
-    auto smem_of = [&](int in_smem) {
-      size_t b = 0;
-      for (int s = 0; s < count; ++s)
-        if (h->hs[s].trd) b = std::max(b, trd_reduce_smem(h->hs[s].n, G[s], in_smem));
-      return b;
-    };
-    long long budget = sms;
-    share(budget);
-    long long ctas = 0;
-    for (int s = 0; s < count; ++s) ctas += G[s];
-    h->trd_plan.smem = smem_of(1);
-    h->trd_plan.in_smem = ctas <= sms && trd_reduce_blocks_per_sm(h->trd_plan.smem, 1, 512) >= 1;
-    if (!h->trd_plan.in_smem) {
-      h->trd_plan.smem = smem_of(0);
-      if (ctas > sms || trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 512) < 1) h->trd_plan.threads = 256;
-    }
-    if (h->trd_plan.threads == 256) {
-      // Where so many searches share the GPU that the large ones get a CTA or two, a few
-      // CTAs would still be at those when the rest has finished. Then launches of at most
-      // an eighth as many searches as there are CTAs follow one another, largest
-      // searches first: together they keep every SM busy to the end. (256 searches of
-      // n = 50 .. 2000: 3453 ms in one launch, 572 in several. Searches small enough
-      // that a step's exchange takes longer than its CTA's columns stay in one.)
-      share(2 * sms);
-      double most = 0.0;
-      for (int s : parts[0]) most = std::max(most, static_cast<double>(h->hs[s].n) * h->hs[s].n / G[s]);
-      if (nact > static_cast<size_t>(sms) / 2 && most > 65536.0) {
-        std::vector<int> order = parts[0];
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return h->hs[x].n > h->hs[y].n; });
-        parts.clear();
-        const size_t each = std::max<size_t>(1, static_cast<size_t>(sms) / 4);
-        for (size_t i = 0; i < order.size(); i += each)
-          parts.emplace_back(order.begin() + i, order.begin() + std::min(order.size(), i + each));
-        share(2 * sms);
-        h->trd_plan.smem = smem_of(0);
-      }
-      // (the accumulators' size depends on the shares)
-      int per_sm = trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 256);
-      for (int pass = 0; pass < 2; ++pass) {
-        budget = static_cast<long long>(per_sm) * sms;
-        share(budget);
-        h->trd_plan.smem = smem_of(0);
-        per_sm = std::min(per_sm, trd_reduce_blocks_per_sm(h->trd_plan.smem, 0, 256));
-      }
-      budget = static_cast<long long>(per_sm) * sms;
-    }
-    if (budget < 1) {
+    TrdShares plan = plan_reduction(h->hs, sms);
+    if (plan.budget < 1) {
       set_error(h, CMAES_EUNSUPPORTED, "the tridiagonal reduction cannot be resident on this device");
       return fail(CMAES_EUNSUPPORTED);
     }
-    std::vector<int4> grp;  // launches of at most `budget` CTAs never split a group
+    h->trd_plan = plan.launch;
+    std::vector<int4> grp;
     h->trd_chunks.clear();
-    int chunk_start = 0;
-    auto close = [&] {
-      if (static_cast<int>(grp.size()) > chunk_start)
-        h->trd_chunks.push_back(TrdChunk{chunk_start, static_cast<int>(grp.size()) - chunk_start});
-      chunk_start = static_cast<int>(grp.size());
-    };
-    for (const std::vector<int>& part : parts) {
-      for (int s : part) {
-        const int Gs = static_cast<int>(std::min<long long>(G[s], budget));
-        if (static_cast<long long>(grp.size()) + Gs - chunk_start > budget) close();
-        for (int r = 0; r < Gs; ++r) grp.push_back(make_int4(s, r, Gs, 0));
-      }
-      close();
-    }
+    plan.chunks([&](const std::vector<int>& searches) {
+      const int start = static_cast<int>(grp.size());
+      for (int s : searches)
+        for (int r = 0; r < plan.G[s]; ++r) grp.push_back(make_int4(s, r, plan.G[s], 0));
+      h->trd_chunks.push_back(TrdChunk{start, static_cast<int>(grp.size()) - start});
+    });
     h->trd_grp_blocks = static_cast<int>(grp.size());
     long long eig_total = 0;
     for (int s = 0; s < count; ++s)
