@@ -62,16 +62,6 @@ constexpr int kRedPolls = 1 << 21;  // polls of a word before the wait gives up 
 constexpr int kRedPad = 1024;       // zero rows after the limb arrays: the largest work unit
 constexpr double kRedRange = 1.75;  // |a| <= kRedRange 2^62
 
-// rint(x 2^sh) for |x| 2^sh < 2^62, on the integer pipe
-__device__ __forceinline__ long long to_fixed(double x, int sh) {
-  const long long b = __double_as_longlong(x);
-  const int e = static_cast<int>((b >> 52) & 0x7ff) - 1075 + sh;
-  u64 m = (static_cast<u64>(b) & 0xfffffffffffffull) | 0x10000000000000ull;
-  if (e >= 0) m <<= e;
-  else m = e < -54 ? 0ull : (m + (1ull << (-e - 1))) >> -e;
-  return b < 0 ? -static_cast<long long>(m) : static_cast<long long>(m);
-}
-
 __device__ __forceinline__ int2 limbs30(long long f) {
   const int h = static_cast<int>((f + (1LL << 29)) >> 30);
   return make_int2(h, static_cast<int>(f - (static_cast<long long>(h) << 30)));
