@@ -234,7 +234,12 @@ DTYPE = {"fp64": "f64", "tf32": "tf32+f64", "bf16": "bf16+f64"}
 # for the sources of that stage's kernels as they were measured (a SHA-256 of
 # the code without comments, stage_sources_sha): after any change to them the
 # roofline's traffic is null until it is measured again.
-KERNEL_TRAFFIC = {}
+#   reduction: dram__bytes_read.sum + dram__bytes_write.sum of the six launches of
+#   k_trd_reduce a generation of the 256-search batch has (one pass each), the mean
+#   of the ten timed generations of two handles.
+KERNEL_TRAFFIC = {
+    "reduction": {"bytes_per_step": 1.877e12, "workload": "batch256-n50..2000", "sources_sha256_16": "9003ca16ca600d7f"},
+}
 
 # The code each stage's kernels are built from: the reduction's source up to
 # its host part (its kernel and every helper it calls) and the headers it
@@ -406,17 +411,34 @@ def measure(args, wl, prec, world, rank, dist, want_clocks, eig_method, secondar
 
 
 def stage_flops(decomps):
-    """Algorithmic flops of the eigendecompositions per stage, from the
-    decompositions done. Householder reduction: LAPACK's 4/3 n^3 for dsytrd
-    (one pass of the integer pipes over the remaining columns per step).
-    Back-transformation: 2 n^3 (dormtr's count) for n <= 256, where it runs in
-    FP64; above, on the tensor cores (0 FP64 flops). The eigenvalue and
-    eigenvector stages are O(n^2) per decomposition and the Newton-Schulz
-    orthogonalisation is not part of the minimal method (0)."""
-    red = sum(k * 4.0 / 3.0 * n ** 3 for n, k in decomps.items())
+    """Algorithmic FP64 flops of the eigendecompositions per stage, from the
+    decompositions done. The Householder reduction has none in its steps (its
+    bound is reduction_roof's). Back-transformation: 2 n^3 (dormtr's count) for
+    n <= 256, where it runs in FP64; above, on the tensor cores (0 FP64 flops).
+    The eigenvalue and eigenvector stages are O(n^2) per decomposition and the
+    Newton-Schulz orthogonalisation is not part of the minimal method (0)."""
     bt = sum(k * 2.0 * n ** 3 for n, k in decomps.items() if n <= 256)
-    return {"reduction": red, "backtransform": bt, "eigenvalues": 0.0, "eigenvectors": 0.0,
-            "orthogonalisation": 0.0}
+    return {"backtransform": bt, "eigenvalues": 0.0, "eigenvectors": 0.0, "orthogonalisation": 0.0}
+
+
+# 32 x 32 + 64-bit integer multiply-adds a clock and SM, measured.
+IMAD_PER_CLOCK = 28.0
+# What the reduction's resident CTAs hold in shared memory, bytes an SM.
+REDUCTION_SMEM = 200e3
+
+
+def reduction_roof(wl, decomps, steps, hbm_gbs, sms, sm_mhz):
+    """The bound of the tridiagonal reduction: (bound, work per step, rate, unit).
+    Each step reads and writes the whole trailing matrix and does nine integer
+    multiply-adds an element, n^3 / 3 elements in all. Where the matrices of the
+    workload do not fit the SMs' shared memory it is 16 bytes an element of HBM
+    bandwidth (the multiply-adds then take less than half of that time), else the
+    multiply-adds. The decompositions of n <= 160 (the Jacobi route) do not count."""
+    elements = sum(k * n ** 3 / 3.0 for n, k in decomps.items() if n > 160) / steps
+    held = sum(8.0 * s.n ** 2 for s in wl.searches if s.n > 160)
+    if held > REDUCTION_SMEM * sms:
+        return "hbm", 16.0 * elements, hbm_gbs * 1e9, "GB/s"
+    return "alu", 9.0 * elements, IMAD_PER_CLOCK * sms * sm_mhz * 1e6, "G integer multiply-adds/s"
 
 
 def phase_flops(wl, prec):
@@ -486,14 +508,23 @@ def run_engine(args):
         peak = bf16 * (0.5 if head == "tf32" else 1.0)
         bound, src = "tensor", ("MEASURED_PEAKS.json bf16 x nominal tf32/bf16 ratio 0.5"
                                 if head == "tf32" else "MEASURED_PEAKS.json bf16")
+    unit = "TFLOP/s"
+    work = {"algorithmic_flops_per_step": flops.get(dom, 0.0)}
+    if dom == "reduction":
+        sms = torch.cuda.get_device_properties(local_rank).multi_processor_count
+        bound, amount, rate, unit = reduction_roof(wl, r["decompositions"], steps, peaks.get("hbm_gbs", 6800.0), sms,
+                                                   r["clocks"]["sm_mhz"] or 2070.0)
+        peak, achieved = rate / 1e9, amount / (dom_ms * 1e-3) / 1e9
+        src = ("MEASURED_PEAKS.json hbm_gbs" if bound == "hbm"
+               else "%g integer multiply-adds a clock and SM at the median clock" % IMAD_PER_CLOCK)
+        work = {"algorithmic_bytes_per_step" if bound == "hbm" else "algorithmic_multiply_adds_per_step": amount}
     traffic = None
     kt = KERNEL_TRAFFIC.get(dom)
-    if kt and stage_sources_sha(dom) == kt["sources_sha256_16"]:
+    if kt and kt["workload"] == wl.name and stage_sources_sha(dom) == kt["sources_sha256_16"]:
         traffic = kt["bytes_per_step"]
-    roofline = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+    roofline = {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit,
                 "frac": achieved / peak if peak else None, "traffic": traffic, "kernel": dom,
-                "peak_source": src, "algorithmic_flops_per_step": flops.get(dom, 0.0),
-                "kernel_ms_per_step": dom_ms}
+                "peak_source": src, **work, "kernel_ms_per_step": dom_ms}
     if rank != 0:
         if dist is not None:
             dist.destroy_process_group()
