@@ -44,6 +44,8 @@ constexpr int kRfRow = (kEigMixedMaxN + 31) / 32;          // elements of a colu
 constexpr int kRfPre = kRfK * kEigMixedMaxN / kRfNT;       // left elements per thread and step
 constexpr double kRfSep = 0x1p-10;                         // largest first-order correction
 constexpr int kRfTiny = 34;                                // corrections below 2^-34 take h h alone
+constexpr int kRfMoreNs = 2;                               // most further Newton-Schulz steps
+constexpr double kRfDefect = 0x1p-28;                      // largest |X^T X - I| that one step takes to rounding
 static_assert(kEigMixedMaxN <= 160, "the integer sums over K hold up to 255 terms, the item lists up to n = 160");
 
 namespace {
@@ -267,6 +269,7 @@ __device__ __forceinline__ void rf_integers(const Rf& f, const double* src, cons
 // Scratch: ET holds C, EX and EH the basis as integers; EG and EA hold S and G.
 __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int head) {
   extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ int sh_again[kRfMoreNs + 1];  // the n-th Newton-Schulz step started from a defect that needs another
   cg::cluster_group cl = cg::this_cluster();
   Rf f;
   f.cs = static_cast<int>(cl.num_blocks());
@@ -297,6 +300,7 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
 
   // own columns of C, B and V32; columns past the last one are zero
   for (int e = f.tid; e < 2 * lay.nc * f.ks; e += kRfNT) f.R0[e] = make_int2(0, 0);
+  if (f.tid <= kRfMoreNs) sh_again[f.tid] = 0;
   auto load = [&](double* dst, const double* src) {
     for (int c = f.warp; c < f.ncl; c += kRfW)
 #pragma unroll
@@ -318,6 +322,7 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
   }
   cl.sync();
 
+  int ns = 0;  // Newton-Schulz steps formed
   for (int p = head ? 3 : 0; p < 4; ++p) {
     if (!head) {
       // X <- X + M T, M the published basis (p = 0: X = 0, M = B, T = V32)
@@ -339,11 +344,17 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
     }
     const int* ex = f.ex + cur * n;
     if (p == 2) {  // G = X^T X
+      bool large = false;
       rf_sym<1>(f, XL[cur], L, f.R0, f.R0, ex, f.e0, f.e0, [&](int i, int c, double g, double) {
         const int j = f.col(c);
         __stcg(Go + i + L * j, g);
         __stcg(Go + j + L * i, g);
+        large |= fabs(g - (i == j ? 1.0 : 0.0)) > kRfDefect;
       });
+      // Groups of repeated eigenvalues far from their old basis leave pairs at the bound of
+      // the first-order corrections, and with them a defect whose square is above rounding:
+      // the step is then repeated, for every CTA of the cluster.
+      if (__syncthreads_or(large) && f.tid < f.cs) cl.map_shared_rank(sh_again, f.tid)[ns] = 1;
       cl.sync();
       // E = (I - G) / 2
       for (int c = f.warp; c < f.ncl; c += kRfW)
@@ -353,6 +364,8 @@ __global__ void __launch_bounds__(kRfNT, 1) k_eig_refine(Search* S, int s0, int 
           if (i < n) f.T[c * f.ns + i] = 0.5 * ((i == j ? 1.0 : 0.0) - __ldcg(Go + i + L * j));
         }
       __syncthreads();
+      if (ns < kRfMoreNs && sh_again[ns]) p = 1;
+      ++ns;
       continue;
     }
     // T = C X

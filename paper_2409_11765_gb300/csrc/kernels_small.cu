@@ -286,7 +286,7 @@ __device__ __forceinline__ void sm_product(int n, int ld, const SmEig& w, double
 // a graded A is left as it is, so that its small eigenvalues keep their FP32
 // relative accuracy. All kSmNT threads call it. Returns the sweeps of both; *rot the
 // FP64 ones' rotations (thread 0).
-constexpr double kSmSep = 0x1p-10;
+constexpr double kSmSep = 0x1p-10, kSmDefect = 0x1p-28;
 struct SmSweeps {
   int f64, f32;
 };
@@ -394,11 +394,24 @@ __device__ SmSweeps small_eig(int n, double* C, double* B, const SmEig& w, int* 
     X = T;
     T = q;
   }
-  // Newton-Schulz, then A = X^T C X
-  sm_product<true, true>(n, ld, w, E, X, X, [](int i, int j, double v) { return 0.5 * ((i == j ? 1.0 : 0.0) - v); });
-  __syncthreads();
-  sm_product<false, false>(n, ld, w, B, X, E, [&](int i, int j, double v) { return X[i + ld * j] + v; });
-  __syncthreads();
+  // Newton-Schulz: one step, or up to three from a defect whose square is above rounding
+  // (pairs of repeated eigenvalues at the bound of the corrections); then A = X^T C X
+#pragma unroll 1
+  for (int ns = 0;; ++ns) {
+    bool large = false;
+    sm_product<true, true>(n, ld, w, E, X, X, [&](int i, int j, double v) {
+      const double d = (i == j ? 1.0 : 0.0) - v;
+      large |= fabs(d) > kSmDefect;
+      return 0.5 * d;
+    });
+    const bool again = __syncthreads_or(large) && ns < 2;
+    double* out = again ? T : B;
+    sm_product<false, false>(n, ld, w, out, X, E, [&](int i, int j, double v) { return X[i + ld * j] + v; });
+    __syncthreads();
+    if (!again) break;
+    T = X;
+    X = out;
+  }
   sm_product<false, false>(n, ld, w, T, C, B, [&](int, int, double v) { return v * up; });
   __syncthreads();
   sm_product<true, true>(n, ld, w, A, B, T, [](int, int, double v) { return v; });
