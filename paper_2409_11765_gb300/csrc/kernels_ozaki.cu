@@ -20,11 +20,11 @@ struct OzPackJob {
   int blocks;  // 64-row blocks
 };
 
-// Packing both operands with one CTA per 64 rows was a serial pass of K / 32 steps on a
-// few CTAs (1000 x 1024 x 2000: 32 CTAs, 240 us). Here CTAs take 64 rows by kOzPackK,
-// first for the rows' exponents (e starts below kOzZeroExp), then, with those complete,
-// for the digits; the second pass finds the operands in L2. Bound by the digits' 14
-// bytes per element on their way to L2: 13 + 28 us for the same operands.
+// CTAs take 64 rows by kOzPackK, first for the rows' exponents (e starts below
+// kOzZeroExp), then, with those complete, for the digits; the second pass finds the
+// operands in L2. Bound by the digits' 14 bytes per element on their way to L2: 13 + 28 us
+// for 1000 x 1024 x 2000, where one CTA per 64 rows is a serial pass of K / 32 steps on 32
+// CTAs, 240 us.
 constexpr int kOzPackKC = 4, kOzPackK = kOzPackKC * kOzKS;
 
 template <class F>

@@ -1,14 +1,13 @@
 // kernels_state.cu -- a search's state to and from host memory in one launch.
 //
-// cmaes_get_state and cmaes_set_state used to move every vector, matrix and scalar
-// record in a copy of its own (10 to 14 blocking copies and, for set, three kernels),
-// each of them latency. Here one kernel moves all of it between the arena and a pinned
-// host buffer of the handle, and the host copies between that buffer and the caller's
-// memory. Larger matrices (n > kStateMaxN) go by copies of their own, which reach the
-// caller's memory without the host's pass. Before -> here, to restore and to read: n = 40
-// 127 -> 39 and 80 -> 14 us, n = 100 137 -> 47 and 83 -> 17, n = 1000 282 -> 242 and
-// 166 -> 122. What is left is the launch, the synchronisation and, to restore, the
-// logarithms of the weights in one CTA.
+// One kernel moves every vector, matrix and scalar of cmaes_get_state and cmaes_set_state
+// between the arena and a pinned host buffer of the handle, and the host copies between
+// that buffer and the caller's memory: a copy of its own for each (10 to 14 blocking ones,
+// and for set three kernels) is latency. Larger matrices (n > kStateMaxN) go by copies of
+// their own, which reach the caller's memory without the host's pass. With a copy for each
+// -> here, to restore and to read: n = 40 127 -> 39 and 80 -> 14 us, n = 100 137 -> 47 and
+// 83 -> 17, n = 1000 282 -> 242 and 166 -> 122. What is left is the launch, the
+// synchronisation and, to restore, the logarithms of the weights in one CTA.
 #include <cmath>
 #include "descent.cuh"
 #include "device_common.cuh"
