@@ -162,12 +162,15 @@ __device__ __forceinline__ int block_or(int v, int* sh) {
 // against 113-bit arithmetic the objectives come out 1.2 to 3 times closer than with
 // FMAs (n = 100, rastrigin: 1.1e-16 rms, was 2.3e-16; n = 1000: 7.8e-17, was
 // 2.5e-16). The steps split K evenly: a last step of a few k would meet them by chance.
-// Bound by the integer multiply-adds and, beside them, by staging, which two CTAs per
-// SM overlap (128 registers; one of 172: 166 us). Evaluating 8704 points of n = 100:
-// 305 us in FP64 FMAs, 143 here (its multiply-adds alone, tile padding included, take
-// ~40), 270 if every output were to go to FP64.
+// Bound by the integer multiply-adds and, beside them, by staging, which two CTAs per SM
+// overlap (PER_SM = 2, 128 registers) where there are more tiles than SMs; a tile that
+// has an SM to itself runs faster with the registers that the compiler takes (PER_SM = 1,
+// 172). n = 500, 88 tiles and 168: 229 and 442 us with one, 248 and 384 with two.
+// Evaluating 8704 points of n = 100: 305 us in FP64 FMAs, 143 here (its multiply-adds
+// alone, tile padding included, take ~40), 270 if every output were to go to FP64.
 // ---------------------------------------------------------------------------
-constexpr int kGBM = 64, kGBN = 64, kGBK = 32, kGNT = 256, kGPerSM = 2;
+constexpr int kGBM = 64, kGBN = 64, kGBK = 32, kGNT = 256;
+constexpr int kGSms = 152;  // tiles from which on two CTAs share an SM
 
 struct GemmSmem {
   int2 As[kGBK][kGBM + 1];  // limbs (h, l), or the doubles themselves
@@ -228,7 +231,7 @@ __device__ __forceinline__ double gemm_scaled(long long hh, long long mid, int e
   return __hiloint2double(hi + (e << 20), __double2loint(d));
 }
 
-template <bool A_I_CONTIG, bool B_K_CONTIG, class LA, class LB, class EPI>
+template <int PER_SM, bool A_I_CONTIG, bool B_K_CONTIG, class LA, class LB, class EPI>
 __device__ __forceinline__ void gemm_tile_f64(int M, int N, int K, int i0, int j0, const LA& la,
                                               const LB& lb, const EPI& epi, GemmSmem& sm) {
   const int tid = threadIdx.x;
@@ -294,7 +297,7 @@ __device__ __forceinline__ void gemm_tile_f64(int M, int N, int K, int i0, int j
     unsigned f64 = 0;  // bit 4 r + c: this output's step is summed in FP64
     {
       unsigned sum[4][4] = {};
-#pragma unroll 2
+#pragma unroll(PER_SM == 1 ? kGBK / 4 : 2)
       for (int w = 0; w < kGBK / 4; ++w) {
         unsigned a[4], b[4];
 #pragma unroll

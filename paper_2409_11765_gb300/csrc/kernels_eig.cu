@@ -47,7 +47,7 @@ int jacobi_smem_bytes(int n) {
 __device__ __forceinline__ bool mixed_route(const Search& s) { return s.n <= kEigBigMaxN; }
 
 // ET = C B (square tiles; only searches whose decomposition is due).
-__global__ void __launch_bounds__(kGNT, kGPerSM) k_eig_gemm_CB(Search* S, TileMap tm) {
+__global__ void __launch_bounds__(kGNT, 2) k_eig_gemm_CB(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_eig_gemm_CB(Search* S, TileMa
   const double* C = s.C;
   const double* B = s.B;
   double* ET = s.ET;
-  gemm_tile_f64<true, true>(
+  gemm_tile_f64<2, true, true>(
       n, n, n, (t % T) * kGBM, (t / T) * kGBN,
       [=] __device__(int i, int k) { return C[i + static_cast<long long>(ldn) * k]; },
       [=] __device__(int k, int j) { return B[k + static_cast<long long>(ldn) * j]; },
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_eig_gemm_CB(Search* S, TileMa
 }
 
 // EA = B^T ET = B^T C B.
-__global__ void __launch_bounds__(kGNT, kGPerSM) k_eig_gemm_BtT(Search* S, TileMap tm) {
+__global__ void __launch_bounds__(kGNT, 2) k_eig_gemm_BtT(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_eig_gemm_BtT(Search* S, TileM
   const double* B = s.B;
   const double* ET = s.ET;
   double* EA = s.EA;
-  gemm_tile_f64<false, true>(
+  gemm_tile_f64<2, false, true>(
       n, n, n, (t % T) * kGBM, (t / T) * kGBN,
       [=] __device__(int i, int k) { return B[k + static_cast<long long>(ldn) * i]; },
       [=] __device__(int k, int j) { return ET[k + static_cast<long long>(ldn) * j]; },

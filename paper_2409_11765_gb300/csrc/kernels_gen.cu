@@ -124,7 +124,8 @@ void launch_sample_z(Search* S, TileMap tm, DevOptions o, cudaStream_t st) {
 }
 
 // Eq. (1) for all candidates (§3.1): Y = (B diag(D)) Z, X = m 1^T + sigma Y.
-__global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_sample(Search* S, TileMap tm) {
+template <int PER_SM>
+__global__ void __launch_bounds__(kGNT, PER_SM) k_gemm_sample(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_sample(Search* S, TileMa
   double* X = s.X;
   const double* m = s.m;
   const double sigma = s.sigma;
-  gemm_tile_f64<true, true>(
+  gemm_tile_f64<PER_SM, true, true>(
       n, lam, n, i0, j0,
       [=] __device__(int i, int k) { return BD[i + static_cast<long long>(ldn) * k]; },
       [=] __device__(int k, int j) { return Z[k + static_cast<long long>(ldn) * j]; },
@@ -153,12 +154,14 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_sample(Search* S, TileMa
 }
 
 void launch_gemm_sample(Search* S, TileMap tm, cudaStream_t st) {
-  if (tm.total > 0) k_gemm_sample<<<tm.total, 256, 0, st>>>(S, tm);
+  if (tm.total > kGSms) k_gemm_sample<2><<<tm.total, kGNT, 0, st>>>(S, tm);
+  else if (tm.total > 0) k_gemm_sample<1><<<tm.total, kGNT, 0, st>>>(S, tm);
 }
 
 // ------------------------------- objective ----------------------------------
 // Rotated objectives: U = Q (X - x*), with x - x* formed in FP64.
-__global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_objective(Search* S, TileMap tm) {
+template <int PER_SM>
+__global__ void __launch_bounds__(kGNT, PER_SM) k_gemm_objective(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -172,7 +175,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_objective(Search* S, Til
   const double* X = s.X;
   const double* xs = s.xstar;
   double* U = s.U;
-  gemm_tile_f64<true, true>(
+  gemm_tile_f64<PER_SM, true, true>(
       n, lam, n, i0, j0,
       [=] __device__(int i, int k) { return Q[i + static_cast<long long>(ldn) * k]; },
       [=] __device__(int k, int j) { return X[k + static_cast<long long>(ldn) * j] - xs[k]; },
@@ -181,7 +184,8 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_gemm_objective(Search* S, Til
 }
 
 void launch_gemm_objective(Search* S, TileMap tm, cudaStream_t st) {
-  if (tm.total > 0) k_gemm_objective<<<tm.total, 256, 0, st>>>(S, tm);
+  if (tm.total > kGSms) k_gemm_objective<2><<<tm.total, kGNT, 0, st>>>(S, tm);
+  else if (tm.total > 0) k_gemm_objective<1><<<tm.total, kGNT, 0, st>>>(S, tm);
 }
 
 // f_k: one warp per candidate column, lanes stride over the rows in order and
@@ -470,7 +474,8 @@ __device__ __forceinline__ void sym_tile(int t, int n, int& ti, int& tj) {
   tj = ti + rem;
 }
 
-__global__ void __launch_bounds__(kGNT, kGPerSM) k_cov_partial(Search* S, TileMap tm) {
+template <int PER_SM>
+__global__ void __launch_bounds__(kGNT, PER_SM) k_cov_partial(Search* S, TileMap tm) {
   __shared__ GemmSmem sm;
   int t;
   const int si = find_search(tm, t);
@@ -491,7 +496,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_cov_partial(Search* S, TileMa
     const double* pc = s.pc;
     const double c1 = s.c1, cmu = s.cmu;
     const double a = cov_keep(c1, cmu, s.cc, s.hsig);
-    gemm_tile_f64<true, false>(
+    gemm_tile_f64<PER_SM, true, false>(
         n, n, k_hi - k_lo, ti * kGBM, tj * kGBN,
         [=] __device__(int i, int r) { return w[r] * Y[i + static_cast<long long>(ldn) * order[r]]; },
         [=] __device__(int r, int j) { return Y[j + static_cast<long long>(ldn) * order[r]]; },
@@ -507,7 +512,7 @@ __global__ void __launch_bounds__(kGNT, kGPerSM) k_cov_partial(Search* S, TileMa
   }
   double* out = s.covpart + (static_cast<long long>(tile) * nch + c) * (kGBM * kGBN);
   const int i0 = ti * kGBM, j0 = tj * kGBN;
-  gemm_tile_f64<true, false>(
+  gemm_tile_f64<PER_SM, true, false>(
       n, n, k_hi - k_lo, i0, j0,
       [=] __device__(int i, int r) { return w[r] * Y[i + static_cast<long long>(ldn) * order[r]]; },
       [=] __device__(int r, int j) { return Y[j + static_cast<long long>(ldn) * order[r]]; },
@@ -542,7 +547,8 @@ __global__ void __launch_bounds__(256) k_cov_reduce(Search* S, TileMap tm) {
 }
 
 void launch_cov_partial(Search* S, TileMap tm, cudaStream_t st) {
-  if (tm.total > 0) k_cov_partial<<<tm.total, 256, 0, st>>>(S, tm);
+  if (tm.total > kGSms) k_cov_partial<2><<<tm.total, kGNT, 0, st>>>(S, tm);
+  else if (tm.total > 0) k_cov_partial<1><<<tm.total, kGNT, 0, st>>>(S, tm);
 }
 void launch_cov_reduce(Search* S, TileMap tm, cudaStream_t st) {
   if (tm.total > 0) k_cov_reduce<<<tm.total, 256, 0, st>>>(S, tm);

@@ -29,13 +29,14 @@ __device__ __align__(256) double g_eval_scratch[kEvalScratchDoubles];
 constexpr int kMaxDevices = 64;
 double* g_scratch_addr[kMaxDevices] = {nullptr};
 
-__global__ void __launch_bounds__(kGNT, kGPerSM) k_noalloc_rotate(int n, int lam, int ld, const double* X,
+template <int PER_SM>
+__global__ void __launch_bounds__(kGNT, PER_SM) k_noalloc_rotate(int n, int lam, int ld, const double* X,
                                                         const double* Q, int ldq,
                                                         const double* xstar, double* U) {
   __shared__ GemmSmem sm;
   const int mt = ceil_div(n, kGBM);
   const int i0 = (blockIdx.x % mt) * kGBM, j0 = (blockIdx.x / mt) * kGBN;
-  gemm_tile_f64<true, true>(
+  gemm_tile_f64<PER_SM, true, true>(
       n, lam, n, i0, j0,
       [=] __device__(int i, int k) { return Q[i + static_cast<long long>(ldq) * k]; },
       [=] __device__(int k, int j) { return X[k + static_cast<long long>(ld) * j] - xstar[k]; },
@@ -114,7 +115,8 @@ extern "C" cmaes_status cmaes_evaluate_noalloc(int kind, int n, int lambda, cons
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (rotated) {
     const int tiles = ceil_div(n, kGBM) * ceil_div(lambda, kGBN);
-    k_noalloc_rotate<<<tiles, 256, 0, st>>>(n, lambda, ld, X, Q, ldq, xstar, U);
+    if (tiles > kGSms) k_noalloc_rotate<2><<<tiles, kGNT, 0, st>>>(n, lambda, ld, X, Q, ldq, xstar, U);
+    else k_noalloc_rotate<1><<<tiles, kGNT, 0, st>>>(n, lambda, ld, X, Q, ldq, xstar, U);
   }
   k_noalloc_reduce<<<ceil_div(lambda, 8), 256, 0, st>>>(kind, n, lambda, ld, X, U, lambda_diag, xstar, f);
   e = cudaGetLastError();

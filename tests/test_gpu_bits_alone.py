@@ -153,3 +153,24 @@ def test_jacobi_route(n, count, precision):
         finally:
             eng.cmaes_destroy(h)
     same(*got)
+
+
+@pytest.mark.parametrize("n,lam", [(40, 30), (100, 64), (161, 70)])
+def test_fp64_products(n, lam):
+    """The products of a few tiles and of more than the GPU has SMs."""
+    d = W.random_state(n, SEED, 7, cond=30.0)
+    prob = W.make_problem(W.RASTRIGIN, n, SEED, 61)
+    got = []
+    for searches in (1, 160):
+        opt = eng.cmaes_default_options(eig_every=1, stop_mask=0)
+        h = eng.cmaes_create_batch([n] * searches, [lam] * searches, [np.zeros(n)] * searches, [1.0] * searches, SEED, opt)
+        try:
+            for i in range(searches):
+                eng.cmaes_set_problem(h, i, W.RASTRIGIN, prob.Q, prob.lamdiag, prob.xstar)
+            eng.cmaes_set_state(h, 0, dict(n=n, lam=lam, sigma=0.3, m=d["m"], ps=d["ps"], pc=d["pc"], C=d["C"],
+                                           B=d["B"], D=d["D"], gen=5))
+            eng.cmaes_step_batch(h, 3)
+            got.append((eng.cmaes_get_state(h, 0, n), eng.cmaes_get_generation(h, 0, n)))
+        finally:
+            eng.cmaes_destroy(h)
+    same(*got)
