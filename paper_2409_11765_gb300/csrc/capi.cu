@@ -76,6 +76,7 @@ struct cmaes_s {
   size_t arena_bytes = 0;
   int* d_off = nullptr;  // TK_COUNT x (count + 1)
   double* state_buf = nullptr;  // pinned: a search's state on its way (get_state, set_state)
+  size_t state_buf_bytes = 0;
   int* d_err = nullptr;  // device status word (bit 0: a bounded wait timed out)
   bool mixed = false;
   std::vector<int> h_off;
@@ -200,6 +201,55 @@ static cmaes_status check_device_status(cmaes_t h) {
     return set_error(h, CMAES_ENUMERIC, "a search's state became non-finite; the search was restarted or ended");
   }
   return CMAES_OK;
+}
+
+// Pinned buffers of handles that are gone, for the next ones: to pin and unpin one takes
+// 300 us, four times the rest of a small handle's creation. At most kPinnedKeep bytes are
+// kept a context, and kPinnedMost buffers in all; a buffer ends with its context, so it is
+// kept under the context's number, which is never given twice.
+namespace {
+constexpr size_t kPinnedKeep = 8u << 20, kPinnedMost = 256;
+struct Pinned {
+  unsigned long long context;
+  void* p;
+  size_t bytes;
+};
+std::mutex g_pinned_mutex;
+std::vector<Pinned> g_pinned;
+}  // namespace
+
+static cudaError_t pinned_take(size_t bytes, void** p, size_t* got) {
+  size_t size = 4096;
+  while (size < bytes) size *= 2;
+  const unsigned long long context = context_number();
+  if (context != 0) {
+    std::lock_guard<std::mutex> lock(g_pinned_mutex);
+    for (size_t i = 0; i < g_pinned.size(); ++i) {
+      if (g_pinned[i].context != context || g_pinned[i].bytes != size) continue;
+      *p = g_pinned[i].p;
+      *got = size;
+      g_pinned.erase(g_pinned.begin() + static_cast<long>(i));
+      return cudaSuccess;
+    }
+  }
+  *got = size;
+  return cudaHostAlloc(p, size, cudaHostAllocPortable);
+}
+
+// (nothing on the device uses the buffer any more)
+static void pinned_give(void* p, size_t bytes) {
+  const unsigned long long context = context_number();
+  if (context != 0) {
+    std::lock_guard<std::mutex> lock(g_pinned_mutex);
+    size_t kept = bytes;
+    for (const Pinned& b : g_pinned)
+      if (b.context == context) kept += b.bytes;
+    if (kept <= kPinnedKeep && g_pinned.size() < kPinnedMost) {
+      g_pinned.push_back(Pinned{context, p, bytes});
+      return;
+    }
+  }
+  cudaFreeHost(p);
 }
 
 // The state's way through the handle's pinned buffer: one kernel for the scalars, the
@@ -716,7 +766,7 @@ void cmaes_destroy(cmaes_t h) {
   if (h->dS) cudaFree(h->dS);
   if (h->d_off) cudaFree(h->d_off);
   if (h->d_err) cudaFree(h->d_err);
-  if (h->state_buf) cudaFreeHost(h->state_buf);
+  if (h->state_buf) pinned_give(h->state_buf, h->state_buf_bytes);
   if (h->d_trd_grp) cudaFree(h->d_trd_grp);
   for (cudaEvent_t e : h->trd_pool) cudaEventDestroy(e);
   if (h->d_trd_bar) cudaFree(h->d_trd_bar);
@@ -873,7 +923,7 @@ cmaes_status cmaes_create_batch(int count, const int* n_arr, const int* lam_arr,
   CREATE_TRY(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
   size_t state_max = 0;
   for (const Search& x : h->hs) state_max = std::max(state_max, state_bytes(x));
-  CREATE_TRY(cudaHostAlloc(reinterpret_cast<void**>(&h->state_buf), state_max, cudaHostAllocPortable));
+  CREATE_TRY(pinned_take(state_max, reinterpret_cast<void**>(&h->state_buf), &h->state_buf_bytes));
   CREATE_TRY(cudaMemsetAsync(h->arena, 0, total, h->stream));
   for (int s = 0; s < count; ++s) {
     Search& x = h->hs[s];
