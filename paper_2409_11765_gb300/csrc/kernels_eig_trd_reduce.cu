@@ -399,40 +399,34 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_trd_reduce(Search* S, const in
         pa[i] = pw1 >> 2;  // p in 8 q
         pa[i2] = pw2 >> 2;
       }
-      long long thi = 0;
-      u64 tlo = 0ull;
+      u64 sum = 0ull;  // p . v in 2 q, each row's product rounded alone: it does not depend on which thread has the row
       unsigned tmx = 0u;
 #pragma unroll 1
       for (int i = k + tid; i < n; i += NT) {
         const long long P = pa[i];
         const int2 y = vc[i];
         const long long v = (static_cast<long long>(y.x) << 30) + y.y;
-        thi += __mul64hi(P, v);
-        tlo += static_cast<u64>(P * v) >> 13;
+        const u64 lo = static_cast<u64>(P * v), low = lo + (1ull << 56);
+        sum += (static_cast<u64>(__mul64hi(P, v) + (low < lo ? 1 : 0)) << 7) + (low >> 57);
         tmx = max(tmx, static_cast<unsigned>((P < 0 ? -P : P) >> 32));
       }
       __syncwarp();
-      // p . v in its high words and, cut for each row alone, its low ones: the sums do
-      // not depend on which thread has a row
-      const u64 pvh = warp_sum_u64(static_cast<u64>(thi)), pvl = warp_sum_u64(tlo);
+      sum = warp_sum_u64(sum);
       tmx = __reduce_max_sync(0xffffffffu, tmx);
       if (lane == 0) {
-        redi[0][warp] = pvh;
-        redi[1][warp] = pvl;
+        redi[0][warp] = sum;
         redm[warp] = tmx;
       }
       if (!__syncthreads_and(ok)) return;
     }
     if (warp == 0) {  // half = (tau / 2) p . v of p = tau A v; the scale of w from |w| <= tau max|A v| + |half|
-      u64 pvh = 0ull, pvl = 0ull;
+      long long pv = 0;
       unsigned mx = 0u;
 #pragma unroll
       for (int w = 0; w < NW; ++w) {
-        pvh += redi[0][w];
-        pvl += redi[1][w];
+        pv += static_cast<long long>(redi[0][w]);
         mx = max(mx, redm[w]);
       }
-      const long long pv = static_cast<long long>((pvh << 7) + (pvl >> 44));
       // p . v is in 2 q: half = tau^2 pv q, from pv 2^zp < 2^62 and tau^2 in 2^-60
       const u64 ap = static_cast<u64>(pv < 0 ? -pv : pv);
       const int zp = ap != 0ull ? __clzll(static_cast<long long>(ap)) - 2 : 61, eh = 66 - zp;
